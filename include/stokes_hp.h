@@ -228,7 +228,7 @@ int stokes_last_ratios(stokes_t ctx, double* ratios, int capacity);
 /* ---- instrumentation (no counterpart in the paper) ------------------------------------------
  * Kernel classes: 0 banded Kronecker passes in FP32, 1 dense mode products on CUDA cores,
  * 2 discrete divergence / transpose, 3 Krylov vector kernels, 4 tensor-core mode products,
- * 5 banded Cholesky line solves, 6 banded Kronecker passes in FP64, 7 the saddle-point operator
+ * 5 pressure-mass inverse along one direction (FP64, b >= 64), 6 banded Kronecker passes in FP64, 7 the saddle-point operator
  * in pair-of-FP32 arithmetic (its banded passes and fused divergence).
  * stokes_profile_begin brackets every later launch of this thread with CUDA events on the
  * launching stream; stokes_profile_end synchronizes, writes per-class totals (launches, summed

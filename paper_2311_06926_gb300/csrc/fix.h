@@ -1,0 +1,95 @@
+// Fixed-point evaluation of FP64 dot products on the FP16 tensor cores.
+//
+// GB300 runs 2 FP64 FMAs per clock and SM, but 1024 FP16 multiply-adds with FP32 sums (mma.sync;
+// measured: 0.62 against 300 T per second). A dot product of doubles is therefore cheaper in
+// slices: the entries of one input line are scaled by one power of two (that of the line's largest
+// entry) to integers, those of an operator column to integers below 2^58, and each integer is
+// written in six balanced digits of ten bits, sum_i d_i 2^(50 - 10 i), |d_i| <= 512, which FP16
+// holds exactly. Products of digits are exact in the tensor cores, and the 21 digit pairs with
+// i + j <= 5 are summed by level l = i + j in FP32. Level 2 is moved to an integer after every 32
+// terms and all levels after every 80 (input integers below 2^57: folded entries and modes) or
+// 64 (below 2^58: plain matrices). Levels 0 to 2 then stay below 2^24 whatever the digits, since
+// |d_0| <= 2^7 or 2^8 and <= 2^8; the higher levels do too unless nearly all digits are extreme,
+// and a rounding there is below 2^-52 of the largest sum. The integer result is rounded to a
+// double once, where an FMA chain rounds at every term. The dropped pairs (i + j >= 6) and the
+// scaling leave an error below that of the FMA chain (host emulation, 9 to 66 terms, rms over
+// random, decaying and smooth lines: 0.2 to 0.56 of the chain's).
+//
+// The integer sums do not depend on the tile or the kernel that forms them, so every launch form
+// gives the same bits.
+//
+// A line with an infinity or a NaN, or whose largest entry is outside [2^-823, 2^777] (its scaled
+// result could leave the normal range), takes the FMA chain instead.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace shp {
+
+constexpr int kFixSlices = 6, kFixDigit = 10;
+// bits of a scaled operator entry, and of the sum of an output's operator magnitudes: the 64-bit
+// sums, in units of 2^60, stay below 2^62
+constexpr int kFixUBits = 58, kFixSumBits = 63, kFixUnit = 60;
+
+// One direction of a parity-split operator (host_setup.h, generalized_eigh_parity) as digit slices
+// in the operand order of mma.sync m16n8k16: half `par` (0: even terms, 1: odd terms), 8 outputs
+// per column tile t < nt, 16 terms per step s < ks, the half zero-padded (a plain matrix has half 0
+// only):
+//   frag[(((par nt + t) ks + s) 3 + c) 32 + lane] = the lane's two registers of slice 2 c, then
+//   those of slice 2 c + 1.
+// Output i of half par is the integer sum times 2^ex[par 8 nt + i].
+struct FixTab {
+  const uint4* frag = nullptr;
+  const int* ex = nullptr;
+  int nt = 0, ks = 0;
+};
+
+// The uses of an operator U (columns [even modes; odd modes]): fw contracts the folded entries of a
+// line with the columns (outputs: modes), bw the modes with the rows (outputs: the even and the
+// odd part of the mirrored entries k and n - 1 - k). A plain matrix has one table, fw, of one half
+// with every entry as a term.
+enum { kFixForward = 0, kFixBackward = 1, kFixPlain = 2 };
+struct FixTabs {
+  FixTab fw, bw;
+};
+
+#ifdef __CUDACC__
+// biased exponents of the largest entry of a line that the fixed-point form takes
+constexpr unsigned kFixMinExp = 200, kFixMaxExp = 1800;
+
+// Magnitude key of an entry: its exponent field and leading bits (the low word only marks a
+// nonzero). The largest key of a line gives its scale; 0 only for a line of zeros.
+__device__ __forceinline__ unsigned fix_key(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
+}
+__device__ __forceinline__ bool fix_slow(unsigned key) {
+  const unsigned e = key >> 20;
+  return key != 0u && (e < kFixMinExp || e > kFixMaxExp);
+}
+// x / 2^(emax - 1022) * 2^xbits, truncated (emax: exponent field of the largest entry)
+__device__ __forceinline__ long long fix_of(double x, int emax, int xbits) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  const unsigned m = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
+  // the 53-bit significand with its leading bit at bit 62
+  const unsigned long long n = ((unsigned long long)__funnelshift_l(lo, m, 10) << 32) | (lo << 10);
+  const int sh = min(63 - xbits + emax - e, 63);
+  const long long v = (long long)(n >> sh);
+  return (int)hi < 0 ? -v : v;
+}
+// s * 2^ex as a double, rounded to nearest (ex keeps it in the normal range). In integers: the
+// conversion instruction runs on the FP64 pipe.
+__device__ __forceinline__ double fix_to_double(long long s, int ex) {
+  unsigned long long u = (unsigned long long)(s < 0 ? -s : s);
+  const int lz = __clzll((long long)u);
+  u <<= lz & 63;
+  // the leading one of u >> 11 adds one to the exponent field
+  const unsigned long long m =
+      (u >> 11) + ((u >> 10) & 1) + ((unsigned long long)(unsigned)(ex + 1085 - lz) << 52);
+  const unsigned hi = (unsigned)(m >> 32) | (s < 0 ? 0x80000000u : 0u);
+  return s == 0 ? 0.0 : __hiloint2double((int)hi, (int)(unsigned)m);
+}
+#endif
+
+}  // namespace shp

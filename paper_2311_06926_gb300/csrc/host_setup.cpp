@@ -388,6 +388,56 @@ bool generalized_eigh_parity(const Dense& K, const Dense& M, std::vector<double>
   return true;
 }
 
+bool banded_inverse(const Dense& A, int p, Dense& inv) {
+  const int n = A.rows, w = p + 1;
+  // L(i, k) at lb[i * w + (k - i + p)] for i - p <= k <= i
+  std::vector<double> lb((size_t)n * w, 0.0);
+  auto L = [&](int i, int k) -> double& { return lb[(size_t)i * w + (k - i + p)]; };
+  for (int j = 0; j < n; ++j) {
+    double d = A(j, j);
+    for (int k = std::max(0, j - p); k < j; ++k) d -= L(j, k) * L(j, k);
+    if (!(d > 0.0)) return false;
+    L(j, j) = std::sqrt(d);
+    for (int i = j + 1; i < std::min(n, j + w); ++i) {
+      double t = A(i, j);
+      for (int k = std::max(0, i - p); k < j; ++k) t -= L(i, k) * L(j, k);
+      L(i, j) = t / L(j, j);
+    }
+  }
+  auto solve = [&](std::vector<double>& v) {
+    for (int i = 0; i < n; ++i) {
+      double t = v[i];
+      for (int k = std::max(0, i - p); k < i; ++k) t -= L(i, k) * v[k];
+      v[i] = t / L(i, i);
+    }
+    for (int i = n - 1; i >= 0; --i) {
+      double t = v[i];
+      for (int k = i + 1; k < std::min(n, i + w); ++k) t -= L(k, i) * v[k];
+      v[i] = t / L(i, i);
+    }
+  };
+  inv = Dense(n, n);
+  std::vector<double> x(n), r(n);
+  for (int c = 0; c < n; ++c) {
+    std::fill(x.begin(), x.end(), 0.0);
+    x[c] = 1.0;
+    solve(x);
+    for (int i = 0; i < n; ++i) {
+      double hi = i == c ? 1.0 : 0.0, lo = 0.0;   // products by fma, sums by TwoSum
+      for (int k = std::max(0, i - p); k < std::min(n, i + w); ++k) {
+        const double a = -A(i, k), pr = a * x[k], e = std::fma(a, x[k], -pr);
+        const double t = hi + pr, z = t - hi;
+        lo += ((hi - (t - z)) + (pr - z)) + e;
+        hi = t;
+      }
+      r[i] = hi + lo;
+    }
+    solve(r);
+    for (int i = 0; i < n; ++i) inv(i, c) = x[i] + r[i];
+  }
+  return true;
+}
+
 Band to_band(const Dense& D, double drop_tol) {
   Band B;
   B.rows = D.rows;

@@ -61,6 +61,11 @@ bool generalized_eigh(const Dense& K, const Dense& M, std::vector<double>& lam, 
 bool generalized_eigh_parity(const Dense& K, const Dense& M, std::vector<double>& lam, Dense& U,
                              int* he);
 
+// Inverse of a symmetric positive definite matrix of half bandwidth p by banded Cholesky, each
+// column refined once with a residual in twice the working precision (entries correct to about an
+// ulp of the column). Returns false if A is not positive definite.
+bool banded_inverse(const Dense& A, int p, Dense& inv);
+
 Band to_band(const Dense& D, double drop_tol);
 
 // 1D load of a sine mode against the interior N functions (own direction) or the M functions.

@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <mutex>
 
+#include "fix.h"
+
 namespace shp {
 
 // ---- programmatic dependent launch ---------------------------------------------------------------
@@ -208,6 +210,8 @@ struct ModeArgs {
   T post;   // if lam1 == null: the result is multiplied by post
   const T* invd;   // if set (FP64 path): the result is multiplied by invd[output index] instead
   int eo_he;       // FP64 path: U's columns are [he even; n - he odd] eigenvectors (0: generic)
+  FixTabs fx;      // FP64 path: U in slices (null: FMA chains)
+  int plain;       // FP64 path: U is a plain matrix (one half, fx.fw; trans = 0)
   int block;       // FP64 path: target threads per block (<= 0: 512); chosen by the setup tuner
 };
 // Both return the status of their launch (cudaSuccess, or the error of the shared-memory limit
@@ -218,7 +222,7 @@ cudaError_t mode_product(const ModeArgs<T>& a, cudaStream_t s);
 constexpr int kMaxModeJobs = 4;
 template <typename T>
 cudaError_t mode_product_multi(const ModeArgs<T>* jobs, int njobs, cudaStream_t s);
-// Dynamic shared memory (bytes) of the FP64 mode-product kernel for this one job.
+// Dynamic shared memory (bytes) of the FP64 product of one job without slice tables.
 int64_t mode_product_smem(const ModeArgs<double>& m);
 
 // Fused FP64 fast-diagonalisation passes (App. A.4), several tensors per launch. The operators
@@ -235,6 +239,7 @@ struct FdPlaneArgs {
   Dims in;
   int eo1, eo2;
   double post;
+  FixTabs fx1, fx2;
 };
 // Lines along x3: the forward product with U3^T, the eigenvalue scaling (invd, or
 // 1 / (scale (lam1 + lam2 + lam3)), or none), and the backward product with U3 (times post).
@@ -247,31 +252,30 @@ struct FdLineArgs {
   const double *lam1, *lam2, *lam3;
   double scale;
   double post;
+  FixTabs fx3;
 };
-// Shared memory of one plane block (two plane buffers); 0 if the plane does not fit.
+// Bytes of two plane buffers; 0 above 200 KiB (the fused forms are not offered then).
 int fd_plane_smem(Dims in);
 // Both return false without launching if a job does not qualify (plane too large for shared
-// memory, no parity split); the caller then uses mode_product_multi.
+// memory, no parity split).
 // cluster: 1, 2 or 4 blocks per plane (a thread-block cluster sharing the plane's intermediate
 // through distributed shared memory).
 bool fd_plane_multi(const FdPlaneArgs* jobs, int njobs, int fwd, int block, int cluster,
                     cudaStream_t s);
 bool fd_line3_multi(const FdLineArgs* jobs, int njobs, int block, cudaStream_t s);
+// The same for operators with slice tables, in fixed point (k_fix.cu); the functions above take
+// them there. A context builds the tables when its halves have more than kFixMinHalf terms.
+constexpr int kFixMinHalf = 12;
+cudaError_t fix_mode_multi(const ModeArgs<double>* jobs, int njobs, cudaStream_t s);
+bool fix_plane_multi(const FdPlaneArgs* jobs, int njobs, int fwd, int block, int cluster,
+                     cudaStream_t s);
+bool fix_line3_multi(const FdLineArgs* jobs, int njobs, int block, cudaStream_t s);
 
 // delta = D_div u (and e = nu delta + q when q is set) and their band pass along x1 in one launch:
 // y0 = D .x1 delta, y1 = D .x1 e on the (b, b, b) pressure grid (FP64 contexts, one item).
 template <typename T>
 void div_band_x1(const T* u1, const T* u2, const T* u3, int a, int b, const T* q, T nu,
                  const BandD<T>& D, T* y0, T* y1, cudaStream_t s);
-
-// Banded Cholesky solves along one direction of a (b, b, b) tensor: y <- post (L L^T)^-1 x (y may
-// be x) with L lower triangular of bandwidth p stored as rows lb[i * (p + 1) + (k - i + p)] for
-// k in [i - p, i], and inv_diag[i] = 1 / L[i][i] (pressure mass inverse). nb items, item k of x and
-// y at k * bs entries. Returns the launch status.
-template <typename T>
-cudaError_t chol_solve_axis(const T* x, T* y, int b, int p, int axis, const T* lb,
-                            const T* inv_diag, T post, cudaStream_t s, int nb = 1,
-                            int64_t bs = 0);
 
 // ---- vector kernels (k_vec.cu) -----------------------------------------------------------
 // Deterministic dot product: fixed grid, fixed-order tree reduction. Result written to *out

@@ -9,7 +9,8 @@
 // into the epilogue of the last forward product.
 //
 // FP32 (CUDA-core fallback of the reduced-precision preconditioner): 64 x 64 tiles, 256 threads,
-// 4 x 4 outputs per thread. FP64 uses the row-streaming kernel further below.
+// 4 x 4 outputs per thread. FP64: the row-streaming kernel further below for short lines, k_fix.cu
+// for the others.
 #include <algorithm>
 #include <atomic>
 
@@ -167,9 +168,13 @@ GemmArgs<T> make_gemm(const ModeArgs<T>& m) {
   return g;
 }
 
-// ---- FP64 mode products ------------------------------------------------------------------------
-// GB300 executes about two FP64 FMA per clock per SM, so an FP64 mode product is bound by the
-// FP64 pipe on every mesh size. Extents are used exactly: no padded tiles.
+// ---- FP64 mode products by FMA chains ------------------------------------------------------------
+// For operators without slice tables (k_fix.cu): the allocation-free entry point, whose caller owns
+// the operators, and meshes whose halves have at most kFixMinHalf terms. There the chains are
+// short and latency bounds either form: one order-2, 1-step preconditioner takes 76 us against
+// 100 in slices at 8^3 p = 2 and 102 against 110 at 20^3 p = 3 (halves of 12), but 123 against
+// 115 at 24^3 p = 3 (halves of 14). GB300 executes about two FP64 FMA per clock per SM, which
+// bounds larger products. Extents are used exactly: no padded tiles.
 struct RowJob {
   const double* X; double* Y; const double* U;
   int64_t op_i, op_j;      // Op(i, j) = U[i * op_i + j * op_j]
@@ -597,6 +602,7 @@ int64_t mode_product_smem(const ModeArgs<double>& m) {
 
 template <>
 cudaError_t mode_product_multi<double>(const ModeArgs<double>* jobs, int njobs, cudaStream_t s) {
+  if (jobs[0].fx.fw.frag) return fix_mode_multi(jobs, njobs, s);
   RowBatch rb{};
   rb.njobs = njobs;
   int blocks = 0, smem = 0, threads = 32;
@@ -679,6 +685,7 @@ std::atomic<int> g_plane_attr{0};
 
 bool fd_plane_multi(const FdPlaneArgs* jobs, int njobs, int fwd, int block, int cluster,
                     cudaStream_t s) {
+  if (jobs[0].fx1.fw.frag) return fix_plane_multi(jobs, njobs, fwd, block, cluster, s);
   PlaneBatch pb{};
   pb.njobs = njobs;
   pb.fwd = fwd;
@@ -723,6 +730,7 @@ bool fd_plane_multi(const FdPlaneArgs* jobs, int njobs, int fwd, int block, int 
 }
 
 bool fd_line3_multi(const FdLineArgs* jobs, int njobs, int block, cudaStream_t s) {
+  if (jobs[0].fx3.fw.frag) return fix_line3_multi(jobs, njobs, block, s);
   LineBatch lbt{};
   lbt.njobs = njobs;
   const int target = block > 0 ? std::min(block, 512) : 512;

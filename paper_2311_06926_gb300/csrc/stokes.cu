@@ -189,6 +189,85 @@ T* upload(Arena& ar, const std::vector<double>& h, cudaStream_t s) {
   return d;
 }
 
+// FP16 bits of an integer of magnitude at most 2048 (exact)
+uint16_t half_bits(int v) {
+  if (v == 0) return 0;
+  const unsigned a = (unsigned)std::abs(v);
+  int e = 0;
+  while ((a >> e) > 1) ++e;
+  return (uint16_t)((v < 0 ? 0x8000u : 0u) | ((unsigned)(e + 15) << 10) |
+                    (((a << 10) >> e) & 0x3ffu));
+}
+
+// One side of FixTabs: u(k, i, par) is the operator entry of term k and output i of half par (0 even,
+// 1 odd; zero where the half has no such entry). Output i is scaled so that its integers stay
+// below 2^kFixUBits and the sum of their magnitudes below 2^kFixSumBits (fix.h); share: one
+// scale for both halves of an output.
+template <typename F>
+FixTab upload_fix_side(Arena& ar, int he, int halves, bool share, F&& u, cudaStream_t s) {
+  FixTab t;
+  t.nt = (he + 7) / 8;
+  t.ks = (he + 15) / 16;
+  std::vector<uint16_t> frag((size_t)halves * t.nt * t.ks * 3 * 32 * 8, 0);
+  std::vector<int> ex(16 * (size_t)t.nt, 0);
+  for (int i = 0; i < he; ++i) {
+    int e[2] = {0, 0};
+    for (int par = 0; par < halves; ++par) {
+      double mx = 0, sum = 0;
+      for (int k = 0; k < he; ++k) {
+        mx = std::max(mx, std::fabs(u(k, i, par)));
+        sum += std::fabs(u(k, i, par));
+      }
+      e[par] = mx > 0 ? std::max(std::ilogb(mx) + 1 - kFixUBits, std::ilogb(sum) + 1 - kFixSumBits)
+                      : -4096;
+    }
+    if (share) e[0] = e[1] = std::max(e[0], e[1]);
+    for (int par = 0; par < halves; ++par) {
+      if (e[par] == -4096) e[par] = 0;   // no entries: zeros at any scale
+      ex[(size_t)par * 8 * t.nt + i] = e[par];
+      for (int k = 0; k < he; ++k) {
+        long long v = std::llrint(std::ldexp(u(k, i, par), -e[par]));
+        // operand position: column i % 8, row k % 16 of step k / 16
+        const int kk = k % 16, lane = (i % 8) * 4 + (kk % 8) / 2, reg = kk / 8;
+        for (int d = kFixSlices - 1; d >= 0; --d) {
+          const int digit = (int)((v + 512) & 1023) - 512;   // balanced, FP16 holds it exactly
+          v = (v - digit) >> kFixDigit;
+          const size_t q = (((size_t)(par * t.nt + i / 8) * t.ks + k / 16) * 3 + d / 2) * 32 + lane;
+          frag[q * 8 + (d % 2) * 4 + reg * 2 + kk % 2] = half_bits(digit);
+        }
+      }
+    }
+  }
+  uint16_t* fd = ar.alloc<uint16_t>(frag.size());
+  int* ed = ar.alloc<int>(ex.size());
+  ck(cudaMemcpyAsync(fd, frag.data(), frag.size() * 2, cudaMemcpyHostToDevice, s), "fix");
+  ck(cudaMemcpyAsync(ed, ex.data(), ex.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
+  ck(cudaStreamSynchronize(s), "fix");
+  t.frag = reinterpret_cast<const uint4*>(fd);
+  t.ex = ed;
+  return t;
+}
+
+// U: columns [he even modes; n - he odd modes], each exactly even or odd
+FixTabs upload_fix(Arena& ar, const Dense& U, int he, cudaStream_t s) {
+  const int h = U.rows - he;
+  FixTabs f;
+  f.fw = upload_fix_side(ar, he, 2, false, [&](int k, int i, int par) {
+    return par == 0 ? U(k, i) : (k < h && i < h ? U(k, he + i) : 0.0);
+  }, s);
+  f.bw = upload_fix_side(ar, he, 2, true, [&](int k, int i, int par) {
+    return par == 0 ? U(i, k) : (k < h && i < h ? U(i, he + k) : 0.0);
+  }, s);
+  return f;
+}
+
+// y = D x
+FixTabs upload_fix_plain(Arena& ar, const Dense& D, cudaStream_t s) {
+  FixTabs f;
+  f.fw = upload_fix_side(ar, D.rows, 1, false, [&](int k, int i, int) { return D(i, k); }, s);
+  return f;
+}
+
 // One hyper-power Horner step applied by the pass that produces A~ t (see PassArgs): mode 1 sets
 // r = x - A~ t, acc = x + r; mode 2 sets r = r - A~ t, acc = acc + r. r, acc, x have the layout of
 // the product.
@@ -215,11 +294,11 @@ struct Ops {
   const T *U_N = nullptr, *lam_N = nullptr, *U_T = nullptr, *lam_T = nullptr;
   const T* invd = nullptr;   // FP64: 1 / (2 nu (l1 + l2 + l3)) per velocity entry
   int eo_N = 0, eo_T = 0;    // FP64: even-mode counts of the parity-split eigenvectors
+  FixTabs fx_N, fx_T;        // FP64: the eigenvectors in slices (fix.h; null for short lines)
   int fd_fused = 0;          // FP64: fast diagonalisation by the fused plane / x3-line kernels,
                              // with this many blocks per plane (0: six single-direction passes)
-  const T* chol_lb = nullptr;          // pressure block: banded Cholesky factor of M-check
-  const T* chol_inv = nullptr;
-  int chol_p = 0;
+  FixTabs fx_Minv;           // FP64: M-check^-1 in slices (plain; null below 64 entries),
+  const T* Minv = nullptr;   // and in doubles
   T *tK = nullptr, *tM = nullptr, *tS = nullptr, *tR = nullptr;   // component-size temporaries
   T *f1 = nullptr, *f2 = nullptr;                                 // mode-product ping-pong
   T *delta = nullptr, *m1 = nullptr, *m2 = nullptr;               // pressure-size temporaries
@@ -553,9 +632,10 @@ struct Ops {
         for (int c = 0; c < 3; ++c) {
           const int64_t o = c * nvc;
           const int e[3] = {c == 0 ? eo_N : eo_T, c == 1 ? eo_N : eo_T, c == 2 ? eo_N : eo_T};
-          pa[c] = FdPlaneArgs{x + o, f1 + o, U[c][0], U[c][1], comp(c), e[0], e[1], 1.0};
+          pa[c] = FdPlaneArgs{x + o, f1 + o, U[c][0], U[c][1], comp(c), e[0], e[1], 1.0,
+                             c == 0 ? fx_N : fx_T, c == 1 ? fx_N : fx_T};
           la[c] = FdLineArgs{f1 + o, f2 + o, U[c][2], comp(c), e[2], invd ? invd + o : nullptr,
-                             L[c][0], L[c][1], L[c][2], 2 * nu, 1.0};
+                             L[c][0], L[c][1], L[c][2], 2 * nu, 1.0, c == 2 ? fx_N : fx_T};
         }
         if (fd_plane_multi(pa, 3, 1, mode_block, fd_fused, s) && fd_line3_multi(la, 3, mode_block, s)) {
           for (int c = 0; c < 3; ++c) {
@@ -587,8 +667,9 @@ struct Ops {
           j[c] = mjob(src, dst, U[c][k], n[c][k], trans_of[st], comp(c), axis_of[st]);
         }
         j[c].eo_he = (k == c) ? eo_N : eo_T;
+        j[c].fx = (k == c) ? fx_N : fx_T;
       }
-      mode_product_multi<T>(j, 3, s);
+      ck(mode_product_multi<T>(j, 3, s), "mode product");
     }
   }
 
@@ -596,21 +677,28 @@ struct Ops {
             int eo = 0) const {
     ModeArgs<T> m = mjob(X, Y, U, n, trans, in, axis, nullptr, nullptr, nullptr, 1, post);
     m.eo_he = eo;
-    mode_product<T>(m, s);
+    m.fx = fx_T;   // (the pressure block's products, all with U_T)
+    ck(mode_product<T>(m, s), "mode product");
   }
 
   // pressure block: y = 2 nu (M-check^-1)^(x)3 x = 2 nu (U_T U_T^T)^(x)3 x
   void minv_Q(const T* x, T* y) const {
-    // FP64: banded Cholesky line solves for large b (4(p + 1) FP64 flops per entry and direction
-    // instead of 2b, exact up to rounding); for small b their sequential recurrence is
-    // latency-bound and the dense route is faster. (In FP32 the tensor-core route below is
-    // faster at every size: the line solves have one thread per line, a few warps per SM.)
+    // FP64, b >= 64: three passes with the dense M-check^-1 (not folded: the rounding of M-check's
+    // entries is not symmetric, and averaging the mirrored entries of its inverse would move it by
+    // 1e-14); below, the eigenvector route (its fused form takes as few launches).
     if constexpr (std::is_same<T, double>::value) {
-      if (chol_lb && b >= 64) {
-        ck(chol_solve_axis<T>(x, y, b, chol_p, 1, chol_lb, chol_inv, T(1), s, nb, bs), "chol");
-        ck(chol_solve_axis<T>(y, y, b, chol_p, 2, chol_lb, chol_inv, T(1), s, nb, bs), "chol");
-        ck(chol_solve_axis<T>(y, y, b, chol_p, 3, chol_lb, chol_inv, T(2) * nu, s, nb, bs),
-           "chol");
+      if (fx_Minv.fw.frag) {
+        const T* src = x;
+        T* dst[3] = {f1, f2, y};
+        for (int k = 0; k < 3; ++k) {
+          ModeArgs<T> m = mjob(src, dst[k], Minv, b, 0, Dims{b, b, b}, k + 1, nullptr, nullptr,
+                               nullptr, 1, k == 2 ? 2 * nu : T(1));
+          m.eo_he = eo_T;
+          m.fx = fx_Minv;
+          m.plain = 1;
+          ck(mode_product<T>(m, s), "mode product");
+          src = dst[k];
+        }
         return;
       }
     }
@@ -621,10 +709,10 @@ struct Ops {
     const Dims d{b, b, b};
     if constexpr (std::is_same<T, double>::value) {
       if (fused_fd_ok()) {
-        FdPlaneArgs pa{x, f1, U_T, U_T, d, eo_T, eo_T, 1.0};
-        FdLineArgs la{f1, f2, U_T, d, eo_T, nullptr, nullptr, nullptr, nullptr, 1.0, 1.0};
+        FdPlaneArgs pa{x, f1, U_T, U_T, d, eo_T, eo_T, 1.0, fx_T, fx_T};
+        FdLineArgs la{f1, f2, U_T, d, eo_T, nullptr, nullptr, nullptr, nullptr, 1.0, 1.0, fx_T};
         if (fd_plane_multi(&pa, 1, 1, mode_block, fd_fused, s) && fd_line3_multi(&la, 1, mode_block, s)) {
-          pa = FdPlaneArgs{f2, y, U_T, U_T, d, eo_T, eo_T, 2 * nu};
+          pa = FdPlaneArgs{f2, y, U_T, U_T, d, eo_T, eo_T, 2 * nu, fx_T, fx_T};
           if (fd_plane_multi(&pa, 1, 0, mode_block, fd_fused, s)) return;
         }
         throw CudaError{cudaErrorInvalidValue, "fused fast diagonalisation rejected its jobs"};
@@ -2243,10 +2331,13 @@ int stokes_setup(stokes_t* out, int n_elems, int degree_p, double nu, const stok
       if (!(l > 0.0)) throw SetupError{"K is not positive definite"};
     const Band bM = to_band(u.M, 1e-15), bK = to_band(u.K, 1e-15);
     const Band bMc = to_band(u.Mc, 1e-15), bTc = to_band(u.Tc, 1e-15);
-    std::vector<double> chol_lb_h, chol_inv_h;   // banded Cholesky factor of M-check (host)
     init_ops<double>(c, c->od, bM, bK, bMc, bTc, UN.v, lN, UT.v, lT);
     c->od.eo_N = heN;
     c->od.eo_T = heT;
+    if (!reduced(c) && heT > kFixMinHalf) {
+      c->od.fx_N = upload_fix(c->arena, UN, heN, c->stream);
+      c->od.fx_T = upload_fix(c->arena, UT, heT, c->stream);
+    }
     {
       // reciprocal eigenvalue sums of the fast diagonalisation, one per velocity entry
       std::vector<double> inv((size_t)c->nvel);
@@ -2261,31 +2352,15 @@ int stokes_setup(stokes_t* out, int n_elems, int degree_p, double nu, const stok
               inv[o++] = 1.0 / (2.0 * nu * ((*l[0])[i1] + (*l[1])[i2] + (*l[2])[i3]));
       }
       c->od.invd = upload<double>(c->arena, inv, c->stream);
-      // banded Cholesky factor of M-check (bandwidth p) for the FP64 pressure block
-      const int b = c->b, p = degree_p, w = p + 1;
-      const Dense& Mc = u.Mc;
-      Dense L(b, b);
-      for (int j = 0; j < b; ++j) {
-        double d = Mc(j, j);
-        for (int k = 0; k < j; ++k) d -= L(j, k) * L(j, k);
-        if (!(d > 0.0)) throw SetupError{"pressure mass matrix is not positive definite"};
-        L(j, j) = std::sqrt(d);
-        for (int i = j + 1; i < b; ++i) {
-          double t = Mc(i, j);
-          for (int k = 0; k < j; ++k) t -= L(i, k) * L(j, k);
-          L(i, j) = t / L(j, j);
-        }
+    }
+    {
+      Dense Minv;
+      if (!banded_inverse(u.Mc, degree_p, Minv))
+        throw SetupError{"pressure mass matrix is not positive definite"};
+      if (!reduced(c) && c->b >= 64) {
+        c->od.Minv = upload<double>(c->arena, Minv.v, c->stream);
+        c->od.fx_Minv = upload_fix_plain(c->arena, Minv, c->stream);
       }
-      chol_lb_h.assign((size_t)b * w, 0.0);
-      chol_inv_h.assign(b, 0.0);
-      for (int i = 0; i < b; ++i) {
-        chol_inv_h[i] = 1.0 / L(i, i);
-        for (int k = std::max(0, i - p); k <= i; ++k)
-          chol_lb_h[(size_t)i * w + (k - i + p)] = L(i, k);
-      }
-      c->od.chol_lb = upload<double>(c->arena, chol_lb_h, c->stream);
-      c->od.chol_inv = upload<double>(c->arena, chol_inv_h, c->stream);
-      c->od.chol_p = p;
     }
     const Ops<double>* odq = nullptr;
     if (!reduced(c)) {

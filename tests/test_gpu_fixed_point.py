@@ -1,0 +1,75 @@
+"""FP64 products in fixed point (FP16 tensor-core slices with 64-bit sums; csrc/fix.h) at the edges
+of their tiles and of the range they take.
+
+Bounds: 1e-12 relative to the largest entry for P_0^-1, the bound of test_base_preconditioner (six
+chained contractions, each within a few ulp of its largest product).
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2311_06926_gb300 import Stokes, synthetic
+
+from gpu_common import dev, host, oracle, relerr
+
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(n, p, **kw):
+    return Stokes(n, p, max_order=2, max_steps=0, **kw)
+
+
+# halves of 12 (FMA chains), 13, 16, 17, 32, 33, 41 terms (tiles of 8 outputs, steps of 16 terms, the
+# level sums moved every 2 and 5 steps); b = 63, 64, 65, 82: the eigenvector route and the dense
+# inverse
+@pytest.mark.parametrize("n,p", [(23, 1), (24, 1), (31, 1), (31, 2), (61, 2), (63, 1), (62, 3),
+                                 (78, 4)])
+def test_base_preconditioner_tile_edges(n, p):
+    S, base, _, _ = oracle(n, p)
+    x = synthetic.random_vector(S.size, 40 + n)
+    ref = np.concatenate([base.pv0_inv(x[:S.n_vel]), base.pq0_inv(x[S.n_vel:])])
+    G = _ctx(n, p, autotune=False)
+    for fused in (0, 1, 4):
+        G.set_tuning(128, 256, fused)
+        got = host(G.apply_P(dev(x)))
+        assert relerr(got[:S.n_vel], ref[:S.n_vel]) < 1e-12
+        assert relerr(got[S.n_vel:], ref[S.n_vel:]) < 1e-12
+    G.close()
+
+
+@pytest.mark.parametrize("n,p", [(29, 2), (63, 1)])
+@pytest.mark.parametrize("fused", [0, 1])
+def test_lines_outside_the_scaled_range(n, p, fused):
+    """Vectors whose lines are too small or too large to be scaled take FMA chains: the result
+    scales with the input."""
+    G = _ctx(n, p, autotune=False)
+    G.set_tuning(256, 256, fused)
+    x = dev(synthetic.random_vector(G.size, 3))
+    y = host(G.apply_P(x))
+    for e in (-900, 800):
+        z = host(G.apply_P(x * 2.0 ** e))
+        assert relerr(np.ldexp(z, -e), y) < 1e-12
+    assert not host(G.apply_P(torch.zeros_like(x))).any()
+    G.close()
+
+
+@pytest.mark.parametrize("n,p", [(29, 2), (63, 1)])
+@pytest.mark.parametrize("fused", [0, 1])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_nonfinite_entry_reaches_its_whole_tensor_only(n, p, fused, bad):
+    """P_0^-1 mixes every entry of a component (or of the pressure) and nothing else."""
+    G = _ctx(n, p, autotune=False)
+    G.set_tuning(256, 256, fused)
+    x = dev(synthetic.random_vector(G.size, 4))
+    y = host(G.apply_P(x))
+    m = G.n_vel // 3
+    for part in range(4):
+        lo, hi = part * m, (part + 1) * m if part < 3 else G.size
+        xb = x.clone()
+        xb[lo + (hi - lo) // 3] = bad
+        z = host(G.apply_P(xb))
+        assert not np.isfinite(z[lo:hi]).any()
+        keep = np.ones(G.size, bool)
+        keep[lo:hi] = False
+        assert np.array_equal(z[keep], y[keep])
+    G.close()
