@@ -67,28 +67,23 @@ __device__ __forceinline__ bool fix_slow(unsigned key) {
   const unsigned e = key >> 20;
   return key != 0u && (e < kFixMinExp || e > kFixMaxExp);
 }
-// x / 2^(emax - 1022) * 2^xbits, truncated (emax: exponent field of the largest entry)
+// x / 2^(emax - 1022) * 2^xbits, rounded (emax: exponent field of the largest entry)
 __device__ __forceinline__ long long fix_of(double x, int emax, int xbits) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (int)((hi >> 20) & 0x7ffu);
   const unsigned m = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
   // the 53-bit significand with its leading bit at bit 62
   const unsigned long long n = ((unsigned long long)__funnelshift_l(lo, m, 10) << 32) | (lo << 10);
-  const int sh = min(63 - xbits + emax - e, 63);
-  const long long v = (long long)(n >> sh);
+  const int sh = min(62 - xbits + emax - e, 63);
+  const long long v = (long long)(((n >> sh) + 1) >> 1);
   return (int)hi < 0 ? -v : v;
 }
-// s * 2^ex as a double, rounded to nearest (ex keeps it in the normal range). In integers: the
-// conversion instruction runs on the FP64 pipe.
+// s * 2^ex as a double (ex keeps it in the normal range). By the conversion instruction, on the FP64
+// pipe that these kernels leave idle (in about 20 integer instructions instead: 128^3 K apply 526
+// against 501 us, P_0^-1 914 against 901).
 __device__ __forceinline__ double fix_to_double(long long s, int ex) {
-  unsigned long long u = (unsigned long long)(s < 0 ? -s : s);
-  const int lz = __clzll((long long)u);
-  u <<= lz & 63;
-  // the leading one of u >> 11 adds one to the exponent field
-  const unsigned long long m =
-      (u >> 11) + ((u >> 10) & 1) + ((unsigned long long)(unsigned)(ex + 1085 - lz) << 52);
-  const unsigned hi = (unsigned)(m >> 32) | (s < 0 ? 0x80000000u : 0u);
-  return s == 0 ? 0.0 : __hiloint2double((int)hi, (int)(unsigned)m);
+  const double d = (double)s;
+  return s == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + ex * (1 << 20), __double2loint(d));
 }
 #endif
 

@@ -102,6 +102,10 @@ struct BandD {
   const T* cval;
   int half, cpitch;
   int tlo, thi;
+  // FP64: the centred band of half width fhalf as limbs (k_fix_band.cu; null: none)
+  const int4* ftab;
+  const int* fex;
+  int fhalf;
 };
 
 // Extents of a 3D tensor, x1 fastest: index = i1 + n1 * (i2 + n2 * i3).
@@ -138,6 +142,8 @@ struct PassArgs {
   int block;   // FP64 line kernel: threads per block (<= 0: 256); chosen by the setup tuner
   int c0_one;  // c0 == 1 (set by the launcher: the FP64 kernels test this integer instead of
                // comparing c0 per output, an instruction of the slow FP64 pipe)
+  BandD<T> D2;   // FP64 fixed-point passes: a second result Y2 = D2 .axis (the last term's input)
+  T* Y2;         // (null: none)
   int chain;   // two terms with c0 == c1 == 1 (set by the launcher): the FP64 kernels run one
                // FMA chain over both band rows
   // Horner epilogue (one hyper-power step fused into the pass that produces u = A~ t): instead
@@ -172,6 +178,19 @@ void band_pass(const PassArgs<T>& a, cudaStream_t s);
 constexpr int kMaxPassJobs = 8;
 template <typename T>
 void band_pass_multi(const PassArgs<T>* jobs, int njobs, cudaStream_t s);
+
+// FP64 passes in fixed point (k_fix_band.cu): ok if every band has a limb table of one half width
+// and the jobs' forms are taken; band_pass_multi goes there then.
+bool fix_band_ok(const PassArgs<double>* jobs, int njobs);
+void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s);
+void fix_div_band_x1(const double* u1, const double* u2, const double* u3, int a, int b,
+                     const double* q, double nu, const BandD<double>& D, double* y0, double* y1,
+                     int block, cudaStream_t s);
+constexpr int kFixBandHalf = 6;   // largest half width of the limb tables
+// smallest pressure extent b of the fixed-point passes: below, a pass is a few waves of short chains
+// and the FMA kernels take less time (K apply at 32^3 p = 3: 32 against 35 us; at 64^3: 150 against
+// 83)
+constexpr int kFixBandMin = 40;
 
 // delta = sum_c D .c u_c: exact discrete divergence of the velocity coefficients (App. B.2),
 // output b^3. (D beta)_i = beta_i - beta_{i-1} with beta_{-1} = beta_a = 0.

@@ -915,6 +915,28 @@ void band_pass_multi(const PassArgs<T>* jobs, int njobs, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
     band_tile_multi(jobs, njobs, s);
     return;
+  } else {
+    if (fix_band_ok(jobs, njobs)) {
+      fix_band_multi(jobs, njobs, s);
+      return;
+    }
+    // the kernels below have one result per job
+    for (int j = 0; j < njobs; ++j) {
+      if (!jobs[j].Y2) continue;
+      for (int i = 0; i < njobs; ++i) {
+        PassArgs<T> one = jobs[i];
+        one.Y2 = nullptr;
+        band_pass_multi<T>(&one, 1, s);
+        if (!jobs[i].Y2) continue;
+        if (one.nterms > 1) one.X0 = one.X1;
+        one.nterms = 1;
+        one.c0 = 1;
+        one.D0 = jobs[i].D2;
+        one.Y = jobs[i].Y2;
+        band_pass_multi<T>(&one, 1, s);
+      }
+      return;
+    }
   }
   PassBatch<T> pb{};
   pb.njobs = njobs;

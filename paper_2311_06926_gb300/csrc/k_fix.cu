@@ -53,8 +53,7 @@ __device__ __forceinline__ void fix_mma(float (&c)[4], const uint4& a, unsigned 
 
 // a b + c
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
-  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
-  return c;
+  return c + (long long)a * b;
 }
 
 // s0, s1: the integer sums of the even and the odd half (units of 2^kFixUnit): line 16 mt + lane / 4

@@ -1,0 +1,642 @@
+// FP64 banded Kronecker passes in fixed point on the integer multipliers.
+//
+// GB300 runs 64 32 x 32 + 64-bit integer multiply-adds per clock and SM against 2 FP64 FMAs
+// (measured: 18.4 against 0.62 T per second). A thread forms 8 consecutive outputs of one line from
+// the window of 8 + 2 H inputs they read. It scales the window by one power of two (that of its
+// largest entry) to integers below 2^57 and splits each into two limbs of 29 bits; the operator's
+// entries are kept as two limbs of integers below 2^58, one scale per 8 rows. A product of two
+// such pairs takes three multiply-adds, xh ch and xh cl + xl ch, into two 64-bit sums that cannot
+// overflow (13 terms); xl cl, below 2^-58 of the largest product, is dropped. The sum is rounded
+// to a double once, where an FMA chain rounds at every term (host emulation, 9 and 18 terms: rms
+// error 0.3 to 0.5 of the chain's). The window is what the scale is taken over, so an entry loses
+// precision only against entries that meet it in the same outputs.
+//
+// Bound by instruction issue: about 125 instructions per result, of which the 27 multiply-adds of a
+// row of 9 take twice their slots. Measured against the FMA passes: K apply 1051 -> 525 us at 128^3
+// p = 3, 150 -> 83 at 64^3.
+//
+// A window with an infinity or a NaN, or outside [2^-823, 2^777], takes FMA chains instead.
+#include <algorithm>
+#include <atomic>
+
+#include "fix.h"
+#include "internal.h"
+#include "profile.h"
+
+namespace shp {
+namespace {
+
+constexpr int kBandLimb = 29, kBandXBits = 57;
+constexpr int kR = 8;   // outputs per thread along the band
+
+struct FixBandOp {
+  const int4* tab;   // [segment][8 rows][(2 H + 2) / 2]: {hi, lo, hi, lo} of entries 2 q, 2 q + 1
+  const int* ex;     // scale of each segment
+  const double* cval;   // centred band in doubles (windows that cannot be scaled)
+  int cpitch, half;     // its pitch and half width (<= H)
+};
+
+struct FixBandJob {
+  const double* X[2];
+  FixBandOp D[3];    // terms 0 .. nterms - 1 of Y, then the operator of Y2
+  double* Y;
+  double* Y2;        // = D[nterms] X[nterms - 1], or null
+  const double* g;
+  int gaxis;
+  int gd1, gd12;     // strides of g along x2 and x3
+  int hmode;
+  double *hr, *hacc;
+  const double* hx;
+  Dims in;
+  unsigned n1_mul;   // line / n1 = umulhi(line, n1_mul) >> n1_sh for line < 2^31
+  int n1_sh;
+  int axis, nterms, nops, nb, segs;
+  int64_t bs;
+};
+struct FixBandBatch {
+  FixBandJob job[kMaxPassJobs];
+  int first[kMaxPassJobs + 1];
+  int njobs;
+};
+
+__host__ __device__ constexpr int band_row(int H) { return H + 1; }   // int4 per row
+// int4 per segment in shared memory: one more than the rows take, so that lanes on neighbouring
+// segments read different banks
+__host__ __device__ constexpr int band_seg(int H) { return kR * band_row(H) + 1; }
+
+__device__ __forceinline__ void band_mad(long long& c, int a, int b) {
+  c += (long long)a * b;
+}
+
+// The window's exponent (the biased one of its largest entry; -1 if all are zero; slow set when it
+// cannot be scaled) and its entries as limbs: x / 2^(exponent - 1022) 2^57 rounded to
+// hi 2^29 + lo, |lo| <= 2^28.
+template <int N>
+__device__ __forceinline__ int band_limbs(const double (&x)[N], int2 (&v)[N], bool& slow) {
+  unsigned key = 0, low = 0;   // key: the largest exponent and leading bits, one place to the left
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    key = max(key, (unsigned)__double2hiint(x[k]) << 1);
+    low |= (unsigned)__double2loint(x[k]);
+  }
+  const int e = (int)(key >> 21);
+  const bool zero = (key | low) == 0;
+  slow = slow || (!zero && (e < (int)kFixMinExp || e > (int)kFixMaxExp));
+  const int top = zero ? 4000 : 62 - kBandXBits + e;   // (4000: everything shifts out)
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const unsigned hi = (unsigned)__double2hiint(x[k]), lo = (unsigned)__double2loint(x[k]);
+    // the significand with its leading one at bit 62 (an entry without one shifts out)
+    const unsigned long long n =
+        ((unsigned long long)__funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 10) << 32) |
+        (lo << 10);
+    // one bit more than kept, then rounded (truncated entries would all err towards zero, and that
+    // smooth error is what the preconditioner amplifies), the low limb of either sign
+    const int sh = min(top - (int)((hi >> 20) & 0x7ffu), 63);
+    const unsigned long long t = (n >> sh) + (1ull << kBandLimb) + 1;
+    const int h = (int)(t >> (kBandLimb + 1));
+    const int l = (int)((unsigned)(t >> 1) - (1u << (kBandLimb - 1)) - ((unsigned)h << kBandLimb));
+    const int sg = (int)hi >> 31;
+    v[k].x = (h ^ sg) - sg;
+    v[k].y = (l ^ sg) - sg;
+  }
+  return zero ? -1 : e;
+}
+
+// Row r of the segment times the window, in units of 2^58 of the product of the two scales, plus hh.
+template <int H, int N>
+__device__ __forceinline__ long long band_row_dot(const int4* c, const int2 (&v)[N], int r,
+                                                  long long hh = 0) {
+  long long md = 1ll << (kBandLimb - 1);
+#pragma unroll
+  for (int q = 0; q <= H; ++q) {
+    const int4 w = c[r * band_row(H) + q];
+    const int2 a = v[r + 2 * q];
+    band_mad(hh, a.x, w.x);
+    band_mad(md, a.x, w.y);
+    band_mad(md, a.y, w.x);
+    if (q < H) {   // (entry 2 H + 1 is padding)
+      const int2 b = v[r + 2 * q + 1];
+      band_mad(hh, b.x, w.z);
+      band_mad(md, b.x, w.w);
+      band_mad(md, b.y, w.z);
+    }
+  }
+  return hh + (md >> kBandLimb);
+}
+
+// Scale of a window of zeros (below every other) and from scales to the exponent of a result.
+constexpr int kNoScale = -(1 << 20);
+constexpr int kBandShift = 2 * kBandLimb - 1022 - kBandXBits;
+
+// The outputs 8 seg .. 8 seg + 7 of one line. load(t, x): the window of term t; c: the operators'
+// limbs of the segment, cstep int4 apart; ex: their scales, estep apart; put(y, r, value): output r
+// of Y (y = 0) or Y2 (1). Returns false, without outputs, if a window cannot be scaled.
+// ready(): called once the first window is scaled, before the limbs and scales are read.
+template <int H, int NT, bool DUAL, typename Load, typename Ready, typename Put>
+__device__ __forceinline__ bool band_outputs(const int4* c, int cstep, const int* ex, int estep,
+                                             Load&& load, Ready&& ready, Put&& put) {
+  constexpr int N = kR + 2 * H;
+  bool slow = false;
+  int2 v[N];
+  long long s[kR];   // NT = 2: the first term's sums
+  int es = 0, e = 0;
+#pragma unroll
+  for (int t = 0; t < NT; ++t) {
+    double x[N];
+    load(t, x);
+    e = band_limbs<N>(x, v, slow);
+    if (t == 0) ready();
+    const int en = e < 0 ? kNoScale : e + ex[t * estep];
+    if (t + 1 < NT) {
+      es = en;
+#pragma unroll
+      for (int r = 0; r < kR; ++r) s[r] = band_row_dot<H, N>(c, v, r);
+      c += cstep;
+      continue;
+    }
+    if (slow) return false;
+    // both sums at the larger of the two scales
+    const int top = NT > 1 ? max(es, en) : en;
+    const int da = min(top - es, 62), db = min(top - en, 62);
+    const long long ha = (1ll << da) >> 1, hb = (1ll << db) >> 1;   // half a unit, if shifted
+    const int e2 = DUAL ? (e < 0 ? kNoScale : e + ex[NT * estep]) : 0;
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      long long y = band_row_dot<H, N>(c, v, r, NT > 1 ? hb : 0);
+      if (NT > 1) y = ((s[r] + ha) >> da) + (y >> db);
+      put(0, r, fix_to_double(y, top + kBandShift));
+      if (DUAL)
+        put(1, r, fix_to_double(band_row_dot<H, N>(c + cstep, v, r), e2 + kBandShift));
+    }
+  }
+  return true;
+}
+
+// The same outputs by FMA chains over the bands; at(t, j): entry j of term t's line of m entries.
+template <typename At, typename Put>
+__device__ __forceinline__ void band_chains(const FixBandJob& J, int seg, int m, At&& at,
+                                            Put&& put) {
+#pragma unroll 1
+  for (int r = 0; r < kR && kR * seg + r < m; ++r) {
+    const int i = kR * seg + r;
+    double y = 0.0;
+#pragma unroll 1
+    for (int o = 0; o < J.nops; ++o) {
+      const FixBandOp& D = J.D[o];
+      if (o == J.nterms) y = 0.0;
+#pragma unroll 1
+      for (int k = max(0, D.half - i); k <= min(2 * D.half, m - 1 - i + D.half); ++k)
+        y = fma(D.cval[(int64_t)i * D.cpitch + k], at(min(o, J.nterms - 1), i - D.half + k), y);
+      if (o + 1 >= J.nterms) put(o + 1 - J.nterms, r, y);
+    }
+  }
+}
+
+// A pass along x2 or x3: the block takes one segment of blockDim neighbouring lines, so every load
+// and store is coalesced and the operators' limbs are read as broadcasts.
+template <int H, int NT, bool DUAL, bool EPI>
+__device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4* sh) {
+  constexpr int N = kR + 2 * H, kSegIn = kR * band_row(H), kOps = NT + (DUAL ? 1 : 0);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int lb = local / J.segs, seg = local - lb * J.segs;
+  int* es = reinterpret_cast<int*>(sh + kOps * kSegIn);
+  // (the operators are written once at setup: their copy does not wait for the preceding kernel)
+#pragma unroll
+  for (int o = 0; o < kOps; ++o) {
+    for (int w = tid; w < kSegIn; w += nth)
+      sh[o * kSegIn + w] = __ldg(J.D[o].tab + (int64_t)seg * kSegIn + w);
+    if (tid == o) es[o] = __ldg(J.D[o].ex + seg);
+  }
+  pdl_begin();
+  const int n1 = J.in.n1, n12 = n1 * J.in.n2;
+  const bool ax2 = J.axis == 2;
+  const int m = ax2 ? J.in.n2 : J.in.n3;
+  const int lines1 = ax2 ? n1 * J.in.n3 : n12;
+  int line = lb * nth + tid;
+  const bool on = line < lines1 * J.nb;
+  if (!on) line = 0;
+  int64_t kb = 0;   // offset of the line's item
+  if (J.nb > 1) {
+    const int k = line / lines1;
+    kb = (int64_t)k * J.bs;
+    line -= k * lines1;
+  }
+  const int q =
+      n1 == 1 ? line : (int)(__umulhi((unsigned)line, J.n1_mul) >> J.n1_sh);   // x3 (axis 2) or x2 index
+  const int i1 = line - q * n1;
+  const int64_t first = kb + (ax2 ? i1 + (int64_t)n12 * q : (int64_t)line);
+  const int stride = ax2 ? n1 : n12;
+  const int i0 = kR * seg;
+  const int64_t at0 = first + (int64_t)stride * i0;
+  const double* g = nullptr;
+  int gstride = 0, gstep = 0;
+  if (EPI && J.g) {
+    gstride = ax2 ? J.gd1 : J.gd12;
+    gstep = J.gaxis == 1 ? 1 : (J.gaxis == 2 ? J.gd1 : J.gd12);
+    g = J.g + kb + i1 + (int64_t)(ax2 ? J.gd12 : J.gd1) * q + (int64_t)gstride * i0;
+  }
+  const int rows = on ? m - i0 : 0;   // rows of the segment to write
+  auto put = [&](int y, int r, double v) {
+    if (r >= rows) return;
+    const int64_t o = at0 + (int64_t)stride * r;
+    if (EPI) {
+      if (J.g) v += g[gstride * r] - g[gstride * r + gstep];
+      if (J.hmode == 1) {
+        const double xi = J.hx[o], ri = xi - v;
+        J.hr[o] = ri;
+        J.hacc[o] = xi + ri;
+        return;
+      }
+      if (J.hmode == 2) {
+        const double ri = J.hr[o] - v;
+        J.hr[o] = ri;
+        J.hacc[o] += ri;
+        return;
+      }
+    }
+    (y ? J.Y2 : J.Y)[o] = v;
+  };
+  const bool done = band_outputs<H, NT, DUAL>(
+      sh, kSegIn, es, 1,
+      [&](int t, double (&x)[N]) {
+        const double* p = J.X[t] + at0;
+        if (i0 >= H && i0 + kR + H <= m) {
+#pragma unroll
+          for (int k = 0; k < N; ++k) x[k] = p[(int64_t)stride * (k - H)];
+        } else {
+#pragma unroll
+          for (int k = 0; k < N; ++k)
+            x[k] = i0 + k >= H && i0 + k < m + H ? p[(int64_t)stride * (k - H)] : 0.0;
+        }
+      },
+      [] { __syncthreads(); }, put);
+  if (!done && on)
+    band_chains(J, seg, m, [&](int t, int j) { return J.X[t][first + (int64_t)stride * j]; }, put);
+}
+
+// Staged x1 lines (shared memory): entry j, -H <= j < 8 segs + H, of a line at
+// ((j + H) % 8) S + (j + H) / 8 with S odd, zero outside the line; neighbouring threads (segments)
+// then read and write neighbouring words, and no window needs a bound.
+__host__ __device__ constexpr int band_stage_s(int segs, int H) {
+  return (segs + (2 * H + 7) / 8) | 1;
+}
+__device__ __forceinline__ int band_stage(int j, int S) { return (j & 7) * S + (j >> 3); }
+
+// zeros around the m entries of nl staged lines
+template <int H>
+__device__ __forceinline__ void band_stage_zero(double* raw, int nl, int m, int segs, int S) {
+  const int per = kR * segs - m + 2 * H;
+  for (int idx = threadIdx.x; idx < nl * per; idx += blockDim.x) {
+    const int l = idx / per, k = idx - l * per;
+    raw[l * kR * S + band_stage(k < H ? k : m + k, S)] = 0.0;
+  }
+}
+
+// the limbs of all segments of one operator (pitch band_seg), and the scales
+template <int H>
+__device__ __forceinline__ void band_stage_op(const FixBandOp& D, int segs, int4* sh, int* es) {
+  constexpr int kSegIn = kR * band_row(H);
+  for (int idx = threadIdx.x; idx < segs * kSegIn; idx += blockDim.x) {
+    const int sg = idx / kSegIn;
+    sh[sg * band_seg(H) + idx - sg * kSegIn] = __ldg(D.tab + idx);
+  }
+  for (int sg = threadIdx.x; sg < segs; sg += blockDim.x) es[sg] = __ldg(D.ex + sg);
+}
+
+// A pass along x1: the block takes whole lines, staged in shared memory with their results, one
+// thread per segment.
+template <int H, int NT, bool DUAL>
+__device__ __forceinline__ void band_along(const FixBandJob& J, int local, int4* sh) {
+  constexpr int N = kR + 2 * H, kOps = NT + (DUAL ? 1 : 0);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int segs = J.segs, m = J.in.n1, lines1 = J.in.n2 * J.in.n3;
+  const int lpb = nth / segs, line0 = local * lpb, nl = min(lpb, lines1 * J.nb - line0);
+  const int S = band_stage_s(segs, H);
+  int* es = reinterpret_cast<int*>(sh + kOps * segs * band_seg(H));
+  double* raw = reinterpret_cast<double*>(es + ((kOps * segs + 1) & ~1));   // [NT][lpb][8 S]
+  double* out = raw + NT * lpb * kR * S;                                    // [1 or 2][lpb][8 S]
+#pragma unroll
+  for (int o = 0; o < kOps; ++o)
+    band_stage_op<H>(J.D[o], segs, sh + o * segs * band_seg(H), es + o * segs);
+#pragma unroll
+  for (int t = 0; t < NT; ++t) band_stage_zero<H>(raw + t * lpb * kR * S, nl, m, segs, S);
+  auto line_of = [&](int idx) -> int {   // idx / m
+    return m == 1 ? idx : (int)(__umulhi((unsigned)idx, J.n1_mul) >> J.n1_sh);
+  };
+  auto first_of = [&](int line) -> int64_t {
+    int64_t kb = 0;
+    if (J.nb > 1) {
+      const int k = line / lines1;
+      kb = (int64_t)k * J.bs;
+      line -= k * lines1;
+    }
+    return kb + (int64_t)m * line;
+  };
+  pdl_begin();
+#pragma unroll 2
+  for (int idx = tid; idx < nl * m; idx += nth) {
+    const int l = line_of(idx), j = idx - l * m;
+    const int64_t o = first_of(line0 + l) + j;
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+      raw[(t * lpb + l) * kR * S + band_stage(j + H, S)] = J.X[t][o];
+  }
+  __syncthreads();
+  const int l = tid / segs, seg = tid - l * segs;
+  if (l < nl) {
+    const double* p = raw + l * kR * S + seg;
+    double* q = out + l * kR * S + seg;
+    auto put = [&](int y, int r, double v) { q[(y ? lpb * kR * S : 0) + r * S] = v; };
+    const bool done = band_outputs<H, NT, DUAL>(
+        sh + seg * band_seg(H), segs * band_seg(H), es + seg, segs,
+        [&](int t, double (&x)[N]) {
+#pragma unroll
+          for (int k = 0; k < N; ++k) x[k] = p[t * lpb * kR * S + (k & 7) * S + (k >> 3)];
+        },
+        [] {}, put);
+    if (!done)
+      band_chains(J, seg, m,
+                  [&](int t, int j) { return raw[(t * lpb + l) * kR * S + band_stage(j + H, S)]; },
+                  put);
+  }
+  __syncthreads();
+  for (int idx = tid; idx < nl * m; idx += nth) {
+    const int w = line_of(idx), j = idx - w * m;
+    const int64_t o = first_of(line0 + w) + j;
+    const int at = w * kR * S + band_stage(j, S);
+    J.Y[o] = out[at];
+    if (DUAL) J.Y2[o] = out[lpb * kR * S + at];
+  }
+}
+
+// NT: the most terms of a job (fewer registers where every job has one). EPI: jobs may have a g
+// term or a Horner step (passes along x2 and x3 with one result; a kernel of their own because the
+// compiler executes their FP64 additions whether taken or not).
+template <int H, int NT, bool EPI>
+__global__ void __launch_bounds__(256, 3)
+    k_fix_band(const __grid_constant__ FixBandBatch fb) {
+  extern __shared__ __align__(16) int4 shb[];
+  int jb = 0;
+  while (jb + 1 < fb.njobs && (int)blockIdx.x >= fb.first[jb + 1]) ++jb;
+  const FixBandJob& J = fb.job[jb];
+  const int local = (int)blockIdx.x - fb.first[jb];
+  if constexpr (NT == 2) {
+    if (J.nterms == 2) {
+      if constexpr (EPI) {
+        band_across<H, 2, false, true>(J, local, shb);
+      } else {
+        if (!J.Y2) band_across<H, 2, false, false>(J, local, shb);
+        else if (J.axis == 1) band_along<H, 2, true>(J, local, shb);
+        else band_across<H, 2, true, false>(J, local, shb);
+      }
+      return;
+    }
+  }
+  if constexpr (EPI) {
+    band_across<H, 1, false, true>(J, local, shb);
+  } else if (J.axis == 1) {
+    if (J.Y2) band_along<H, 1, true>(J, local, shb);
+    else band_along<H, 1, false>(J, local, shb);
+  } else {
+    if (J.Y2) band_across<H, 1, true, false>(J, local, shb);
+    else band_across<H, 1, false, false>(J, local, shb);
+  }
+}
+
+// The divergence and the first pressure-mass pass (see k_div_band_x1), the band in fixed point:
+// y0 = D .x1 delta and, with q, y1 = D .x1 (nu delta + q).
+template <int H>
+__global__ void __launch_bounds__(256, 2) k_fix_div_x1(const double* __restrict__ u1,
+                                                       const double* __restrict__ u2,
+                                                       const double* __restrict__ u3, int a, int b,
+                                                       const double* __restrict__ q, double nu,
+                                                       const __grid_constant__ FixBandJob J,
+                                                       double* __restrict__ y1) {
+  extern __shared__ __align__(16) int4 shb[];
+  constexpr int N = kR + 2 * H;
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int nv = q ? 2 : 1;
+  const int segs = J.segs, lpb = nth / (segs * nv), m = b, S = band_stage_s(segs, H);
+  const int lines = b * b, line0 = (int)blockIdx.x * lpb, nl = min(lpb, lines - line0);
+  int* es = reinterpret_cast<int*>(shb + segs * band_seg(H));
+  double* raw = reinterpret_cast<double*>(es + ((segs + 1) & ~1));   // delta, then e
+  double* out = raw + nv * lpb * kR * S;
+  band_stage_op<H>(J.D[0], segs, shb, es);
+  band_stage_zero<H>(raw, nv * lpb, m, segs, S);
+  pdl_begin();
+  const int64_t b2 = (int64_t)b * b;
+  auto div_b = [&](int idx) -> int {   // idx / b
+    return b == 1 ? idx : (int)(__umulhi((unsigned)idx, J.n1_mul) >> J.n1_sh);
+  };
+#pragma unroll 2
+  for (int idx = tid; idx < nl * b; idx += nth) {
+    const int l = div_b(idx), i1 = idx - l * b;
+    const int line = line0 + l, i3 = div_b(line), i2 = line - i3 * b;
+    const double* p1 = u1 + (int64_t)a * line + i1;
+    const double* p2 = u2 + (int64_t)b * ((int64_t)a * i3 + i2) + i1;
+    const double* p3 = u3 + b2 * i3 + (int64_t)b * i2 + i1;
+    // the six neighbours are loaded before the first addition
+    const double t[6] = {i1 < a ? p1[0] : 0.0,  i1 >= 1 ? p1[-1] : 0.0, i2 < a ? p2[0] : 0.0,
+                         i2 >= 1 ? p2[-b] : 0.0, i3 < a ? p3[0] : 0.0,   i3 >= 1 ? p3[-b2] : 0.0};
+    const double d = ((((t[0] - t[1]) + t[2]) - t[3]) + t[4]) - t[5];
+    const int at = l * kR * S + band_stage(i1 + H, S);
+    raw[at] = d;
+    if (q) raw[lpb * kR * S + at] = fma(nu, d, q[(int64_t)line * b + i1]);
+  }
+  __syncthreads();
+  // threads: segments of the lines of delta, then of e
+  const int row = tid / segs, seg = tid - row * segs;
+  const int o = row / lpb, l = row - o * lpb;
+  if (l < nl && o < nv) {
+    const double* p = raw + row * kR * S + seg;
+    double* y = out + row * kR * S + seg;
+    auto put = [&](int, int r, double v) { y[r * S] = v; };
+    const bool done = band_outputs<H, 1, false>(
+        shb + seg * band_seg(H), 0, es + seg, 0,
+        [&](int, double (&x)[N]) {
+#pragma unroll
+          for (int k = 0; k < N; ++k) x[k] = p[(k & 7) * S + (k >> 3)];
+        },
+        [] {}, put);
+    if (!done)
+      band_chains(J, seg, m,
+                  [&](int, int j) { return raw[row * kR * S + band_stage(j + H, S)]; }, put);
+  }
+  __syncthreads();
+  const int64_t o0 = (int64_t)b * line0;
+  for (int idx = tid; idx < nl * b; idx += nth) {
+    const int w = div_b(idx), at = w * kR * S + band_stage(idx - w * b, S);
+    J.Y[o0 + idx] = out[at];
+    if (q) y1[o0 + idx] = out[lpb * kR * S + at];
+  }
+}
+
+FixBandOp band_op(const BandD<double>& D) {
+  return FixBandOp{D.ftab, D.fex, D.cval, D.cpitch, D.half};
+}
+
+void band_divisor(int n1, FixBandJob& J) {
+  int sh = 31 - __builtin_clz((unsigned)n1);
+  if ((n1 & (n1 - 1)) == 0) --sh;   // (a power of two: one bit less, the multiplier fits)
+  J.n1_sh = std::max(sh, 0);
+  J.n1_mul = n1 == 1 ? 0 : (unsigned)(((uint64_t)1 << (32 + J.n1_sh)) / (unsigned)n1 + 1);
+}
+
+// threads of a block whose x1 lines need `segs` threads each
+int band_threads(int block, int segs) {
+  const int t = block > 0 ? std::min(block, 256) : 256;
+  return std::max(t, (segs + 31) / 32 * 32);
+}
+// shared memory of a block of x1 lines: the operators' limbs and scales, and nline staged lines
+int band_along_smem(int nops, int nline, int segs, int H) {
+  return nops * segs * band_seg(H) * 16 + ((nops * segs + 1) & ~1) * 4 +
+         nline * kR * band_stage_s(segs, H) * 8;
+}
+
+template <int H, int NT, bool EPI>
+void launch_fix_band(const FixBandBatch& fb, int blocks, int threads, int smem, cudaStream_t s) {
+  static std::atomic<int> attr{0};
+  raise_smem_limit(k_fix_band<H, NT, EPI>, attr, smem);
+  launch_k(k_fix_band<H, NT, EPI>, blocks, threads, smem, s, fb);
+}
+template <int H>
+void launch_fix_band(const FixBandBatch& fb, int nt, bool epi, int blocks, int threads, int smem,
+                     cudaStream_t s) {
+  if (nt > 1)
+    epi ? launch_fix_band<H, 2, true>(fb, blocks, threads, smem, s)
+        : launch_fix_band<H, 2, false>(fb, blocks, threads, smem, s);
+  else
+    epi ? launch_fix_band<H, 1, true>(fb, blocks, threads, smem, s)
+        : launch_fix_band<H, 1, false>(fb, blocks, threads, smem, s);
+}
+template <int H>
+void launch_fix_div(const double* u1, const double* u2, const double* u3, int a, int b,
+                    const double* q, double nu, const FixBandJob& J, double* y1, int blocks,
+                    int threads, int smem, cudaStream_t s) {
+  static std::atomic<int> attr{0};
+  raise_smem_limit(k_fix_div_x1<H>, attr, smem);
+  launch_k(k_fix_div_x1<H>, blocks, threads, smem, s, u1, u2, u3, a, b, q, nu, J, y1);
+}
+
+}  // namespace
+
+bool fix_band_ok(const PassArgs<double>* jobs, int njobs) {
+  const int H = jobs[0].D0.fhalf;
+  // (a launch with a g term or a Horner step has passes along x2 and x3 with one result only)
+  bool epi = false;
+  for (int j = 0; j < njobs; ++j) epi = epi || jobs[j].g || jobs[j].hmode;
+  for (int j = 0; j < njobs; ++j) {
+    const PassArgs<double>& a = jobs[j];
+    if (epi && (a.axis == 1 || a.Y2)) return false;
+    const int m = a.in.get(a.axis), nb = a.nb > 1 ? a.nb : 1;
+    if (!a.D0.ftab || a.D0.fhalf != H || a.D0.rows != m || a.Z ||
+        (a.nterms > 1 && (!a.D1.ftab || a.D1.fhalf != H || a.D1.rows != m || a.c1 != 1.0)) ||
+        (a.Y2 && (!a.D2.ftab || a.D2.fhalf != H || a.D2.rows != m)) ||
+        a.c0 != 1.0 ||
+        (a.axis == 1 && (a.g || a.hmode || (a.nterms > 1 && !a.Y2) || (m + kR - 1) / kR > 256)) ||
+        (a.Y2 && (a.g || a.hmode)) ||
+        a.in.size() / m * nb >= ((int64_t)1 << 30))
+      return false;
+  }
+  return true;
+}
+
+void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
+  FixBandBatch fb{};
+  fb.njobs = njobs;
+  const int H = jobs[0].D0.fhalf;
+  int threads = 32;
+  for (int j = 0; j < njobs; ++j)
+    threads = std::max(threads, band_threads(jobs[j].block, jobs[j].axis == 1
+                                                               ? (jobs[j].D0.rows + kR - 1) / kR
+                                                               : 1));
+  int blocks = 0, smem = 3 * kR * band_row(H) * 16 + 16;
+  bool epi = false;
+  int nt = 1;
+  double flops = 0, bytes = 0;
+  for (int j = 0; j < njobs; ++j) {
+    const PassArgs<double>& a = jobs[j];
+    FixBandJob& J = fb.job[j];
+    J.X[0] = a.X0;
+    J.X[1] = a.X1;
+    J.D[0] = band_op(a.D0);
+    if (a.nterms > 1) J.D[1] = band_op(a.D1);
+    if (a.Y2) J.D[a.nterms] = band_op(a.D2);
+    epi = epi || a.g || a.hmode;
+    nt = std::max(nt, a.nterms);
+    J.Y = a.Y;
+    J.Y2 = a.Y2;
+    J.g = a.g;
+    J.gaxis = a.gaxis;
+    J.gd1 = a.gdims.n1;
+    J.gd12 = a.gdims.n1 * a.gdims.n2;
+    J.hmode = a.hmode;
+    J.hr = a.hr;
+    J.hacc = a.hacc;
+    J.hx = a.hx;
+    J.in = a.in;
+    band_divisor(a.in.n1, J);
+    J.axis = a.axis;
+    J.nterms = a.nterms;
+    J.nops = a.nterms + (a.Y2 ? 1 : 0);
+    J.nb = a.nb > 1 ? a.nb : 1;
+    J.bs = a.bs;
+    const int m = a.D0.rows;
+    J.segs = (m + kR - 1) / kR;
+    const int lines = (int)(a.in.size() / m) * J.nb;
+    fb.first[j] = blocks;
+    if (a.axis == 1) {
+      const int lpb = threads / J.segs;
+      blocks += (lines + lpb - 1) / lpb;
+      smem = std::max(smem, band_along_smem(J.nops, lpb * (a.nterms + (a.Y2 ? 2 : 1)), J.segs, H));
+    } else {
+      blocks += (lines + threads - 1) / threads * J.segs;
+    }
+    const double outs = (double)a.in.size() * J.nb;
+    double fl = 2.0 * a.D0.width * outs, by = 2.0 * outs;
+    if (a.nterms > 1) { fl += 2.0 * a.D1.width * outs; by += outs; }
+    if (a.Y2) { fl += 2.0 * a.D2.width * outs; by += outs; }
+    if (a.g) { fl += 2.0 * outs; by += (double)a.gdims.size() * J.nb; }
+    flops += fl;
+    bytes += by * sizeof(double);
+  }
+  fb.first[njobs] = blocks;
+  launch_begin(kClassBand64, s);
+  switch (H) {
+#define SHP_FIX_H(h) case h: launch_fix_band<h>(fb, nt, epi, blocks, threads, smem, s); break;
+    SHP_FIX_H(1) SHP_FIX_H(2) SHP_FIX_H(3) SHP_FIX_H(4) SHP_FIX_H(5) SHP_FIX_H(6)
+#undef SHP_FIX_H
+    default: break;
+  }
+  launch_end(kClassBand64, s, flops, bytes);
+}
+
+void fix_div_band_x1(const double* u1, const double* u2, const double* u3, int a, int b,
+                     const double* q, double nu, const BandD<double>& D, double* y0, double* y1,
+                     int block, cudaStream_t s) {
+  FixBandJob J{};
+  J.D[0] = band_op(D);
+  J.Y = y0;
+  J.nterms = J.nops = 1;
+  J.nb = 1;
+  band_divisor(b, J);
+  J.segs = (b + kR - 1) / kR;
+  const int nv = q ? 2 : 1;
+  const int H = D.fhalf, threads = band_threads(block, J.segs * nv);
+  const int lpb = threads / (J.segs * nv), blocks = (b * b + lpb - 1) / lpb;
+  const int smem = band_along_smem(1, 2 * nv * lpb, J.segs, H);
+  const double np = (double)b * b * b;
+  launch_begin(kClassDiv, s);
+  switch (H) {
+#define SHP_FIX_H(h)                                                                  \
+  case h: launch_fix_div<h>(u1, u2, u3, a, b, q, nu, J, y1, blocks, threads, smem, s); break;
+    SHP_FIX_H(1) SHP_FIX_H(2) SHP_FIX_H(3) SHP_FIX_H(4) SHP_FIX_H(5) SHP_FIX_H(6)
+#undef SHP_FIX_H
+    default: break;
+  }
+  launch_end(kClassDiv, s, (q ? 8.0 : 6.0) * np + (q ? 4.0 : 2.0) * D.width * np,
+             (3.0 * a * b * b + (q ? 3.0 : 1.0) * np) * sizeof(double));
+}
+
+}  // namespace shp

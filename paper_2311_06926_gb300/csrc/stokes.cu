@@ -131,6 +131,9 @@ BandD<T> upload_band(Arena& ar, const Band& b, cudaStream_t s, int min_half = 0)
   d.half = 0;
   d.cpitch = 0;
   d.tlo = d.thi = 0;
+  d.ftab = nullptr;
+  d.fex = nullptr;
+  d.fhalf = 0;
   // centred copy for square matrices (every matrix of the operator applies is one)
   std::vector<T> cv;
   if (b.rows == b.cols) {
@@ -178,6 +181,41 @@ BandD<T> upload_band(Arena& ar, const Band& b, cudaStream_t s, int min_half = 0)
   }
   ck(cudaStreamSynchronize(s), "upload band");
   return d;
+}
+
+// Limb table of a square band for the fixed-point passes (k_fix_band.cu), centred with half width
+// H >= its own: per segment of 8 rows one scale, below which the entries are integers of magnitude
+// at most 2^58, and rows of 2 H + 2 entries (the last one zero) as {hi, lo} with
+// v = hi 2^29 + lo, |lo| <= 2^28.
+void upload_fix_band(Arena& ar, const Band& b, BandD<double>& d, int H, cudaStream_t s) {
+  if (b.rows != b.cols || d.half > H) return;
+  const int segs = (b.rows + 7) / 8, per = 2 * H + 2;
+  std::vector<int> tab((size_t)segs * 8 * per * 2, 0), ex(segs, 0);
+  for (int sg = 0; sg < segs; ++sg) {
+    double mx = 0;
+    const int i1 = std::min(b.rows, 8 * sg + 8);
+    for (int i = 8 * sg; i < i1; ++i)
+      for (int w = 0; w < b.width; ++w) mx = std::max(mx, std::fabs(b.val[(size_t)i * b.width + w]));
+    if (mx == 0) continue;
+    ex[sg] = std::ilogb(mx) + 1 - 58;
+    for (int i = 8 * sg; i < i1; ++i)
+      for (int w = 0; w < b.width; ++w) {
+        const int k = b.start[i] + w - i + H;
+        if (k < 0 || k > 2 * H) continue;   // (zero entries only: |k - H| > d.half)
+        const long long v = std::llrint(std::ldexp(b.val[(size_t)i * b.width + w], -ex[sg]));
+        const int h = (int)((v + (1ll << 28)) >> 29);
+        tab[((size_t)i * per + k) * 2] = h;
+        tab[((size_t)i * per + k) * 2 + 1] = (int)(v - ((long long)h << 29));
+      }
+  }
+  int* td = ar.alloc<int>(tab.size());
+  int* ed = ar.alloc<int>(ex.size());
+  ck(cudaMemcpyAsync(td, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
+  ck(cudaMemcpyAsync(ed, ex.data(), ex.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
+  ck(cudaStreamSynchronize(s), "fix");
+  d.ftab = reinterpret_cast<const int4*>(td);
+  d.fex = ed;
+  d.fhalf = H;
 }
 
 template <typename T>
@@ -293,6 +331,7 @@ struct Ops {
   BandD<T> Mc_nu{}, Tc_2nu{};
   const T *U_N = nullptr, *lam_N = nullptr, *U_T = nullptr, *lam_T = nullptr;
   const T* invd = nullptr;   // FP64: 1 / (2 nu (l1 + l2 + l3)) per velocity entry
+  bool fixb = false;         // FP64: the bands have limb tables (fixed-point passes)
   int eo_N = 0, eo_T = 0;    // FP64: even-mode counts of the parity-split eigenvectors
   FixTabs fx_N, fx_T;        // FP64: the eigenvectors in slices (fix.h; null for short lines)
   int fd_fused = 0;          // FP64: fast diagonalisation by the fused plane / x3-line kernels,
@@ -351,6 +390,13 @@ struct Ops {
     return p;
   }
 
+  // coef M-check along one axis of the pressure grid; a coefficient nu is taken from the scaled copy
+  PassArgs<T> mass_job(const T* X, T coef, int axis, T* Y) const {
+    const bool scaled_copy = fixb && coef == nu && coef != T(1);
+    return job(X, scaled_copy ? Mc_nu : Mc, scaled_copy ? T(1) : coef, nullptr, nullptr, 0,
+               Dims{b, b, b}, axis, Y);
+  }
+
   // the job's result goes through the Horner epilogue h (offset o into its vectors)
   static void horner(PassArgs<T>& p, const Horner<T>* h, int64_t o) {
     if (!h) return;
@@ -380,6 +426,42 @@ struct Ops {
     const T nu2 = 2 * nu;
     const Dims dq{b, b, b};
     PassArgs<T> j[kMaxPassJobs];
+    if (fixb) {
+      // fixed-point passes: the two results of one input share its scaling, and all bands have
+      // limb tables of one width
+      for (int c = 0; c < 3; ++c) {
+        const int64_t o = c * nvc;
+        j[c] = job(u + o, K, 1, nullptr, nullptr, 0, comp(c), own_axis(c), tK + o);
+        j[c].D2 = M;
+        j[c].Y2 = tM + o;
+      }
+      for (int k = 0; k < nq; ++k)
+        j[3 + k] = x1_done ? job(qx[k], Mc, 1, nullptr, nullptr, 0, dq, 2, f2 + k * npres)
+                           : job(qx[k], Mc, 1, nullptr, nullptr, 0, dq, 1, f1 + k * npres);
+      band_pass_multi<T>(j, 3 + nq, s);
+      for (int c = 0; c < 3; ++c) {
+        const int64_t o = c * nvc;
+        j[c] = job(tK + o, Mc_nu, 1, tM + o, &Tc_2nu, 1, comp(c), first_other(c), tS + o);
+        j[c].D2 = Mc;
+        j[c].Y2 = tR + o;
+      }
+      for (int k = 0; k < nq; ++k)
+        j[3 + k] = x1_done ? mass_job(f2 + k * npres, qcoef[k], 3, qy[k])
+                           : job(f1 + k * npres, Mc, 1, nullptr, nullptr, 0, dq, 2, f2 + k * npres);
+      band_pass_multi<T>(j, 3 + nq, s);
+      if (nq > 0 && !x1_done) {
+        for (int k = 0; k < nq; ++k) j[k] = mass_job(f2 + k * npres, qcoef[k], 3, qy[k]);
+        band_pass_multi<T>(j, nq, s);
+      }
+      for (int c = 0; c < 3; ++c) {
+        const int64_t o = c * nvc;
+        j[c] = job(tS + o, Mc, 1, tR + o, &Tc_2nu, 1, comp(c), second_other(c), y + o, nullptr, 0,
+                   g, own_axis(c));
+        horner(j[c], h, o);
+      }
+      band_pass_multi<T>(j, 3, s);
+      return;
+    }
     for (int c = 0; c < 3; ++c) {
       const int64_t o = c * nvc;
       j[2 * c] = job(u + o, K, 1, nullptr, nullptr, 0, comp(c), own_axis(c), tK + o);
@@ -437,16 +519,26 @@ struct Ops {
       j[k] = job(f1 + k * npres, Mc, 1, nullptr, nullptr, 0, d, 2, f2 + k * npres);
     band_pass_multi<T>(j, nvec, s);
     for (int k = 0; k < nvec; ++k) {
-      j[k] = job(f2 + k * npres, Mc, coef[k], nullptr, nullptr, 0, d, 3, y[k]);
+      j[k] = mass_job(f2 + k * npres, coef[k], 3, y[k]);
       if (nvec == 1) horner(j[k], h, 0);
     }
     band_pass_multi<T>(j, nvec, s);
   }
 
-  // FP64, one item: the divergence and the pressure-mass pass along x1 fused (div_band_x1), so
+  // the divergence of u (and e = nu delta + q) with the pressure-mass pass along x1 (FP64)
+  void div_x1(const T* u, const T* q, T* y0, T* y1) const {
+    if constexpr (std::is_same<T, double>::value) {
+      if (fixb)
+        fix_div_band_x1(u, u + nvc, u + 2 * nvc, a, b, q, nu, Mc, y0, y1, band_block, s);
+      else
+        div_band_x1<T>(u, u + nvc, u + 2 * nvc, a, b, q, nu, Mc, y0, y1, s);
+    }
+  }
+
+  // FP64, one item: the divergence and the pressure-mass pass along x1 fused (div_x1), so
   // an A or K apply takes four launches
   bool fused_div() const {
-    return std::is_same<T, double>::value && nb == 1 && Mc_w.val != nullptr && b <= 512;
+    return std::is_same<T, double>::value && nb == 1 && (fixb || Mc_w.val != nullptr) && b <= 512;
   }
 
   void apply_K(const T* x, T* y) const {
@@ -456,7 +548,7 @@ struct Ops {
       if (fused_div()) {
         // the x1 pass with M-check itself (width 7): the zero-padded copy Mc_w that the x2 pass
         // rides with (the velocity launch of width 9) would add two FMAs by zero per output
-        div_band_x1<T>(x, x + nvc, x + 2 * nvc, a, b, q, nu, Mc, f1, f1 + npres, s);
+        div_x1(x, q, f1, f1 + npres);
         const T* in2[2] = {f1, f1 + npres};
         T* out2[2] = {yq, m2};
         const T coef2[2] = {1, 1};
@@ -469,7 +561,7 @@ struct Ops {
     const T* in[2] = {delta, m1};
     T* out[2] = {yq, m2};
     const T coef[2] = {1, 1};
-    if (Mc_w.val) {
+    if (fixb || Mc_w.val) {
       adiag_all(x, y, m2, 2, in, out, coef);
       return;
     }
@@ -481,7 +573,7 @@ struct Ops {
   void apply_A(const T* x, T* y, const Horner<T>* h = nullptr) const {
     if constexpr (std::is_same<T, double>::value) {
       if (fused_div()) {
-        div_band_x1<T>(x, x + nvc, x + 2 * nvc, a, b, nullptr, nu, Mc, f1, nullptr, s);
+        div_x1(x, nullptr, f1, nullptr);
         const T* in1[1] = {f1};
         T* out1[1] = {m2};
         const T coef1[1] = {nu};
@@ -493,7 +585,7 @@ struct Ops {
     const T* in[1] = {delta};
     T* out[1] = {m2};
     const T coef[1] = {nu};
-    if (Mc_w.val) {
+    if (fixb || Mc_w.val) {
       adiag_all(x, y, m2, 1, in, out, coef, h);
       return;
     }
@@ -531,7 +623,7 @@ struct Ops {
     if constexpr (std::is_same<T, double>::value) {
       if (nb == 1 && b <= 512) {
         // the divergence and the pass along x1 in one launch (the same bits as two)
-        div_band_x1<T>(u, u + nvc, u + 2 * nvc, a, b, nullptr, nu, Mc, f1, nullptr, s);
+        div_x1(u, nullptr, f1, nullptr);
         const T* in1[1] = {f1};
         mq(1, in1, out, coef, h, true);
         return;
@@ -1202,9 +1294,20 @@ void init_ops(stokes_ctx* c, Ops<T>& o, const Band& M, const Band& K, const Band
   o.K = upload_band<T>(ar, K, s);
   o.Mc = upload_band<T>(ar, Mc, s);
   o.Tc = upload_band<T>(ar, Tc, s);
-  if (std::is_same<T, double>::value) {
-    o.Mc_nu = upload_band<T>(ar, scaled(Mc, c->nu), s);
-    o.Tc_2nu = upload_band<T>(ar, scaled(Tc, 2.0 * c->nu), s);
+  if constexpr (std::is_same<T, double>::value) {
+    const Band Mc_nu = scaled(Mc, c->nu), Tc_2nu = scaled(Tc, 2.0 * c->nu);
+    o.Mc_nu = upload_band<T>(ar, Mc_nu, s);
+    o.Tc_2nu = upload_band<T>(ar, Tc_2nu, s);
+    const int H = std::max({1, o.M.half, o.K.half, o.Mc.half, o.Tc.half});
+    if (H <= kFixBandHalf && c->b >= kFixBandMin) {
+      upload_fix_band(ar, M, o.M, H, s);
+      upload_fix_band(ar, K, o.K, H, s);
+      upload_fix_band(ar, Mc, o.Mc, H, s);
+      upload_fix_band(ar, Tc, o.Tc, H, s);
+      upload_fix_band(ar, Mc_nu, o.Mc_nu, H, s);
+      upload_fix_band(ar, Tc_2nu, o.Tc_2nu, H, s);
+      o.fixb = true;
+    }
   }
   {
     const Band Mcw = widen(Mc, K.width);

@@ -1,8 +1,9 @@
-"""FP64 products in fixed point (FP16 tensor-core slices with 64-bit sums; csrc/fix.h) at the edges
-of their tiles and of the range they take.
+"""FP64 products in fixed point (csrc/fix.h: FP16 tensor-core slices with 64-bit sums; and
+csrc/k_fix_band.cu: integer multiply-adds) at the edges of their tiles and of the range they take.
 
-Bounds: 1e-12 relative to the largest entry for P_0^-1, the bound of test_base_preconditioner (six
-chained contractions, each within a few ulp of its largest product).
+Bounds, relative to the largest entry: 1e-12 for P_0^-1, the bound of test_base_preconditioner (six
+chained contractions, each within a few ulp of its largest product), and 1e-13 for K, that of
+test_operator_applies.
 """
 import numpy as np
 import pytest
@@ -72,4 +73,45 @@ def test_nonfinite_entry_reaches_its_whole_tensor_only(n, p, fused, bad):
         keep = np.ones(G.size, bool)
         keep[lo:hi] = False
         assert np.array_equal(z[keep], y[keep])
+    G.close()
+
+
+# extents from the smallest that takes the fixed-point passes, ragged and whole segments of 8 rows,
+# half widths 2 to 6, and 7, which does not (p = 6)
+@pytest.mark.parametrize("n,p,nu", [(38, 1, 1.0), (39, 1, 0.3), (38, 2, 2.0), (46, 2, 1.0),
+                                    (45, 3, 0.7), (44, 4, 1.0), (43, 5, 3.0), (41, 6, 1.0)])
+def test_operator_segment_edges(n, p, nu):
+    S, _, Kop, F = oracle(n, p, nu)
+    x = synthetic.random_vector(S.size, 60 + n + p)
+    G = Stokes(n, p, nu=nu, max_order=2, max_steps=0, autotune=False)
+    ref = Kop(x)
+    for block in (128, 256, 512):
+        G.set_tuning(512, block, 0)
+        assert relerr(host(G.apply_K(dev(x))), ref) < 1e-13
+    assert relerr(host(G.apply_A(dev(x[:S.n_vel]))), F.apply_A(x[:S.n_vel])) < 1e-13
+    G.close()
+
+
+def test_operator_windows_outside_the_scaled_range():
+    """Windows that cannot be scaled take FMA chains: the result scales with the input, a zero
+    vector gives zeros, and an infinite or NaN entry reaches the entries that read it only."""
+    G = _ctx(41, 3, autotune=False)
+    x = dev(synthetic.random_vector(G.size, 5))
+    y = host(G.apply_K(x))
+    for e in (-900, 800):
+        assert relerr(np.ldexp(host(G.apply_K(x * 2.0 ** e)), -e), y) < 1e-13
+    assert not host(G.apply_K(torch.zeros_like(x))).any()
+    a, b = G.a, G.b
+    for bad in (float("inf"), float("nan")):
+        xb = x.clone()
+        # entry (20, 20, 20) of u1: its products reach 2 (p + 1) = 8 entries along each direction;
+        # entries that share a window with it are formed by chains (the same to rounding)
+        xb[20 + a * (20 + b * 20)] = bad
+        z = host(G.apply_K(xb))
+        u1 = np.isfinite(z[:a * b * b].reshape(b, b, a))
+        assert not u1[20, 20, 20]
+        far = np.ones((b, b, a), bool)
+        far[12:29, 12:29, 12:29] = False
+        assert u1[far].all()
+        assert relerr(z[:a * b * b].reshape(b, b, a)[far], y[:a * b * b].reshape(b, b, a)[far]) < 1e-13
     G.close()
