@@ -115,6 +115,14 @@ int stokes_setup(stokes_t* out, int n_elems, int degree_p, double nu, const stok
 /* n_vel = 3 a b^2 and n_pres = b^3 (either pointer may be NULL). */
 int stokes_sizes(stokes_t ctx, int64_t* n_vel, int64_t* n_pres);
 
+/* Order the context's stream against another stream of the same device (a cudaStream_t, NULL: the
+ * legacy default stream), without waiting on the host: stokes_wait_for makes later work of the
+ * context wait for what `stream` holds now (inputs written there), stokes_release_to makes later
+ * work of `stream` wait for what the context has enqueued (outputs read there). Nothing is done
+ * when it is the context's own stream. Errors: STOKES_ERR_ARG, STOKES_ERR_CUDA. */
+int stokes_wait_for(stokes_t ctx, void* stream);
+int stokes_release_to(stokes_t ctx, void* stream);
+
 /* Select the preconditioner used by stokes_solve: the order-`order` hyper-power sequence after
  * `steps` steps (Eq. 2.1 for order 2; steps = 0 is the base P_0). Requires 2 <= order <=
  * max_order and 0 <= steps <= max_steps. */

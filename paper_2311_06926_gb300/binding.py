@@ -69,6 +69,8 @@ def load_library(path=None):
         "stokes_setup": (ctypes.c_int, [ctypes.POINTER(vp), ctypes.c_int, ctypes.c_int,
                                         ctypes.c_double, ctypes.POINTER(_Opts)]),
         "stokes_sizes": (ctypes.c_int, [vp, i64p, i64p]),
+        "stokes_wait_for": (ctypes.c_int, [vp, vp]),
+        "stokes_release_to": (ctypes.c_int, [vp, vp]),
         "stokes_set_preconditioner": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int]),
         "stokes_apply_A": (ctypes.c_int, [vp, vp, vp]),
         "stokes_apply_K": (ctypes.c_int, [vp, vp, vp]),
@@ -159,7 +161,7 @@ def fd_apply_noalloc(U, lam, scale, x, y):
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()   # (the argument types convert it)
 
 
 class Stokes:
@@ -210,10 +212,12 @@ class Stokes:
 
     # -- helpers -------------------------------------------------------------------------------
     def _call(self, fn, *args):
-        cur = torch.cuda.current_stream(self.device)
-        self.stream.wait_stream(cur)
+        # ordered by the library (one event per direction, made at setup): two torch events per call
+        # were half of what a small call cost on the host
+        cur = torch.cuda.current_stream(self.device).cuda_stream
+        self._check(self.lib.stokes_wait_for(self.h, cur))
         rc = fn(*args)
-        cur.wait_stream(self.stream)
+        self._check(self.lib.stokes_release_to(self.h, cur))
         return rc
 
     def _check(self, rc):

@@ -21,32 +21,29 @@ std::vector<double> open_knots(int n, int d) {
   return t;
 }
 
-// Index s with t[s] <= x < t[s+1]; x = 1 belongs to the last non-empty span.
+// Index s with t[s] <= x < t[s+1]; x = 1 belongs to the last non-empty span (0 below the knots).
 int find_span(const std::vector<double>& t, double x) {
-  int last = 0;
-  for (int i = 0; i + 1 < (int)t.size(); ++i)
-    if (t[i] < t[i + 1]) {
-      if (t[i] <= x) last = i;
-    }
-  return last;
+  int s = (int)(std::upper_bound(t.begin(), t.end(), x) - t.begin()) - 1;
+  s = std::min(s, (int)t.size() - 2);
+  while (s > 0 && !(t[s] < t[s + 1])) --s;
+  return std::max(s, 0);
 }
 
-// Values of all degree-d B-splines at x (size nf = len(t) - d - 1).
+// Values of all degree-d B-splines at x (size nf = len(t) - d - 1). Only the functions that can be
+// nonzero on x's span are formed (the recursion's other terms are products with zero).
 std::vector<double> bspline_values(const std::vector<double>& t, int d, double x) {
-  const int m = (int)t.size() - 1;
+  const int m = (int)t.size() - 1, s = find_span(t, x);
   std::vector<double> N(m, 0.0);
-  N[find_span(t, x)] = 1.0;
-  for (int k = 1; k <= d; ++k) {
-    std::vector<double> Nn(m - k, 0.0);
-    for (int i = 0; i < m - k; ++i) {
+  N[s] = 1.0;
+  for (int k = 1; k <= d; ++k)
+    for (int i = std::max(0, s - k); i <= std::min(s, m - k - 1); ++i) {
       double v = 0.0;
       const double d1 = t[i + k] - t[i], d2 = t[i + k + 1] - t[i + 1];
       if (d1 > 0) v += (x - t[i]) / d1 * N[i];
       if (d2 > 0) v += (t[i + k + 1] - x) / d2 * N[i + 1];
-      Nn[i] = v;
+      N[i] = v;
     }
-    N.swap(Nn);
-  }
+  N.resize(m - d);
   return N;
 }
 
@@ -484,10 +481,12 @@ std::vector<double> sine_load(const Univariate& u, int k, bool use_N) {
     const double f = std::sin(k * M_PI * xs[qi]) * ws[qi];
     if (use_N) {
       std::vector<double> Nv = bspline_values(tN, p + 1, xs[qi]);
-      for (int i = 0; i < u.a; ++i) out[i] += f * Nv[i + 1];
+      for (int i = 0; i < u.a; ++i)
+        if (Nv[i + 1] != 0.0) out[i] += f * Nv[i + 1];
     } else {
       std::vector<double> Mv = bspline_values(tM, p, xs[qi]);
-      for (int i = 0; i < u.b; ++i) out[i] += f * Mv[i] * (p + 1) / (tM[i + p + 1] - tM[i]);
+      for (int i = 0; i < u.b; ++i)
+        if (Mv[i] != 0.0) out[i] += f * Mv[i] * (p + 1) / (tM[i + p + 1] - tM[i]);
     }
   }
   return out;
@@ -514,8 +513,10 @@ Dense lid_profile_matrix(const Univariate& u, int ncoef) {
     for (size_t q = 0; q < g.size(); ++q) {
       const double x = 0.5 * (lo + hi) + 0.5 * (hi - lo) * g[q], w = 0.5 * (hi - lo) * gw[q];
       const std::vector<double> Nv = bspline_values(tN, p + 1, x), Sv = bspline_values(tS, 3, x);
-      for (int i = 0; i < u.a; ++i)
+      for (int i = 0; i < u.a; ++i) {
+        if (Nv[i + 1] == 0.0) continue;
         for (int k = 0; k < ncoef; ++k) G(i, k) += w * Nv[i + 1] * Sv[k];
+      }
     }
   }
   return G;

@@ -1063,6 +1063,7 @@ struct stokes_ctx {
   Ops<double> od;
   Ops<double> odq;                       // FP64 operators of the concurrent pressure branch
   cudaStream_t stream_q = nullptr;       // its stream (owned)
+  cudaEvent_t ev_in = nullptr, ev_out = nullptr;   // stokes_wait_for, stokes_release_to
   Ops<float> of;
   Ops<float> ofq;                        // reduced-precision operators of the pressure branch
   QuadOps* quad = nullptr;               // quadrature-based forward operator (opts.forward)
@@ -2341,6 +2342,20 @@ void autotune(stokes_ctx* c) {
 }
 
 
+// The 1D sine loads of one call, each wave number formed once: a mode needs three of them, and the
+// 24 modes of a call share a few wave numbers (64^3 gradient: 144 loads of 1536 quadrature points
+// took 100 of its 142 ms).
+struct SineLoads {
+  const Univariate& u;
+  std::map<std::pair<int, bool>, std::vector<double>> have;
+  const std::vector<double>& get(int k, bool own) {
+    auto it = have.find({k, own});
+    if (it == have.end())
+      it = have.emplace(std::make_pair(k, own), own ? sine_load_N(u, k) : sine_load_M(u, k)).first;
+    return it->second;
+  }
+};
+
 }  // namespace
 
 // ============================================================================================
@@ -2417,6 +2432,8 @@ int stokes_setup(stokes_t* out, int n_elems, int degree_p, double nu, const stok
       ck(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking), "stream");
       c->own_stream = true;
     }
+    ck(cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming), "event");
+    ck(cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming), "event");
     c->uv = build_univariate(n_elems, degree_p, o.c_pen);
     const Univariate& u = c->uv;
     std::vector<double> lN, lT;
@@ -2564,6 +2581,26 @@ int stokes_sizes(stokes_t c, int64_t* n_vel, int64_t* n_pres) {
   return STOKES_OK;
 }
 
+namespace {
+// later work of `after` waits for what `before` holds now
+int order_streams(stokes_t c, cudaStream_t before, cudaStream_t after, cudaEvent_t ev) {
+  if (before == after) return STOKES_OK;
+  const cudaError_t e = cudaEventRecord(ev, before);
+  const cudaError_t f = e == cudaSuccess ? cudaStreamWaitEvent(after, ev, 0) : e;
+  return f == cudaSuccess ? STOKES_OK : cuda_fail(c, CudaError{f, "stream order"});
+}
+}  // namespace
+
+int stokes_wait_for(stokes_t c, void* stream) {
+  if (!c) return STOKES_ERR_ARG;
+  return order_streams(c, static_cast<cudaStream_t>(stream), c->stream, c->ev_in);
+}
+
+int stokes_release_to(stokes_t c, void* stream) {
+  if (!c) return STOKES_ERR_ARG;
+  return order_streams(c, c->stream, static_cast<cudaStream_t>(stream), c->ev_out);
+}
+
 int stokes_set_preconditioner(stokes_t c, int order, int steps) {
   if (!c) return STOKES_ERR_ARG;
   if (order < 2 || order > c->opts.max_order || steps < 0 || steps > c->opts.max_steps)
@@ -2672,6 +2709,7 @@ int stokes_rhs_body(stokes_t c, int n_modes, const double* coef, const int* wave
     fill_zero(tmp, c->nvel * sizeof(double), c->stream);
     const int ld = c->b + 1;
     std::vector<double> l(3 * (size_t)ld);
+    SineLoads loads{u, {}};
     for (int comp = 0; comp < 3; ++comp) {
       const int e1 = comp == 0 ? c->a : c->b, e2 = comp == 1 ? c->a : c->b;
       const int e3 = comp == 2 ? c->a : c->b;
@@ -2679,9 +2717,9 @@ int stokes_rhs_body(stokes_t c, int n_modes, const double* coef, const int* wave
         const double cf = coef[comp * n_modes + m];
         if (cf == 0.0) continue;
         const int* k = waves + (size_t)(comp * n_modes + m) * 3;
-        const std::vector<double> l1 = comp == 0 ? sine_load_N(u, k[0]) : sine_load_M(u, k[0]);
-        const std::vector<double> l2 = comp == 1 ? sine_load_N(u, k[1]) : sine_load_M(u, k[1]);
-        const std::vector<double> l3 = comp == 2 ? sine_load_N(u, k[2]) : sine_load_M(u, k[2]);
+        const std::vector<double>& l1 = loads.get(k[0], comp == 0);
+        const std::vector<double>& l2 = loads.get(k[1], comp == 1);
+        const std::vector<double>& l3 = loads.get(k[2], comp == 2);
         std::copy(l1.begin(), l1.end(), l.begin());
         std::copy(l2.begin(), l2.end(), l.begin() + ld);
         std::copy(l3.begin(), l3.end(), l.begin() + 2 * ld);
@@ -2777,6 +2815,7 @@ int stokes_body_load_dots(stokes_t c, int n_modes, const int* waves, const doubl
     if (waves[i] < 1 || waves[i] > 64) return fail(c, STOKES_ERR_ARG, "wave numbers in [1, 64]");
   const Univariate& u = c->uv;
   const int ld = c->b + 1;
+  SineLoads loads{u, {}};
   try {
     for (int comp = 0; comp < 3; ++comp) {
       const int e1 = comp == 0 ? c->a : c->b, e2 = comp == 1 ? c->a : c->b;
@@ -2784,9 +2823,9 @@ int stokes_body_load_dots(stokes_t c, int n_modes, const int* waves, const doubl
       std::vector<double> fac((size_t)n_modes * 3 * ld, 0.0);
       for (int m = 0; m < n_modes; ++m) {
         const int* k = waves + (size_t)(comp * n_modes + m) * 3;
-        const std::vector<double> l1 = comp == 0 ? sine_load_N(u, k[0]) : sine_load_M(u, k[0]);
-        const std::vector<double> l2 = comp == 1 ? sine_load_N(u, k[1]) : sine_load_M(u, k[1]);
-        const std::vector<double> l3 = comp == 2 ? sine_load_N(u, k[2]) : sine_load_M(u, k[2]);
+        const std::vector<double>& l1 = loads.get(k[0], comp == 0);
+        const std::vector<double>& l2 = loads.get(k[1], comp == 1);
+        const std::vector<double>& l3 = loads.get(k[2], comp == 2);
         double* f = fac.data() + (size_t)m * 3 * ld;
         std::copy(l1.begin(), l1.end(), f);
         std::copy(l2.begin(), l2.end(), f + ld);
@@ -3023,6 +3062,8 @@ void stokes_destroy(stokes_t c) {
   if (c->stream_q) cudaStreamSynchronize(c->stream_q);
   cudaStream_t s = c->own_stream ? c->stream : nullptr;
   cudaStream_t sq = c->stream_q;
+  if (c->ev_in) cudaEventDestroy(c->ev_in);
+  if (c->ev_out) cudaEventDestroy(c->ev_out);
   delete c;   // frees the arena
   if (s) cudaStreamDestroy(s);
   if (sq) cudaStreamDestroy(sq);
