@@ -356,7 +356,6 @@ struct FixBatch {
 // entry arithmetic (int below 2^31 entries: 64-bit division issues FP64-pipe instructions).
 template <typename IT>
 __global__ void __launch_bounds__(320, 2) k_fix_mode(const __grid_constant__ FixBatch fb) {
-  pdl_begin();
   extern __shared__ __align__(16) uint4 xf[];
   constexpr int lb = 16;
   __shared__ unsigned key[lb];
@@ -378,6 +377,7 @@ __global__ void __launch_bounds__(320, 2) k_fix_mode(const __grid_constant__ Fix
     base[l] = (line - r * JL) + JL * ((IT)K * r);
   }
   if (tid == 0) any = 0;
+  pdl_begin();
   __syncthreads();
   const auto ptr = [&](int l) { return J.X + base[l]; };
   const auto row = [&](int l) { return base[l]; };
@@ -436,7 +436,6 @@ __global__ void __launch_bounds__(512) k_fix_plane(const __grid_constant__ FixPl
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-  pdl_begin();
   extern __shared__ __align__(16) uint4 xf[];
   __shared__ unsigned key[2][256];
   __shared__ int any[2];
@@ -464,6 +463,7 @@ __global__ void __launch_bounds__(512) k_fix_plane(const __grid_constant__ FixPl
   const FixOp& B = J.second;
   for (int l = tid; l < 512; l += nth) (&key[0][0])[l] = 0;
   if (tid < 2) any[tid] = 0;
+  pdl_begin();
   __syncthreads();
   const auto ptr_a = [&](int l) { return X + (fwd ? (a0 + l) * n1 : a0 + l); };
   const auto ptr_b = [&](int l) { return (const double*)raw + l; };
@@ -514,7 +514,6 @@ struct FixLineBatch {
 // The forward x3 product, the eigenvalue scaling and the backward x3 product of 16 neighbouring x3
 // lines.
 __global__ void __launch_bounds__(512) k_fix_line3(const __grid_constant__ FixLineBatch fb) {
-  pdl_begin();
   extern __shared__ __align__(16) uint4 xf[];
   constexpr int lb = 16, P = lb + 1;
   __shared__ unsigned key[2][lb];
@@ -529,6 +528,7 @@ __global__ void __launch_bounds__(512) k_fix_line3(const __grid_constant__ FixLi
   const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, nw = nth >> 5;
   for (int l = tid; l < 2 * lb; l += nth) (&key[0][0])[l] = 0;
   if (tid < 2) any[tid] = 0;
+  pdl_begin();
   __syncthreads();
   const auto ptr_a = [&](int l) { return J.X + line0 + l; };
   const auto ptr_b = [&](int l) { return (const double*)raw + l; };

@@ -336,7 +336,7 @@ struct Ops {
   FixTabs fx_N, fx_T;        // FP64: the eigenvectors in slices (fix.h; null for short lines)
   int fd_fused = 0;          // FP64: fast diagonalisation by the fused plane / x3-line kernels,
                              // with this many blocks per plane (0: six single-direction passes)
-  FixTabs fx_Minv;           // FP64: M-check^-1 in slices (plain; null below 64 entries),
+  FixTabs fx_Minv;           // FP64: M-check^-1 in slices (plain; null for short lines),
   const T* Minv = nullptr;   // and in doubles
   T *tK = nullptr, *tM = nullptr, *tS = nullptr, *tR = nullptr;   // component-size temporaries
   T *f1 = nullptr, *f2 = nullptr;                                 // mode-product ping-pong
@@ -775,7 +775,7 @@ struct Ops {
 
   // pressure block: y = 2 nu (M-check^-1)^(x)3 x = 2 nu (U_T U_T^T)^(x)3 x
   void minv_Q(const T* x, T* y) const {
-    // FP64, b >= 64: three passes with the dense M-check^-1 (not folded: the rounding of M-check's
+    // FP64, long lines: three passes with the dense M-check^-1 (not folded: the rounding of M-check's
     // entries is not symmetric, and averaging the mirrored entries of its inverse would move it by
     // 1e-14); below, the eigenvector route (its fused form takes as few launches).
     if constexpr (std::is_same<T, double>::value) {
@@ -2477,7 +2477,7 @@ int stokes_setup(stokes_t* out, int n_elems, int degree_p, double nu, const stok
       Dense Minv;
       if (!banded_inverse(u.Mc, degree_p, Minv))
         throw SetupError{"pressure mass matrix is not positive definite"};
-      if (!reduced(c) && c->b >= 64) {
+      if (!reduced(c) && heT > kFixMinHalf) {
         c->od.Minv = upload<double>(c->arena, Minv.v, c->stream);
         c->od.fx_Minv = upload_fix_plain(c->arena, Minv, c->stream);
       }
