@@ -102,9 +102,11 @@ struct BandD {
   const T* cval;
   int half, cpitch;
   int tlo, thi;
-  // FP64: the centred band of half width fhalf as limbs (k_fix_band.cu; null: none)
+  // FP64: the band as limbs (k_fix_band.cu; null: none), centred with half width fhalf, or
+  // rectangular (fhalf = 0) with the first input of each 8-row segment in fw0
   const int4* ftab;
   const int* fex;
+  const int* fw0;
   int fhalf;
 };
 
@@ -191,6 +193,8 @@ constexpr int kFixBandHalf = 6;   // largest half width of the limb tables
 // and the FMA kernels take less time (K apply at 32^3 p = 3: 32 against 35 us; at 64^3: 150 against
 // 83)
 constexpr int kFixBandMin = 40;
+// smallest number of points per direction of the fixed-point quadrature passes
+constexpr int kFixRectMin = 64;
 
 // delta = sum_c D .c u_c: exact discrete divergence of the velocity coefficients (App. B.2),
 // output b^3. (D beta)_i = beta_i - beta_{i-1} with beta_{-1} = beta_a = 0.

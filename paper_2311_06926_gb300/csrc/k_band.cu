@@ -921,20 +921,26 @@ void band_pass_multi(const PassArgs<T>* jobs, int njobs, cudaStream_t s) {
       return;
     }
     // the kernels below have one result per job
-    for (int j = 0; j < njobs; ++j) {
-      if (!jobs[j].Y2) continue;
-      for (int i = 0; i < njobs; ++i) {
-        PassArgs<T> one = jobs[i];
-        one.Y2 = nullptr;
-        band_pass_multi<T>(&one, 1, s);
-        if (!jobs[i].Y2) continue;
-        if (one.nterms > 1) one.X0 = one.X1;
-        one.nterms = 1;
-        one.c0 = 1;
-        one.D0 = jobs[i].D2;
-        one.Y = jobs[i].Y2;
-        band_pass_multi<T>(&one, 1, s);
+    bool two = false;
+    for (int j = 0; j < njobs; ++j) two = two || jobs[j].Y2;
+    if (two) {
+      PassArgs<T> one[2 * kMaxPassJobs];
+      int n = 0;
+      for (int j = 0; j < njobs; ++j) {
+        one[n] = jobs[j];
+        one[n++].Y2 = nullptr;
+        if (!jobs[j].Y2) continue;
+        PassArgs<T>& a = one[n++];
+        a = jobs[j];
+        if (a.nterms > 1) a.X0 = a.X1;
+        a.nterms = 1;
+        a.c0 = 1;
+        a.D0 = jobs[j].D2;
+        a.Y = jobs[j].Y2;
+        a.Y2 = nullptr;
       }
+      for (int j = 0; j < n; j += kMaxPassJobs)
+        band_pass_multi<T>(one + j, std::min(kMaxPassJobs, n - j), s);
       return;
     }
   }
@@ -1104,18 +1110,22 @@ __global__ void __launch_bounds__(256) k_quad_stress(double* __restrict__ G, dou
       i3 = (int)(q12 / nq);
       i2 = (int)(q12 - (int64_t)i3 * nq);
     }
-    const double W = w[i1] * w[i2] * w[i3];
+    // 17 FP64 operations per point (the FP64 pipe bounds this kernel as much as memory does): the
+    // off-diagonal entries are symmetric, and the weight is applied once
+    const double W = w[i1] * w[i2] * w[i3], wn = W * nu;
     double g[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) g[k] = G[k * n3 + o];
-    const double q = P[o];
+    const double wq = W * P[o], wn2 = wn + wn;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) G[(4 * c) * n3 + o] = fma(wn2, g[4 * c], wq);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        double t = W * (nu * (g[3 * c + d] + g[3 * d + c]));
-        if (c == d) t += W * q;
+      for (int d = c + 1; d < 3; ++d) {
+        const double t = wn * (g[3 * c + d] + g[3 * d + c]);
         G[(3 * c + d) * n3 + o] = t;
+        G[(3 * d + c) * n3 + o] = t;
       }
     P[o] = W * (g[0] + g[4] + g[8]);
   }

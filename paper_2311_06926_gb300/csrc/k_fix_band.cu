@@ -30,10 +30,12 @@ constexpr int kBandLimb = 29, kBandXBits = 57;
 constexpr int kR = 8;   // outputs per thread along the band
 
 struct FixBandOp {
-  const int4* tab;   // [segment][8 rows][(2 H + 2) / 2]: {hi, lo, hi, lo} of entries 2 q, 2 q + 1
+  const int4* tab;   // [segment][8 rows][band_row]: {hi, lo, hi, lo} of entries 2 q, 2 q + 1
   const int* ex;     // scale of each segment
-  const double* cval;   // centred band in doubles (windows that cannot be scaled)
-  int cpitch, half;     // its pitch and half width (<= H)
+  const int* w0;     // rectangular bands (H = 0): first input of each segment's window
+  const double* val;    // the band in doubles (windows that cannot be scaled): row i's entries from
+  const int* start;     // input start[i]
+  int width;
 };
 
 struct FixBandJob {
@@ -48,6 +50,7 @@ struct FixBandJob {
   double *hr, *hacc;
   const double* hx;
   Dims in;
+  int rows;          // outputs of a line (the extent of Y along the axis)
   unsigned n1_mul;   // line / n1 = umulhi(line, n1_mul) >> n1_sh for line < 2^31
   int n1_sh;
   int axis, nterms, nops, nb, segs;
@@ -59,7 +62,10 @@ struct FixBandBatch {
   int njobs;
 };
 
-__host__ __device__ constexpr int band_row(int H) { return H + 1; }   // int4 per row
+// Half width H >= 1: centred square bands, row r of a segment reads entries r .. r + 2 H of the
+// window (2 H + 2 stored, the last one zero). H = 0: rectangular bands (the quadrature tables: several
+// points per element), whose segments read at most 8 inputs; every row has all 8.
+__host__ __device__ constexpr int band_row(int H) { return H ? H + 1 : 4; }   // int4 per row
 // int4 per segment in shared memory: one more than the rows take, so that lanes on neighbouring
 // segments read different banks
 __host__ __device__ constexpr int band_seg(int H) { return kR * band_row(H) + 1; }
@@ -108,15 +114,16 @@ template <int H, int N>
 __device__ __forceinline__ long long band_row_dot(const int4* c, const int2 (&v)[N], int r,
                                                   long long hh = 0) {
   long long md = 1ll << (kBandLimb - 1);
+  const int k0 = H ? r : 0;
 #pragma unroll
-  for (int q = 0; q <= H; ++q) {
+  for (int q = 0; q < band_row(H); ++q) {
     const int4 w = c[r * band_row(H) + q];
-    const int2 a = v[r + 2 * q];
+    const int2 a = v[k0 + 2 * q];
     band_mad(hh, a.x, w.x);
     band_mad(md, a.x, w.y);
     band_mad(md, a.y, w.x);
-    if (q < H) {   // (entry 2 H + 1 is padding)
-      const int2 b = v[r + 2 * q + 1];
+    if (H == 0 || q < H) {   // (entry 2 H + 1 is padding)
+      const int2 b = v[k0 + 2 * q + 1];
       band_mad(hh, b.x, w.z);
       band_mad(md, b.x, w.w);
       band_mad(md, b.y, w.z);
@@ -186,8 +193,8 @@ __device__ __forceinline__ void band_chains(const FixBandJob& J, int seg, int m,
       const FixBandOp& D = J.D[o];
       if (o == J.nterms) y = 0.0;
 #pragma unroll 1
-      for (int k = max(0, D.half - i); k <= min(2 * D.half, m - 1 - i + D.half); ++k)
-        y = fma(D.cval[(int64_t)i * D.cpitch + k], at(min(o, J.nterms - 1), i - D.half + k), y);
+      for (int k = 0; k < D.width; ++k)
+        y = fma(D.val[(int64_t)i * D.width + k], at(min(o, J.nterms - 1), D.start[i] + k), y);
       if (o + 1 >= J.nterms) put(o + 1 - J.nterms, r, y);
     }
   }
@@ -211,7 +218,7 @@ __device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4
   pdl_begin();
   const int n1 = J.in.n1, n12 = n1 * J.in.n2;
   const bool ax2 = J.axis == 2;
-  const int m = ax2 ? J.in.n2 : J.in.n3;
+  const int nin = ax2 ? J.in.n2 : J.in.n3, m = H ? nin : J.rows;
   const int lines1 = ax2 ? n1 * J.in.n3 : n12;
   int line = lb * nth + tid;
   const bool on = line < lines1 * J.nb;
@@ -228,7 +235,8 @@ __device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4
   const int64_t first = kb + (ax2 ? i1 + (int64_t)n12 * q : (int64_t)line);
   const int stride = ax2 ? n1 : n12;
   const int i0 = kR * seg;
-  const int64_t at0 = first + (int64_t)stride * i0;
+  // the segment's outputs (a rectangular pass along x2 has planes of another size)
+  const int64_t at0 = (H == 0 && ax2 ? kb + i1 + (int64_t)n1 * m * q : first) + (int64_t)stride * i0;
   const double* g = nullptr;
   int gstride = 0, gstep = 0;
   if (EPI && J.g) {
@@ -260,6 +268,13 @@ __device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4
   const bool done = band_outputs<H, NT, DUAL>(
       sh, kSegIn, es, 1,
       [&](int t, double (&x)[N]) {
+        if constexpr (H == 0) {
+          const int w0 = __ldg(J.D[t].w0 + seg);
+          const double* p = J.X[t] + first + (int64_t)stride * w0;
+#pragma unroll
+          for (int k = 0; k < N; ++k) x[k] = w0 + k < nin ? p[(int64_t)stride * k] : 0.0;
+          return;
+        }
         const double* p = J.X[t] + at0;
         if (i0 >= H && i0 + kR + H <= m) {
 #pragma unroll
@@ -381,7 +396,11 @@ __global__ void __launch_bounds__(256, 3)
   while (jb + 1 < fb.njobs && (int)blockIdx.x >= fb.first[jb + 1]) ++jb;
   const FixBandJob& J = fb.job[jb];
   const int local = (int)blockIdx.x - fb.first[jb];
-  if constexpr (NT == 2) {
+  if constexpr (H == 0) {
+    if (J.Y2) band_across<H, 1, true, false>(J, local, shb);
+    else band_across<H, 1, false, false>(J, local, shb);
+    return;
+  } else if constexpr (NT == 2) {
     if (J.nterms == 2) {
       if constexpr (EPI) {
         band_across<H, 2, false, true>(J, local, shb);
@@ -393,7 +412,8 @@ __global__ void __launch_bounds__(256, 3)
       return;
     }
   }
-  if constexpr (EPI) {
+  if constexpr (H == 0) {
+  } else if constexpr (EPI) {
     band_across<H, 1, false, true>(J, local, shb);
   } else if (J.axis == 1) {
     if (J.Y2) band_along<H, 1, true>(J, local, shb);
@@ -473,7 +493,7 @@ __global__ void __launch_bounds__(256, 2) k_fix_div_x1(const double* __restrict_
 }
 
 FixBandOp band_op(const BandD<double>& D) {
-  return FixBandOp{D.ftab, D.fex, D.cval, D.cpitch, D.half};
+  return FixBandOp{D.ftab, D.fex, D.fw0, D.val, D.start, D.width};
 }
 
 void band_divisor(int n1, FixBandJob& J) {
@@ -529,14 +549,17 @@ bool fix_band_ok(const PassArgs<double>* jobs, int njobs) {
   for (int j = 0; j < njobs; ++j) {
     const PassArgs<double>& a = jobs[j];
     if (epi && (a.axis == 1 || a.Y2)) return false;
-    const int m = a.in.get(a.axis), nb = a.nb > 1 ? a.nb : 1;
+    // rectangular bands: single-term passes along x2 and x3 of one item
+    if (H == 0 && (epi || a.axis == 1 || a.nterms > 1 || a.nb > 1)) return false;
+    const int m = H ? a.in.get(a.axis) : a.D0.rows, nb = a.nb > 1 ? a.nb : 1;
     if (!a.D0.ftab || a.D0.fhalf != H || a.D0.rows != m || a.Z ||
         (a.nterms > 1 && (!a.D1.ftab || a.D1.fhalf != H || a.D1.rows != m || a.c1 != 1.0)) ||
         (a.Y2 && (!a.D2.ftab || a.D2.fhalf != H || a.D2.rows != m)) ||
         a.c0 != 1.0 ||
         (a.axis == 1 && (a.g || a.hmode || (a.nterms > 1 && !a.Y2) || (m + kR - 1) / kR > 256)) ||
         (a.Y2 && (a.g || a.hmode)) ||
-        a.in.size() / m * nb >= ((int64_t)1 << 30))
+        (H == 0 && a.D0.cols != a.in.get(a.axis)) ||
+        a.in.size() / a.in.get(a.axis) * nb >= ((int64_t)1 << 30))
       return false;
   }
   return true;
@@ -583,8 +606,9 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
     J.nb = a.nb > 1 ? a.nb : 1;
     J.bs = a.bs;
     const int m = a.D0.rows;
+    J.rows = m;
     J.segs = (m + kR - 1) / kR;
-    const int lines = (int)(a.in.size() / m) * J.nb;
+    const int lines = (int)(a.in.size() / a.in.get(a.axis)) * J.nb;
     fb.first[j] = blocks;
     if (a.axis == 1) {
       const int lpb = threads / J.segs;
@@ -593,8 +617,8 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
     } else {
       blocks += (lines + threads - 1) / threads * J.segs;
     }
-    const double outs = (double)a.in.size() * J.nb;
-    double fl = 2.0 * a.D0.width * outs, by = 2.0 * outs;
+    const double outs = (double)lines * m;
+    double fl = 2.0 * a.D0.width * outs, by = (double)a.in.size() * J.nb + outs;
     if (a.nterms > 1) { fl += 2.0 * a.D1.width * outs; by += outs; }
     if (a.Y2) { fl += 2.0 * a.D2.width * outs; by += outs; }
     if (a.g) { fl += 2.0 * outs; by += (double)a.gdims.size() * J.nb; }
@@ -605,6 +629,7 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
   launch_begin(kClassBand64, s);
   switch (H) {
 #define SHP_FIX_H(h) case h: launch_fix_band<h>(fb, nt, epi, blocks, threads, smem, s); break;
+    case 0: launch_fix_band<0, 1, false>(fb, blocks, threads, smem, s); break;
     SHP_FIX_H(1) SHP_FIX_H(2) SHP_FIX_H(3) SHP_FIX_H(4) SHP_FIX_H(5) SHP_FIX_H(6)
 #undef SHP_FIX_H
     default: break;

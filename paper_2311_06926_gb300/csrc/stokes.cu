@@ -133,6 +133,7 @@ BandD<T> upload_band(Arena& ar, const Band& b, cudaStream_t s, int min_half = 0)
   d.tlo = d.thi = 0;
   d.ftab = nullptr;
   d.fex = nullptr;
+  d.fw0 = nullptr;
   d.fhalf = 0;
   // centred copy for square matrices (every matrix of the operator applies is one)
   std::vector<T> cv;
@@ -216,6 +217,44 @@ void upload_fix_band(Arena& ar, const Band& b, BandD<double>& d, int H, cudaStre
   d.ftab = reinterpret_cast<const int4*>(td);
   d.fex = ed;
   d.fhalf = H;
+}
+
+// The same for a rectangular band whose 8-row segments read at most 8 inputs each (none otherwise):
+// rows of 8 entries, from the segment's first input fw0.
+void upload_fix_rect(Arena& ar, const Band& b, BandD<double>& d, cudaStream_t s) {
+  const int segs = (b.rows + 7) / 8;
+  std::vector<int> tab((size_t)segs * 8 * 8 * 2, 0), ex(2 * (size_t)segs, 0);
+  for (int sg = 0; sg < segs; ++sg) {
+    const int i1 = std::min(b.rows, 8 * sg + 8);
+    int lo = b.cols, hi = 0;
+    double mx = 0;
+    for (int i = 8 * sg; i < i1; ++i) {
+      lo = std::min(lo, b.start[i]);
+      hi = std::max(hi, b.start[i] + b.width);
+      for (int w = 0; w < b.width; ++w) mx = std::max(mx, std::fabs(b.val[(size_t)i * b.width + w]));
+    }
+    if (hi - lo > 8) return;
+    ex[segs + sg] = lo;
+    if (mx == 0) continue;
+    ex[sg] = std::ilogb(mx) + 1 - 58;
+    for (int i = 8 * sg; i < i1; ++i)
+      for (int w = 0; w < b.width; ++w) {
+        const long long v = std::llrint(std::ldexp(b.val[(size_t)i * b.width + w], -ex[sg]));
+        const int h = (int)((v + (1ll << 28)) >> 29);
+        const size_t k = ((size_t)i * 8 + (b.start[i] + w - lo)) * 2;
+        tab[k] = h;
+        tab[k + 1] = (int)(v - ((long long)h << 29));
+      }
+  }
+  int* td = ar.alloc<int>(tab.size());
+  int* ed = ar.alloc<int>(ex.size());
+  ck(cudaMemcpyAsync(td, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
+  ck(cudaMemcpyAsync(ed, ex.data(), ex.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
+  ck(cudaStreamSynchronize(s), "fix");
+  d.ftab = reinterpret_cast<const int4*>(td);
+  d.fex = ed;
+  d.fw0 = ed + segs;
+  d.fhalf = 0;
 }
 
 template <typename T>
@@ -892,9 +931,10 @@ struct QuadOps {
       j[1] = pj(u, tab(c, 1, true, false), 1, nullptr, nullptr, 0, e, 1, s1[1]);
       band_pass_multi<double>(j, 2, s);
       j[0] = pj(s1[0], tab(c, 2, false, false), 1, nullptr, nullptr, 0, d1, 2, s2[0]);   // v v
-      j[1] = pj(s1[0], tab(c, 2, true, false), 1, nullptr, nullptr, 0, d1, 2, s2[1]);    // v d
-      j[2] = pj(s1[1], tab(c, 2, false, false), 1, nullptr, nullptr, 0, d1, 2, s2[2]);   // d v
-      band_pass_multi<double>(j, 3, s);
+      j[0].D2 = tab(c, 2, true, false);                                                  // v d
+      j[0].Y2 = s2[1];
+      j[1] = pj(s1[1], tab(c, 2, false, false), 1, nullptr, nullptr, 0, d1, 2, s2[2]);   // d v
+      band_pass_multi<double>(j, 2, s);
       double* g = G + (int64_t)3 * c * n3;
       j[0] = pj(s2[2], tab(c, 3, false, false), 1, nullptr, nullptr, 0, d2, 3, g);            // d/dx1
       j[1] = pj(s2[1], tab(c, 3, false, false), 1, nullptr, nullptr, 0, d2, 3, g + n3);       // d/dx2
@@ -2253,6 +2293,12 @@ void init_quad(stokes_ctx* c) {
   q->DN = upload_band<double>(ar, to_band(qt.DN, 0.0), s);
   q->BM = upload_band<double>(ar, to_band(qt.BM, 0.0), s);
   q->DM = upload_band<double>(ar, to_band(qt.DM, 0.0), s);
+  if (qt.nq >= kFixRectMin) {
+    upload_fix_rect(ar, to_band(qt.BN, 0.0), q->BN, s);
+    upload_fix_rect(ar, to_band(qt.DN, 0.0), q->DN, s);
+    upload_fix_rect(ar, to_band(qt.BM, 0.0), q->BM, s);
+    upload_fix_rect(ar, to_band(qt.DM, 0.0), q->DM, s);
+  }
   q->BNt = upload_band<double>(ar, to_band(transposed(qt.BN), 0.0), s);
   q->DNt = upload_band<double>(ar, to_band(transposed(qt.DN), 0.0), s);
   q->BMt = upload_band<double>(ar, to_band(transposed(qt.BM), 0.0), s);
