@@ -94,7 +94,7 @@ inline void launch_kc(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, 
 // cval is null when the matrix is not of that form. Rows tlo <= i < thi of the centred copy are
 // identical (the Toeplitz interior of a matrix on a uniform knot vector); tlo = thi = 0 if none.
 template <typename T>
-struct BandD {
+struct BandCore {
   int rows, cols, width;
   const int* start;
   const T* val;
@@ -102,12 +102,18 @@ struct BandD {
   const T* cval;
   int half, cpitch;
   int tlo, thi;
-  // FP64: the band as limbs (k_fix_band.cu; null: none), centred with half width fhalf, or
-  // rectangular (fhalf = 0) with the first input of each 8-row segment in fw0
-  const int4* ftab;
-  const int* fex;
-  const int* fw0;
-  int fhalf;
+};
+// FP64: the band as limbs (k_fix_band.cu; tab null: none), centred with half width `half`, or
+// rectangular (half = 0) with the first input of each 8-row segment in w0.
+struct BandFix {
+  const int4* tab;
+  const int* ex;
+  const int* w0;
+  int half;
+};
+template <typename T>
+struct BandD : BandCore<T> {
+  BandFix fix;
 };
 
 // Extents of a 3D tensor, x1 fastest: index = i1 + n1 * (i2 + n2 * i3).
@@ -129,9 +135,9 @@ struct Dims {
 // Batches: nb items (nb <= 1: one), item k of every tensor of the job (X0, X1, Z, g, Y) at
 // offset k * bs elements from its pointer.
 template <typename T>
-struct PassArgs {
+struct PassCore {
   const T* X0; const T* X1;
-  BandD<T> D0, D1;
+  BandCore<T> D0, D1;
   T c0, c1;
   const T* Z; T cz;
   const T* g; int gaxis; Dims gdims;
@@ -144,8 +150,6 @@ struct PassArgs {
   int block;   // FP64 line kernel: threads per block (<= 0: 256); chosen by the setup tuner
   int c0_one;  // c0 == 1 (set by the launcher: the FP64 kernels test this integer instead of
                // comparing c0 per output, an instruction of the slow FP64 pipe)
-  BandD<T> D2;   // FP64 fixed-point passes: a second result Y2 = D2 .axis (the last term's input)
-  T* Y2;         // (null: none)
   int chain;   // two terms with c0 == c1 == 1 (set by the launcher): the FP64 kernels run one
                // FMA chain over both band rows
   // Horner epilogue (one hyper-power step fused into the pass that produces u = A~ t): instead
@@ -156,11 +160,19 @@ struct PassArgs {
   T* hacc;
   const T* hx;
 };
+// ... and what only the host and the fixed-point passes read (the kernels above take PassCore: the
+// size of a launch's arguments is part of its cost).
+template <typename T>
+struct PassArgs : PassCore<T> {
+  BandFix f0, f1;   // the limbs of D0 and D1
+  BandD<T> D2;      // FP64 fixed-point passes: a second result Y2 = D2 .axis (the last term's input)
+  T* Y2;            // (null: none)
+};
 
 // The Horner epilogue of PassArgs as one store: the same operations as writing Y and then
 // hp_first / hp_update (vector kernels), so the two routes give the same bits.
 template <typename T>
-__device__ __forceinline__ void pass_store(const PassArgs<T>& a, int64_t o, T v) {
+__device__ __forceinline__ void pass_store(const PassCore<T>& a, int64_t o, T v) {
   if (a.hmode == 0) {
     a.Y[o] = v;
   } else if (a.hmode == 1) {

@@ -23,7 +23,7 @@ inline int grid_for(int64_t total, int threads) {
 
 template <typename T>
 struct PassBatch {
-  PassArgs<T> job[kMaxPassJobs];
+  PassCore<T> job[kMaxPassJobs];
   int first_block[kMaxPassJobs + 1];
   int njobs;
   int seg;     // outputs per thread along the band direction
@@ -46,7 +46,7 @@ constexpr int seg_len() { return sizeof(T) == 4 ? 32 : 1; }
 // multiply besides the FMAs costs as much as an FMA (the pipe has the warps to hide the chain's
 // latency).
 template <int W, typename T, typename IT>
-__device__ __forceinline__ T band_dot(const BandD<T>& D, int i, const T* __restrict__ X, IT base,
+__device__ __forceinline__ T band_dot(const BandCore<T>& D, int i, const T* __restrict__ X, IT base,
                                       IT stride, T sum = T(0)) {
   const int s0 = __ldg(D.start + i);
   const T* x = X + (base + (IT)s0 * stride);
@@ -72,7 +72,7 @@ __device__ __forceinline__ T band_dot(const BandD<T>& D, int i, const T* __restr
 // division issues FP64-pipe instructions, the pipe these FP64 passes are bound by); int64_t
 // otherwise. Item offsets k * bs are always 64-bit.
 template <typename T, int W, typename IT>
-__device__ __forceinline__ void band_pass_flat_x1(const PassArgs<T>& a, IT t) {
+__device__ __forceinline__ void band_pass_flat_x1(const PassCore<T>& a, IT t) {
   const int m = a.D0.rows;
   const Dims out = a.in.with(1, m);
   const int nb = a.nb > 1 ? a.nb : 1;
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(512) k_band_pass(const __grid_constant__ PassB
   pdl_begin();
   int jb = 0;
   while (jb + 1 < pb.njobs && (int)blockIdx.x >= pb.first_block[jb + 1]) ++jb;
-  const PassArgs<T>& a = pb.job[jb];
+  const PassCore<T>& a = pb.job[jb];
   const int axis = a.axis;
   if constexpr (W > 0) {
     if (pb.flat1 && axis == 1) {
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(256) k_band_tile(const __grid_constant__ PassB
   extern __shared__ __align__(16) float sh[];
   int jb = 0;
   while (jb + 1 < pb.njobs && (int)blockIdx.x >= pb.first_block[jb + 1]) ++jb;
-  const PassArgs<float>& a = pb.job[jb];
+  const PassCore<float>& a = pb.job[jb];
   const int axis = a.axis;
   const int nin = a.in.get(axis);
   const int m = a.D0.rows;
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(256) k_band_tile(const __grid_constant__ PassB
   const int lane = tid % 32, warp = tid / 32, nwarps = blockDim.x / 32;
   // band coefficients and starts of this launch's operator(s)
   for (int t = 0; t < nt; ++t) {
-    const BandD<float>& D = t == 0 ? a.D0 : a.D1;
+    const BandCore<float>& D = t == 0 ? a.D0 : a.D1;
     const int width = t == 0 ? wt0 : wt1;
     for (int idx = tid; idx < m * wp; idx += blockDim.x) {
       const int i = idx / wp, w = idx - i * wp;
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(256, 4) k_band_slide(const __grid_constant__ P
   extern __shared__ __align__(16) float sh[];
   int jb = 0;
   while (jb + 1 < pb.njobs && (int)blockIdx.x >= pb.first_block[jb + 1]) ++jb;
-  const PassArgs<float>& a = pb.job[jb];
+  const PassCore<float>& a = pb.job[jb];
   const int axis = a.axis;
   const int m = a.D0.rows;   // square: output extent = input extent along the axis
   const int mr = slide_rows(m);
@@ -811,7 +811,7 @@ void band_tile_multi(const PassArgs<float>* jobs, int njobs, cudaStream_t s) {
     const PassArgs<float>& a = jobs[j];
     const int nt = a.nterms > 1 ? 2 : 1;
     for (int t = 0; t < nt; ++t) {
-      const BandD<float>& D = t == 0 ? a.D0 : a.D1;
+      const BandCore<float>& D = t == 0 ? a.D0 : a.D1;
       if (!D.cval || D.rows != D.cols || D.rows != a.in.get(a.axis) || 2 * D.half + 1 != Wc ||
           D.cpitch != ((Wc + 3) & ~3))
         Wc = 0;
@@ -936,6 +936,7 @@ void band_pass_multi(const PassArgs<T>* jobs, int njobs, cudaStream_t s) {
         a.nterms = 1;
         a.c0 = 1;
         a.D0 = jobs[j].D2;
+        a.f0 = jobs[j].D2.fix;
         a.Y = jobs[j].Y2;
         a.Y2 = nullptr;
       }

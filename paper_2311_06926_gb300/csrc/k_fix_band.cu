@@ -492,8 +492,8 @@ __global__ void __launch_bounds__(256, 2) k_fix_div_x1(const double* __restrict_
   }
 }
 
-FixBandOp band_op(const BandD<double>& D) {
-  return FixBandOp{D.ftab, D.fex, D.fw0, D.val, D.start, D.width};
+FixBandOp band_op(const BandCore<double>& D, const BandFix& f) {
+  return FixBandOp{f.tab, f.ex, f.w0, D.val, D.start, D.width};
 }
 
 void band_divisor(int n1, FixBandJob& J) {
@@ -542,7 +542,7 @@ void launch_fix_div(const double* u1, const double* u2, const double* u3, int a,
 }  // namespace
 
 bool fix_band_ok(const PassArgs<double>* jobs, int njobs) {
-  const int H = jobs[0].D0.fhalf;
+  const int H = jobs[0].f0.half;
   // (a launch with a g term or a Horner step has passes along x2 and x3 with one result only)
   bool epi = false;
   for (int j = 0; j < njobs; ++j) epi = epi || jobs[j].g || jobs[j].hmode;
@@ -552,9 +552,9 @@ bool fix_band_ok(const PassArgs<double>* jobs, int njobs) {
     // rectangular bands: single-term passes along x2 and x3 of one item
     if (H == 0 && (epi || a.axis == 1 || a.nterms > 1 || a.nb > 1)) return false;
     const int m = H ? a.in.get(a.axis) : a.D0.rows, nb = a.nb > 1 ? a.nb : 1;
-    if (!a.D0.ftab || a.D0.fhalf != H || a.D0.rows != m || a.Z ||
-        (a.nterms > 1 && (!a.D1.ftab || a.D1.fhalf != H || a.D1.rows != m || a.c1 != 1.0)) ||
-        (a.Y2 && (!a.D2.ftab || a.D2.fhalf != H || a.D2.rows != m)) ||
+    if (!a.f0.tab || a.f0.half != H || a.D0.rows != m || a.Z ||
+        (a.nterms > 1 && (!a.f1.tab || a.f1.half != H || a.D1.rows != m || a.c1 != 1.0)) ||
+        (a.Y2 && (!a.D2.fix.tab || a.D2.fix.half != H || a.D2.rows != m)) ||
         a.c0 != 1.0 ||
         (a.axis == 1 && (a.g || a.hmode || (a.nterms > 1 && !a.Y2) || (m + kR - 1) / kR > 256)) ||
         (a.Y2 && (a.g || a.hmode)) ||
@@ -568,7 +568,7 @@ bool fix_band_ok(const PassArgs<double>* jobs, int njobs) {
 void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
   FixBandBatch fb{};
   fb.njobs = njobs;
-  const int H = jobs[0].D0.fhalf;
+  const int H = jobs[0].f0.half;
   int threads = 32;
   for (int j = 0; j < njobs; ++j)
     threads = std::max(threads, band_threads(jobs[j].block, jobs[j].axis == 1
@@ -583,9 +583,9 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
     FixBandJob& J = fb.job[j];
     J.X[0] = a.X0;
     J.X[1] = a.X1;
-    J.D[0] = band_op(a.D0);
-    if (a.nterms > 1) J.D[1] = band_op(a.D1);
-    if (a.Y2) J.D[a.nterms] = band_op(a.D2);
+    J.D[0] = band_op(a.D0, a.f0);
+    if (a.nterms > 1) J.D[1] = band_op(a.D1, a.f1);
+    if (a.Y2) J.D[a.nterms] = band_op(a.D2, a.D2.fix);
     epi = epi || a.g || a.hmode;
     nt = std::max(nt, a.nterms);
     J.Y = a.Y;
@@ -641,14 +641,14 @@ void fix_div_band_x1(const double* u1, const double* u2, const double* u3, int a
                      const double* q, double nu, const BandD<double>& D, double* y0, double* y1,
                      int block, cudaStream_t s) {
   FixBandJob J{};
-  J.D[0] = band_op(D);
+  J.D[0] = band_op(D, D.fix);
   J.Y = y0;
   J.nterms = J.nops = 1;
   J.nb = 1;
   band_divisor(b, J);
   J.segs = (b + kR - 1) / kR;
   const int nv = q ? 2 : 1;
-  const int H = D.fhalf, threads = band_threads(block, J.segs * nv);
+  const int H = D.fix.half, threads = band_threads(block, J.segs * nv);
   const int lpb = threads / (J.segs * nv), blocks = (b * b + lpb - 1) / lpb;
   const int smem = band_along_smem(1, 2 * nv * lpb, J.segs, H);
   const double np = (double)b * b * b;

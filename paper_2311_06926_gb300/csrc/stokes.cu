@@ -131,10 +131,7 @@ BandD<T> upload_band(Arena& ar, const Band& b, cudaStream_t s, int min_half = 0)
   d.half = 0;
   d.cpitch = 0;
   d.tlo = d.thi = 0;
-  d.ftab = nullptr;
-  d.fex = nullptr;
-  d.fw0 = nullptr;
-  d.fhalf = 0;
+  d.fix = BandFix{};
   // centred copy for square matrices (every matrix of the operator applies is one)
   std::vector<T> cv;
   if (b.rows == b.cols) {
@@ -214,9 +211,7 @@ void upload_fix_band(Arena& ar, const Band& b, BandD<double>& d, int H, cudaStre
   ck(cudaMemcpyAsync(td, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
   ck(cudaMemcpyAsync(ed, ex.data(), ex.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
   ck(cudaStreamSynchronize(s), "fix");
-  d.ftab = reinterpret_cast<const int4*>(td);
-  d.fex = ed;
-  d.fhalf = H;
+  d.fix = BandFix{reinterpret_cast<const int4*>(td), ed, nullptr, H};
 }
 
 // The same for a rectangular band whose 8-row segments read at most 8 inputs each (none otherwise):
@@ -251,10 +246,7 @@ void upload_fix_rect(Arena& ar, const Band& b, BandD<double>& d, cudaStream_t s)
   ck(cudaMemcpyAsync(td, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
   ck(cudaMemcpyAsync(ed, ex.data(), ex.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
   ck(cudaStreamSynchronize(s), "fix");
-  d.ftab = reinterpret_cast<const int4*>(td);
-  d.fex = ed;
-  d.fw0 = ed + segs;
-  d.fhalf = 0;
+  d.fix = BandFix{reinterpret_cast<const int4*>(td), ed, ed + segs, 0};
 }
 
 template <typename T>
@@ -413,6 +405,8 @@ struct Ops {
     p.c0 = c0;
     p.X1 = X1;
     p.D1 = D1 ? *D1 : D0;
+    p.f0 = D0.fix;
+    p.f1 = D1 ? D1->fix : D0.fix;
     p.c1 = c1;
     p.nterms = X1 ? 2 : 1;
     p.Z = Z;
@@ -900,6 +894,8 @@ struct QuadOps {
     p.c0 = c0;
     p.X1 = X1;
     p.D1 = D1 ? *D1 : D0;
+    p.f0 = D0.fix;
+    p.f1 = D1 ? D1->fix : D0.fix;
     p.c1 = c1;
     p.nterms = X1 ? 2 : 1;
     p.Z = Z;
