@@ -20,6 +20,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <climits>
 #include <cstdint>
 #include <cstring>
 
@@ -453,25 +454,79 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
 }
 
-template <typename TO>
+constexpr int kPadUnroll = 5;   // entries per lane in flight: rows of up to 160 in one step
+
+struct PadBatch {
+  PadJob job[kMaxPadJobs];
+  int64_t first[kMaxPadJobs + 1];   // first row of each job (items in order within a job)
+  int njobs, nb;
+  int64_t bs;
+};
+
 // One warp per row (rows of all items in order), lanes along the row: coalesced loads and stores,
-// one division per row instead of one per element.
-__global__ void k_pad_rows(const float* __restrict__ x, int e1, int64_t R, int ld,
-                           TO* __restrict__ y, int nb, int64_t xbs) {
+// one division per row instead of one per element, all loads of a step before its stores. Bound by
+// the memory passes over tensors that mostly sit in L2, so what counts is passes and launches: MODE
+// 1 and 2 take the Horner step into the copy that would otherwise read its result back, the last
+// step of a recursion stores the copy only, and the components share one launch. One order-3 step
+// at 128^3 p = 3 in TF32: vector launches 297 -> 178 us (both branches, one after the other), the
+// preconditioner 1078 -> 1023 us; order 4 at 48^3 p = 4, six vectors, BF16: 1395 -> 1330 us. (With
+// loads and stores interleaved and the grid bounded by 4864 blocks, most warps with one row and some
+// with two, the first gained nothing.)
+template <typename TO, int MODE>
+__global__ void __launch_bounds__(256) k_pad_rows(const __grid_constant__ PadBatch b) {
   pdl_trigger();   // the mode product that reads this copy sets up while the copy runs
   pdl_begin();
-  const int64_t rows = R * nb;
   const int lane = threadIdx.x % 32;
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
   const int64_t nw = (int64_t)gridDim.x * blockDim.x / 32;
-  for (int64_t r = w0; r < rows; r += nw) {
-    const int64_t k = nb > 1 ? r / R : 0;     // item
-    const float* src = x + k * xbs + (r - k * R) * e1;
-    TO* dst = y + r * ld;
-    for (int j = lane; j < e1; j += 32) {
-      // the FP32 copy feeds TF32 products: rounded to TF32 here (BF16 rounds in store_val)
-      if constexpr (sizeof(TO) == 4) store_val<TO>(dst + j, round_tf32(src[j]));
-      else store_val<TO>(dst + j, src[j]);
+  for (int64_t w = w0; w < b.first[b.njobs]; w += nw) {
+    int jb = 0;
+    while (jb + 1 < b.njobs && w >= b.first[jb + 1]) ++jb;
+    const PadJob& J = b.job[jb];
+    const int64_t row = w - b.first[jb], R = J.R;
+    int64_t k = 0;   // item
+    if (b.nb > 1)
+      k = (row | R) >> 32 ? row / R : (int64_t)((uint32_t)row / (uint32_t)R);
+    const int e1 = J.e1;
+    const int64_t o = k * b.bs + (row - k * R) * e1;
+    TO* __restrict__ dst = static_cast<TO*>(J.y) + row * J.ld;
+    // the FP32 copy feeds TF32 products: rounded to TF32 here (BF16 rounds in store_val)
+    auto put = [&](int j, float v) {
+      if constexpr (sizeof(TO) == 4) store_val<TO>(dst + j, round_tf32(v));
+      else store_val<TO>(dst + j, v);
+    };
+    const float* x = J.x + o;
+    const float* u = J.u + o;
+    float* acc = J.acc + o;
+    float* r = J.r + o;
+    for (int j0 = lane; j0 < e1; j0 += 32 * kPadUnroll) {
+      // all loads of up to kPadUnroll entries per lane before the first store
+      float xv[kPadUnroll], uv[kPadUnroll], av[kPadUnroll];
+#pragma unroll
+      for (int i = 0; i < kPadUnroll; ++i) {
+        const int j = j0 + 32 * i;
+        if (j >= e1) continue;
+        xv[i] = MODE == 2 ? r[j] : x[j];
+        if (MODE != 0) uv[i] = u[j];
+        if (MODE == 2) av[i] = acc[j];
+      }
+#pragma unroll
+      for (int i = 0; i < kPadUnroll; ++i) {
+        const int j = j0 + 32 * i;
+        if (j >= e1) continue;
+        if (MODE == 0) {
+          put(j, xv[i]);
+          continue;
+        }
+        // k_hp_first, k_hp_update: the same operations
+        const float rj = xv[i] - uv[i];
+        const float aj = (MODE == 1 ? xv[i] : av[i]) + rj;
+        if (!J.last) {
+          r[j] = rj;
+          acc[j] = aj;
+        }
+        put(j, J.last ? aj : rj);
+      }
     }
   }
 }
@@ -604,20 +659,34 @@ void launch_rmp(const RmpPlan& p, int* err, int sms, cudaStream_t s, uint32_t sp
   launch_rmp_multi(&one, 1, err, sms, s, spin_limit, nsplit);
 }
 
-void pad_rows(const float* x, int e1, int64_t R, int ld, void* y, bool to_bf16, cudaStream_t s,
-              int nb, int64_t xbs) {
-  if (nb < 1) nb = 1;
-  const int64_t total = (int64_t)e1 * R * nb;
-  int64_t blocks = (R * nb + 7) / 8;   // 8 warps (rows) per block
-  if (blocks > 152 * 32) blocks = 152 * 32;
+void pad_rows(const PadJob* jobs, int njobs, int mode, bool to_bf16, cudaStream_t s, int nb,
+              int64_t bs) {
+  PadBatch b{};
+  b.njobs = njobs;
+  b.nb = nb > 1 ? nb : 1;
+  b.bs = bs;
+  double total = 0;
+  for (int j = 0; j < njobs; ++j) {
+    b.job[j] = jobs[j];
+    b.first[j + 1] = b.first[j] + jobs[j].R * b.nb;
+    total += (double)jobs[j].R * b.nb * jobs[j].e1;
+  }
+  int64_t blocks = (b.first[njobs] + 7) / 8;   // 8 warps (rows) per block
+  if (blocks > INT_MAX) blocks = INT_MAX;
+  const int out = to_bf16 ? 2 : 4;
+  const double per = mode == 0 ? 4 : (mode == 1 ? 8 : 12) + (jobs[0].last ? 0 : 8);
   launch_begin(kClassVector, s);
-  if (to_bf16)
-    launch_k(k_pad_rows<__nv_bfloat16>, (int)blocks, 256, 0, s, x, e1, R, ld,
-             static_cast<__nv_bfloat16*>(y), nb, xbs);
-  else
-    launch_k(k_pad_rows<float>, (int)blocks, 256, 0, s, x, e1, R, ld, static_cast<float*>(y), nb,
-             xbs);
-  launch_end(kClassVector, s, 0.0, (double)total * (to_bf16 ? 6.0 : 8.0));
+  auto go = [&](auto kernel) { launch_k(kernel, (int)blocks, 256, 0, s, b); };
+  if (to_bf16) {
+    if (mode == 0) go(k_pad_rows<__nv_bfloat16, 0>);
+    else if (mode == 1) go(k_pad_rows<__nv_bfloat16, 1>);
+    else go(k_pad_rows<__nv_bfloat16, 2>);
+  } else {
+    if (mode == 0) go(k_pad_rows<float, 0>);
+    else if (mode == 1) go(k_pad_rows<float, 1>);
+    else go(k_pad_rows<float, 2>);
+  }
+  launch_end(kClassVector, s, mode == 0 ? 0.0 : 2.0 * total, total * (per + out));
 }
 
 }  // namespace shp

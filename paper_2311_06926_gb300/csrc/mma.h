@@ -55,10 +55,24 @@ void launch_rmp(const RmpPlan& p, int* err, int sms, cudaStream_t s, uint32_t sp
 void launch_rmp_multi(const RmpPlan* const* plans, int njobs, int* err, int sms, cudaStream_t s,
                       uint32_t spin_limit = 0, int nsplit = 1);
 
-// Copy a canonical float tensor (rows of e1 entries, R rows) into rows of pitch ld, converting
-// to bfloat16 if to_bf16. nb items: item k's tensor starts xbs elements after item k - 1's in x,
-// its rows follow item k - 1's in y.
-void pad_rows(const float* x, int e1, int64_t R, int ld, void* y, bool to_bf16, cudaStream_t s,
-              int nb = 1, int64_t xbs = 0);
+// Staging copy of a canonical float tensor (rows of e1 entries, R rows) into rows of pitch ld, as
+// the tensor-core products read them (rounded to TF32, or converted to bfloat16). nb items: item k's
+// tensors start bs elements after item k - 1's (y: its rows follow item k - 1's).
+// mode 0: the copy of x. mode 1, 2: a hyper-power Horner step first (hp_first: r = x - u,
+// acc = x + r; hp_update: r = r - u, acc = acc + r), then the copy of what the next fast
+// diagonalisation takes: of r, or of acc if it is the recursion's last step; the last step stores
+// neither r nor acc, which nothing reads again. Up to kMaxPadJobs tensors per launch.
+constexpr int kMaxPadJobs = 3;
+struct PadJob {
+  const float* x;
+  int e1, ld;
+  int64_t R;
+  void* y;
+  const float* u;   // mode 1, 2
+  float *r, *acc;
+  int last;
+};
+void pad_rows(const PadJob* jobs, int njobs, int mode, bool to_bf16, cudaStream_t s, int nb = 1,
+              int64_t bs = 0);
 
 }  // namespace shp

@@ -340,12 +340,15 @@ FixTabs upload_fix_plain(Arena& ar, const Dense& D, cudaStream_t s) {
 // One hyper-power Horner step applied by the pass that produces A~ t (see PassArgs): mode 1 sets
 // r = x - A~ t, acc = x + r; mode 2 sets r = r - A~ t, acc = acc + r. r, acc, x have the layout of
 // the product.
+// stage: the step also writes the tensor-core input copy of what the next fast diagonalisation
+// takes (stages()): of r, or, `last`, of acc, and then r and acc are not stored.
 template <typename T>
 struct Horner {
   int mode;
   T* r;
   T* acc;
   const T* x;
+  bool stage = false, last = false;
 };
 
 // ---- operators in precision T ------------------------------------------------------------------
@@ -603,7 +606,30 @@ struct Ops {
   }
 
   // y = A x; with h, the Horner step of h is applied to A x instead (y is scratch then)
+  // the next fast diagonalisation after a Horner step whose result is one reads a staging copy
+  bool stages() const { return std::is_same<T, float>::value && tc; }
+
+  // one Horner step with the product A~ t in u, with the staging copy (tensors t0 .. t0 + nt - 1)
+  void stage_horner(const T* u, const Horner<T>& h, int t0, int nt) const {
+    if constexpr (std::is_same<T, float>::value) {
+      PadJob j[3];
+      for (int c = 0; c < nt; ++c) {
+        j[c] = pad_job(t0 + c, h.x + c * nvc);
+        j[c].u = u + c * nvc;
+        j[c].r = h.r + c * nvc;
+        j[c].acc = h.acc + c * nvc;
+        j[c].last = h.last;
+      }
+      pad_rows(j, nt, h.mode, tc_bf16, s, nb, bs);
+    }
+  }
+
   void apply_A(const T* x, T* y, const Horner<T>* h = nullptr) const {
+    if (h && h->stage) {
+      apply_A(x, y);
+      stage_horner(y, *h, 0, 3);
+      return;
+    }
     if constexpr (std::is_same<T, double>::value) {
       if (fused_div()) {
         div_x1(x, nullptr, f1, nullptr);
@@ -651,6 +677,11 @@ struct Ops {
 
   // B^T u = M_q D_div u; with h, the Horner step of h is applied to it instead
   void apply_Bt(const T* u, T* yq, const Horner<T>* h = nullptr) const {
+    if (h && h->stage) {
+      apply_Bt(u, yq);
+      stage_horner(yq, *h, 3, 1);
+      return;
+    }
     T* out[1] = {yq};
     const T coef[1] = {1};
     if constexpr (std::is_same<T, double>::value) {
@@ -695,9 +726,23 @@ struct Ops {
   // The pressure tensor (t = 3) takes three passes with the dense inverse of M-check instead:
   // (M-check^-1)^(x)3 is a Kronecker product of one dense matrix, so one rotation of the three
   // directions applies it (the eigenvector route U_T U_T^T needs six).
-  void tc_fd(int t, const float* x, float* y) const {
+  PadJob pad_job(int t, const float* x) const {
     const Dims d = t < 3 ? comp(t) : Dims{b, b, b};
-    pad_rows(x, d.n1, (int64_t)d.n2 * d.n3, tc_ld0[t], tc_p0[t], tc_bf16, s, nb, bs);
+    PadJob j{};
+    j.x = x;
+    j.e1 = d.n1;
+    j.R = (int64_t)d.n2 * d.n3;
+    j.ld = tc_ld0[t];
+    j.y = tc_p0[t];
+    return j;
+  }
+
+  // staged: the Horner step before has written x's staging copy (x is not read)
+  void tc_fd(int t, const float* x, float* y, bool staged) const {
+    if (!staged) {
+      const PadJob j = pad_job(t, x);
+      pad_rows(&j, 1, 0, tc_bf16, s, nb, bs);
+    }
     const int passes = t < 3 ? 6 : 3;
     for (int st = 0; st < passes; ++st) {
       RmpPlan p = tc_plan[t * 6 + st];
@@ -715,13 +760,14 @@ struct Ops {
            fd_plane_smem(Dims{b, a, b}) > 0 && fd_plane_smem(Dims{b, b, b}) > 0;
   }
 
-  void fd_V(const T* x, T* y) const {
+  void fd_V(const T* x, T* y, bool staged = false) const {
     if (tc) {
-      // the three components share each of the six tensor-core launches
-      for (int c = 0; c < 3; ++c) {
-        const Dims d = comp(c);
-        pad_rows(reinterpret_cast<const float*>(x + c * nvc), d.n1, (int64_t)d.n2 * d.n3,
-                 tc_ld0[c], tc_p0[c], tc_bf16, s, nb, bs);
+      // the three components share the staging copy and each of the six tensor-core launches
+      if (!staged) {
+        PadJob j[3];
+        for (int c = 0; c < 3; ++c)
+          j[c] = pad_job(c, reinterpret_cast<const float*>(x + c * nvc));
+        pad_rows(j, 3, 0, tc_bf16, s, nb, bs);
       }
       for (int st = 0; st < 6; ++st) {
         RmpPlan p[3];
@@ -807,7 +853,7 @@ struct Ops {
   }
 
   // pressure block: y = 2 nu (M-check^-1)^(x)3 x = 2 nu (U_T U_T^T)^(x)3 x
-  void minv_Q(const T* x, T* y) const {
+  void minv_Q(const T* x, T* y, bool staged = false) const {
     // FP64, long lines: three passes with the dense M-check^-1 (not folded: the rounding of M-check's
     // entries is not symmetric, and averaging the mirrored entries of its inverse would move it by
     // 1e-14); below, the eigenvector route (its fused form takes as few launches).
@@ -828,7 +874,7 @@ struct Ops {
       }
     }
     if (tc) {
-      tc_fd(3, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y));
+      tc_fd(3, reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), staged);
       return;
     }
     const Dims d{b, b, b};
@@ -1012,21 +1058,22 @@ struct HyperPower {
   T *bv = nullptr, *hv = nullptr;     // velocity buffers of the Schur approximation
   int64_t counts[4] = {0, 0, 0, 0};   // fd_V, minv_Q, A, (B + B^T)
 
-  void V(const Ops<T>& o, const VLevels& L, int s, const T* x, T* y) {
+  void V(const Ops<T>& o, const VLevels& L, int s, const T* x, T* y, bool staged = false) {
     if (s == 0) {
-      o.fd_V(x, y);
+      o.fd_V(x, y, staged);
       ++counts[0];
       return;
     }
     T *r = L.r[s], *acc = L.acc[s], *t = L.t[s], *u = L.u[s];
     // Horner steps from r = acc = x; the first reads x directly
+    const bool stage = s == 1 && o.stages();
     for (int j = 1; j < order; ++j) {
-      V(o, L, s - 1, j == 1 ? x : r, t);
-      const Horner<T> h{j == 1 ? 1 : 2, r, acc, x};
+      V(o, L, s - 1, j == 1 ? x : r, t, stage && j > 1);
+      const Horner<T> h{j == 1 ? 1 : 2, r, acc, x, stage, j == order - 1};
       o.apply_A(t, u, &h);   // the step r, acc <- (r - A~ t, acc + r) in the last pass
       ++counts[2];
     }
-    V(o, L, s - 1, acc, y);
+    V(o, L, s - 1, acc, y, stage);
   }
 
   int level_of(int m) const {
@@ -1034,24 +1081,25 @@ struct HyperPower {
     return m == 1 ? 0 : m;
   }
 
-  void Q(const Ops<T>& o, const VLevels& L, int m, const T* x, T* y) {
+  void Q(const Ops<T>& o, const VLevels& L, int m, const T* x, T* y, bool staged = false) {
     if (m == 0) {
-      o.minv_Q(x, y);
+      o.minv_Q(x, y, staged);
       ++counts[1];
       return;
     }
     T *r = qr[m], *acc = qacc[m], *t = qt[m], *u = qu[m];
     const int l = level_of(m);
     // Horner steps from r = acc = x; the first reads x directly
+    const bool stage = m == 1 && o.stages();
     for (int j = 1; j < order; ++j) {
-      Q(o, L, m - 1, j == 1 ? x : r, t);
+      Q(o, L, m - 1, j == 1 ? x : r, t, stage && j > 1);
       o.apply_B(t, bv);          // A~_Q t = B^T P_{V,l}^-1 B t
       V(o, L, l, bv, hv);
-      const Horner<T> h{j == 1 ? 1 : 2, r, acc, x};
+      const Horner<T> h{j == 1 ? 1 : 2, r, acc, x, stage, j == order - 1};
       o.apply_Bt(hv, u, &h);   // the step r, acc <- (r - A~_Q t, acc + r) in the last pass
       ++counts[3];
     }
-    Q(o, L, m - 1, acc, y);
+    Q(o, L, m - 1, acc, y, stage);
   }
 
   void apply(int steps, const T* x, T* y) {
