@@ -205,8 +205,12 @@ constexpr int kFixBandHalf = 6;   // largest half width of the limb tables
 // and the FMA kernels take less time (K apply at 32^3 p = 3: 32 against 35 us; at 64^3: 150 against
 // 83)
 constexpr int kFixBandMin = 40;
-// smallest number of points per direction of the fixed-point quadrature passes
-constexpr int kFixRectMin = 64;
+// smallest number of points per direction of the fixed-point quadrature passes. K apply in us, chains
+// against fixed point: p = 1 39 points 141 / 141, 48 155 / 149, 63 202 / 178, 96 388 / 308; p = 2
+// 40 points 179 / 179, 48 198 / 193, 64 239 / 210; p = 3 40 points 222 / 217, 60 266 / 243, 95
+// 510 / 401; p = 4 36 points 260 / 261, 48 288 / 276, 96 557 / 429; below 40 the chains' launches
+// are the shorter ones (p = 1 24 points 123 / 128, p = 3 20 points 195 / 199).
+constexpr int kFixRectMin = 48;
 
 // delta = sum_c D .c u_c: exact discrete divergence of the velocity coefficients (App. B.2),
 // output b^3. (D beta)_i = beta_i - beta_{i-1} with beta_{-1} = beta_a = 0.

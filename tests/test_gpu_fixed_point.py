@@ -115,3 +115,22 @@ def test_operator_windows_outside_the_scaled_range():
         assert u1[far].all()
         assert relerr(z[:a * b * b].reshape(b, b, a)[far], y[:a * b * b].reshape(b, b, a)[far]) < 1e-13
     G.close()
+
+
+# points per direction below, at and above 48 (where the fixed-point passes begin; p + 2 points per
+# element), windows of 8 that hold p = 1..6, and the last segment of 8 rows ragged and whole
+@pytest.mark.parametrize("n,p,nu", [(15, 1, 1.0), (16, 1, 0.6), (21, 1, 1.0), (11, 2, 1.0),
+                                    (12, 2, 2.0), (10, 3, 1.0), (13, 3, 1.0), (8, 4, 0.5),
+                                    (7, 5, 1.0), (10, 5, 1.0), (6, 6, 1.0), (9, 6, 1.0)])
+def test_quadrature_segment_edges(n, p, nu):
+    """Bound: that of test_quadrature_operator_equals_kronecker_and_oracle."""
+    S, _, Kop, F = oracle(n, p, nu)
+    x = synthetic.random_vector(S.size, 80 + n + p)
+    ref = Kop(x)
+    G = Stokes(n, p, nu=nu, max_order=2, max_steps=0, autotune=False, forward="quadrature")
+    for block in (128, 256, 512):
+        G.set_tuning(512, block, 0)
+        assert relerr(host(G.apply_K(dev(x))), ref) < 1e-12
+    for e in (-900, 800):   # windows that cannot be scaled take chains
+        assert relerr(np.ldexp(host(G.apply_K(dev(x) * 2.0 ** e)), -e), ref) < 1e-12
+    G.close()
