@@ -385,7 +385,7 @@ bool generalized_eigh_parity(const Dense& K, const Dense& M, std::vector<double>
   return true;
 }
 
-bool banded_inverse(const Dense& A, int p, Dense& inv) {
+bool banded_inverse(const Dense& A, int p, Dense& inv, Dense& low) {
   const int n = A.rows, w = p + 1;
   // L(i, k) at lb[i * w + (k - i + p)] for i - p <= k <= i
   std::vector<double> lb((size_t)n * w, 0.0);
@@ -414,6 +414,7 @@ bool banded_inverse(const Dense& A, int p, Dense& inv) {
     }
   };
   inv = Dense(n, n);
+  low = Dense(n, n);
   std::vector<double> x(n), r(n);
   for (int c = 0; c < n; ++c) {
     std::fill(x.begin(), x.end(), 0.0);
@@ -430,7 +431,10 @@ bool banded_inverse(const Dense& A, int p, Dense& inv) {
       r[i] = hi + lo;
     }
     solve(r);
-    for (int i = 0; i < n; ++i) inv(i, c) = x[i] + r[i];
+    for (int i = 0; i < n; ++i) {
+      inv(i, c) = x[i] + r[i];
+      low(i, c) = r[i] - (inv(i, c) - x[i]);
+    }
   }
   return true;
 }

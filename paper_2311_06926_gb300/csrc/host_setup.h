@@ -62,9 +62,9 @@ bool generalized_eigh_parity(const Dense& K, const Dense& M, std::vector<double>
                              int* he);
 
 // Inverse of a symmetric positive definite matrix of half bandwidth p by banded Cholesky, each
-// column refined once with a residual in twice the working precision (entries correct to about an
-// ulp of the column). Returns false if A is not positive definite.
-bool banded_inverse(const Dense& A, int p, Dense& inv);
+// column refined once with a residual in twice the working precision: inv + low, low the part
+// of the refined entries that doubles lose. Returns false if A is not positive definite.
+bool banded_inverse(const Dense& A, int p, Dense& inv, Dense& low);
 
 Band to_band(const Dense& D, double drop_tol);
 

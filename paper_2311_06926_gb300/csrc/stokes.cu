@@ -272,8 +272,10 @@ uint16_t half_bits(int v) {
 // 1 odd; zero where the half has no such entry). Output i is scaled so that its integers stay
 // below 2^kFixUBits and the sum of their magnitudes below 2^kFixSumBits (fix.h); share: one
 // scale for both halves of an output.
-template <typename F>
-FixTab upload_fix_side(Arena& ar, int he, int halves, bool share, F&& u, cudaStream_t s) {
+// lo(k, i, par): what u lacks of an entry known to more than a double (the integers have up to 5
+// bits more).
+template <typename F, typename G>
+FixTab upload_fix_side(Arena& ar, int he, int halves, bool share, F&& u, cudaStream_t s, G&& lo) {
   FixTab t;
   t.nt = (he + 7) / 8;
   t.ks = (he + 15) / 16;
@@ -296,6 +298,7 @@ FixTab upload_fix_side(Arena& ar, int he, int halves, bool share, F&& u, cudaStr
       ex[(size_t)par * 8 * t.nt + i] = e[par];
       for (int k = 0; k < he; ++k) {
         long long v = std::llrint(std::ldexp(u(k, i, par), -e[par]));
+        v += std::llrint(std::ldexp(lo(k, i, par), -e[par]));
         // operand position: column i % 8, row k % 16 of step k / 16
         const int kk = k % 16, lane = (i % 8) * 4 + (kk % 8) / 2, reg = kk / 8;
         for (int d = kFixSlices - 1; d >= 0; --d) {
@@ -321,19 +324,21 @@ FixTab upload_fix_side(Arena& ar, int he, int halves, bool share, F&& u, cudaStr
 FixTabs upload_fix(Arena& ar, const Dense& U, int he, cudaStream_t s) {
   const int h = U.rows - he;
   FixTabs f;
+  const auto none = [](int, int, int) { return 0.0; };
   f.fw = upload_fix_side(ar, he, 2, false, [&](int k, int i, int par) {
     return par == 0 ? U(k, i) : (k < h && i < h ? U(k, he + i) : 0.0);
-  }, s);
+  }, s, none);
   f.bw = upload_fix_side(ar, he, 2, true, [&](int k, int i, int par) {
     return par == 0 ? U(i, k) : (k < h && i < h ? U(i, he + k) : 0.0);
-  }, s);
+  }, s, none);
   return f;
 }
 
-// y = D x
-FixTabs upload_fix_plain(Arena& ar, const Dense& D, cudaStream_t s) {
+// y = (D + low) x
+FixTabs upload_fix_plain(Arena& ar, const Dense& D, const Dense& low, cudaStream_t s) {
   FixTabs f;
-  f.fw = upload_fix_side(ar, D.rows, 1, false, [&](int k, int i, int) { return D(i, k); }, s);
+  f.fw = upload_fix_side(ar, D.rows, 1, false, [&](int k, int i, int) { return D(i, k); }, s,
+                         [&](int k, int i, int) { return low(i, k); });
   return f;
 }
 
@@ -2564,12 +2569,12 @@ int stokes_setup(stokes_t* out, int n_elems, int degree_p, double nu, const stok
       c->od.invd = upload<double>(c->arena, inv, c->stream);
     }
     {
-      Dense Minv;
-      if (!banded_inverse(u.Mc, degree_p, Minv))
+      Dense Minv, low;
+      if (!banded_inverse(u.Mc, degree_p, Minv, low))
         throw SetupError{"pressure mass matrix is not positive definite"};
       if (!reduced(c) && heT > kFixMinHalf) {
         c->od.Minv = upload<double>(c->arena, Minv.v, c->stream);
-        c->od.fx_Minv = upload_fix_plain(c->arena, Minv, c->stream);
+        c->od.fx_Minv = upload_fix_plain(c->arena, Minv, low, c->stream);
       }
     }
     const Ops<double>* odq = nullptr;
