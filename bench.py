@@ -48,29 +48,38 @@ TF32_NOMINAL_TFLOPS = 1100.0
 # reports it only while that source is unchanged, and null otherwise.
 TRAFFIC = {
     ("mode_product", "fp64", "cavity32", "per-direction"): {
-        "bytes_per_launch": 1035634,
-        "source": "k_dense.cu",
-        "sha256": "d05c14c82b258149fb7e1b53760b0abff0cde9339623d5309a23fb8b03d0c98f",
-        "profile": "profiles/k_mode_tile_fp64_cavity32.md"},
+        "bytes_per_launch": 1266325,
+        "source": "k_fix.cu",
+        "sha256": "89ca42cd053c857e0ce54d368c49285e642c654ab2e426fd89532b594a2f1be4",
+        "profile": "profiles/k_fix_fp64_cavity128.md"},
     ("band_pass_fp64", "tf32", "cavity128", "per-direction"): {
-        "bytes_per_launch": 202983358,
-        "source": "k_band.cu",
-        "sha256": "e78575f2233db7e235a87cf1ac012c93873e1e8aa42a741bf11a5eac6349d39a",
-        "profile": "profiles/k_band_pass_fp64_cavity128.md"},
-    ("mode_product", "fp64", "cavity32", "fused, 4 block(s) per plane"): {
-        "bytes_per_launch": 1029889,
-        "source": "k_dense.cu",
-        "sha256": "61e438359185f0bf02457abbb4b35a9d25bc8bf38ee72e6c89be7a2bce8c995e",
-        "profile": "profiles/k_fd_plane_fp64_cavity32.md"},
+        "bytes_per_launch": 174363008,
+        "source": "k_fix_band.cu",
+        "sha256": "d39e4349692b4215d123d17a4d6c86aa616cff917da1b7cdc6cf921be3e496cd",
+        "profile": "profiles/k_fix_fp64_cavity128.md"},
 }
 
 
 KERNEL_NAMES = {
     "mma_mode_product": "k_rmp (tcgen05 mode products of the fast diagonalisation)",
     "band_pass": "k_band_slide / k_band_tile (FP32 banded passes)",
-    "band_pass_fp64": "k_band_pass<double> (FP64 banded passes of the outer K apply)",
+    "band_pass_fp64": "k_fix_band (FP64 banded passes of the outer K apply)",
     "vector": "Krylov vector kernels (Gram-Schmidt sweeps, conversions, padded copies)",
 }
+
+
+def fixed_point_classes(n, p):
+    """FP64 kernel classes that a mesh runs in fixed point (integer multipliers, FP16 tensor
+    cores): their rate is not bounded by the FP64 pipe and is reported against HBM. The library's
+    rules: banded passes from 40 pressure entries per direction and p <= 5 (from 48 points for
+    the quadrature tables), mode products from half lengths above 12."""
+    b = n + p
+    out = set()
+    if b >= 40 and p <= 5:
+        out.add("band_pass_fp64")
+    if (b + 1) // 2 > 12:
+        out.update(("mode_product", "line_solve"))
+    return out
 
 
 def fd_form(fd_fused):
@@ -517,10 +526,10 @@ def schur_variants(Stokes, n=32, p=3):
     return out
 
 
-def class_rooflines(prof, step_ms, prec, peaks):
+def class_rooflines(prof, step_ms, prec, peaks, fixed=()):
     """Per kernel class of one profiled step: launches, time, share, and the achieved rate of its
     algorithmic work against the bound of that class (FP64 pipe for FP64 band passes and mode
-    products, HBM for the rest). Times include the per-launch events of the profiled pass."""
+    products formed in FP64, HBM for the rest and for the classes in `fixed`). Times include the per-launch events of the profiled pass."""
     hbm = peaks.get("hbm_gbs", 6800.0)
     out = {}
     for k, v in prof.items():
@@ -528,7 +537,8 @@ def class_rooflines(prof, step_ms, prec, peaks):
              "share": round(v["ms"] / step_ms, 4) if step_ms > 0 else 0.0}
         if v["launches"] and v["ms"] > 0:
             sec = v["ms"] / 1e3
-            if k == "band_pass_fp64" or (prec == "fp64" and k in ("band_pass", "mode_product")):
+            if k not in fixed and (k == "band_pass_fp64" or (
+                    prec == "fp64" and k in ("band_pass", "mode_product"))):
                 tf = v["flops"] / sec / 1e12
                 e.update(bound="fp64", achieved_tflops=round(tf, 4),
                          frac=round(tf / FP64_PEAK_TFLOPS, 4))
@@ -838,7 +848,7 @@ def run_cavity128(args, wl):
               "share_of_solve": dom["ms"] / step_ms_profiled,
               "measurement": "CUDA events around every launch of one profiled solve "
                              "(algorithmic work: each input read once, each output written once)"}
-    if dom_name == "band_pass_fp64":
+    if dom_name == "band_pass_fp64" and dom_name not in fixed_point_classes(n, p):
         achieved = dom["flops"] / (dom["ms"] / 1e3) / 1e12
         roof = dict(common, bound="alu", achieved=achieved, peak=FP64_PEAK_TFLOPS,
                     unit="TFLOP/s", frac=achieved / FP64_PEAK_TFLOPS, traffic=None,
@@ -996,7 +1006,8 @@ def run_cavity128(args, wl):
             "forms": forms,
             "roofline": roof,
             "tensor_core_fd": tc_roof,
-            "kernel_classes": class_rooflines(prof, step_ms_profiled, prec, peaks),
+            "kernel_classes": class_rooflines(prof, step_ms_profiled, prec, peaks,
+                                               fixed_point_classes(n, p)),
             "setup_ms": round(setup_ms, 1),
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": "solves/s",
@@ -1186,15 +1197,16 @@ def run_sweep(args, wl):
     dom = prof[dom_name]
     peaks = load_peaks() or {}
     if dom_name == "mode_product" and prec == "fp64":
-        # Live throughput of the class: the base preconditioner P_0 consists of mode products
-        # only (velocity and pressure fast diagonalisations, run as two concurrent branches), so
-        # back-to-back P_0 applications between two events on the library stream time exactly
+        # Live throughput of the class: the base preconditioner P_0 consists of dense products
+        # only (velocity fast diagonalisation and pressure mass inverse, run as two concurrent
+        # branches; classes mode_product and line_solve), so back-to-back P_0 applications between two events on the library stream time exactly
         # these kernels as they run inside the solves (no per-launch events in between).
         xP = torch.randn(G.size, dtype=torch.float64, device="cuda")
         yP = torch.empty_like(xP)
         G.profile_begin()
         G.apply_P(xP, out=yP)
-        one = G.profile_end()["mode_product"]
+        one = G.profile_end()
+        one = {k: one["mode_product"][k] + one["line_solve"][k] for k in ("flops", "launches")}
         reps = 100
         for _ in range(5):
             G.apply_P(xP, out=yP)
@@ -1208,20 +1220,31 @@ def run_sweep(args, wl):
         ms_p = a.elapsed_time(b)
         achieved = one["flops"] * reps / (ms_p / 1e3) / 1e12
         fused = G.tuning()[2]
-        roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
-                "kernel": ("k_fd_plane + k_fd_line3 (mode_product class, fused fast "
-                           "diagonalisation)" if fused else "k_mode_tile (mode_product class)"),
+        if "mode_product" in fixed_point_classes(n, p):
+            # each FP64 product as 21 FP16 digit products on the tensor cores (padding not counted)
+            achieved, bound = 21 * achieved, "tensor"
+            peak = peaks.get("bf16_tflops", 1900.0)
+            note = ("measured BF16 burst; FP16 digit products, 21 per FP64 product" if
+                    "bf16_tflops" in peaks else "fallback; FP16 digit products, 21 per FP64 product")
+            kernel = "k_fix_plane + k_fix_line3" if fused else "k_fix_mode"
+        else:
+            bound, peak = "alu", FP64_PEAK_TFLOPS
+            note = "nominal GB300 FP64 1.25 TFLOP/s (an FMA probe measured 1.20)"
+            kernel = "k_fd_plane + k_fd_line3" if fused else "k_mode_tile"
+        roof = {"bound": bound, "achieved": achieved, "peak": peak,
+                "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
+                "kernel": kernel + " (mode_product class)",
                 "form": fd_form(fused),
                 "measurement": f"{reps} back-to-back P_0 applications ({one['launches']} mode-product "
                                f"launches each) between two CUDA events on the library stream",
                 "avg_launch_us": 1e3 * ms_p / (reps * max(one["launches"], 1)),
                 "launches_per_step": dom["launches"],
-                "profiled_pass": {"achieved": dom["flops"] / (dom["ms"] / 1e3) / 1e12,
+                "profiled_pass": {"fp64_tflops": dom["flops"] / (dom["ms"] / 1e3) / 1e12,
                                   "avg_launch_us": 1e3 * dom["ms"] / max(dom["launches"], 1),
                                   "note": "CUDA events around every launch, branches serial"},
-                "peak_note": "nominal GB300 FP64 1.25 TFLOP/s (an FMA probe measured 1.20)"}
-    elif dom_name in ("band_pass", "band_pass_fp64") and prec == "fp64":
+                "peak_note": note}
+    elif (dom_name in ("band_pass", "band_pass_fp64") and prec == "fp64"
+          and dom_name not in fixed_point_classes(n, p)):
         achieved = dom["flops"] / (dom["ms"] / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
                 "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
@@ -1322,7 +1345,8 @@ def run_sweep(args, wl):
             "table1_form": table1,
             "sweep_concurrent": sweep_conc,
             "roofline": roof,
-            "kernel_classes": class_rooflines(prof, step_ms_profiled, prec, peaks),
+            "kernel_classes": class_rooflines(prof, step_ms_profiled, prec, peaks,
+                                               fixed_point_classes(n, p)),
             "setup_ms": round(setup_ms, 1),
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": "solves/s",

@@ -91,7 +91,7 @@ typedef struct stokes_opts {
                          preconditioner runs in reduced precision (z is then its FP32 output):
                          STOKES_OUTER_FP64 (default) or STOKES_OUTER_PAIR (every value carried as
                          an unevaluated sum of two FP32 numbers, about 48 significant bits, w
-                         rounded to FP64; on this GPU's reduced FP64 pipe about twice as fast).
+                         rounded to FP64; about as fast as the FP64 form).
                          Residuals of the iterate (restarts, the final true residual),
                          stokes_apply_K and every FP64-preconditioned solve use the FP64
                          operator either way. Used with the Kronecker forward operator when
@@ -234,10 +234,11 @@ int stokes_solve_batch(stokes_t* ctxs, int count, const double* const* rhs, doub
 int stokes_last_ratios(stokes_t ctx, double* ratios, int capacity);
 
 /* ---- instrumentation (no counterpart in the paper) ------------------------------------------
- * Kernel classes: 0 banded Kronecker passes in FP32, 1 dense mode products on CUDA cores,
+ * Kernel classes: 0 banded Kronecker passes in FP32, 1 dense mode products of FP64 and FP32,
  * 2 discrete divergence / transpose, 3 Krylov vector kernels, 4 tensor-core mode products,
- * 5 pressure-mass inverse along one direction (FP64, b >= 64), 6 banded Kronecker passes in FP64, 7 the saddle-point operator
- * in pair-of-FP32 arithmetic (its banded passes and fused divergence).
+ * 5 pressure-mass inverse along one direction (FP64, n_elems + degree_p > 24), 6 banded Kronecker
+ * passes in FP64, 7 the saddle-point operator in pair-of-FP32 arithmetic (its banded passes and
+ * fused divergence).
  * stokes_profile_begin brackets every later launch of this thread with CUDA events on the
  * launching stream; stokes_profile_end synchronizes, writes per-class totals (launches, summed
  * event intervals in ms, algorithmic flops and bytes: each input read once, each output written

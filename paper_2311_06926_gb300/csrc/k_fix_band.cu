@@ -12,7 +12,7 @@
 // precision only against entries that meet it in the same outputs.
 //
 // Bound by instruction issue: about 125 instructions per result, of which the 27 multiply-adds of a
-// row of 9 take twice their slots. Measured against the FMA passes: K apply 1051 -> 525 us at 128^3
+// row of 9 take twice their slots. Measured against the FMA passes: K apply 1052 -> 530 us at 128^3
 // p = 3, 150 -> 83 at 64^3.
 //
 // A window with an infinity or a NaN, or outside [2^-823, 2^777], takes FMA chains instead.

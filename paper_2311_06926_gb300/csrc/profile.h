@@ -14,7 +14,7 @@ enum KernelClass {
   kClassDiv = 2,       // discrete divergence and its transpose
   kClassVector = 3,    // Krylov vector kernels, dot products, conversions
   kClassMma = 4,       // tensor-core mode products
-  kClassLine = 5,      // pressure-mass inverse along one direction (FP64, 64 entries or more)
+  kClassLine = 5,      // pressure-mass inverse along one direction (FP64, more than 24 entries)
   kClassBand64 = 6,    // FP64 banded Kronecker passes (class 0 then holds the FP32 ones)
   kClassPair = 7,      // banded passes and divergence in pair-of-FP32 arithmetic
   kNumClasses = 8
