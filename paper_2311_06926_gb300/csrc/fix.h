@@ -25,6 +25,12 @@
 
 #include <cstdint>
 
+#ifdef __CUDACC__
+#define SHP_HD __host__ __device__ __forceinline__
+#else
+#define SHP_HD inline
+#endif
+
 namespace shp {
 
 constexpr int kFixSlices = 6, kFixDigit = 10;

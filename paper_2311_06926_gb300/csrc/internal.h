@@ -200,7 +200,6 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s);
 void fix_div_band_x1(const double* u1, const double* u2, const double* u3, int a, int b,
                      const double* q, double nu, const BandD<double>& D, double* y0, double* y1,
                      int block, cudaStream_t s);
-constexpr int kFixBandHalf = 6;   // largest half width of the limb tables
 // smallest pressure extent b of the fixed-point passes: below, a pass is a few waves of short chains
 // and the FMA kernels take less time (K apply at 32^3 p = 3: 32 against 35 us; at 64^3: 150 against
 // 83)

@@ -19,7 +19,7 @@
 #include <algorithm>
 #include <atomic>
 
-#include "fix.h"
+#include "fix_band.h"
 #include "internal.h"
 #include "profile.h"
 
@@ -27,7 +27,6 @@ namespace shp {
 namespace {
 
 constexpr int kBandLimb = 29, kBandXBits = 57;
-constexpr int kR = 8;   // outputs per thread along the band
 
 struct FixBandOp {
   const int4* tab;   // [segment][8 rows][band_row]: {hi, lo, hi, lo} of entries 2 q, 2 q + 1
@@ -61,14 +60,6 @@ struct FixBandBatch {
   int first[kMaxPassJobs + 1];
   int njobs;
 };
-
-// Half width H >= 1: centred square bands, row r of a segment reads entries r .. r + 2 H of the
-// window (2 H + 2 stored, the last one zero). H = 0: rectangular bands (the quadrature tables: several
-// points per element), whose segments read at most 8 inputs; every row has all 8.
-__host__ __device__ constexpr int band_row(int H) { return H ? H + 1 : 4; }   // int4 per row
-// int4 per segment in shared memory: one more than the rows take, so that lanes on neighbouring
-// segments read different banks
-__host__ __device__ constexpr int band_seg(int H) { return kR * band_row(H) + 1; }
 
 __device__ __forceinline__ void band_mad(long long& c, int a, int b) {
   c += (long long)a * b;
@@ -290,12 +281,7 @@ __device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4
     band_chains(J, seg, m, [&](int t, int j) { return J.X[t][first + (int64_t)stride * j]; }, put);
 }
 
-// Staged x1 lines (shared memory): entry j, -H <= j < 8 segs + H, of a line at
-// ((j + H) % 8) S + (j + H) / 8 with S odd, zero outside the line; neighbouring threads (segments)
-// then read and write neighbouring words, and no window needs a bound.
-__host__ __device__ constexpr int band_stage_s(int segs, int H) {
-  return (segs + (2 * H + 7) / 8) | 1;
-}
+// position of entry j - H of a staged line (fix_band.h)
 __device__ __forceinline__ int band_stage(int j, int S) { return (j & 7) * S + (j >> 3); }
 
 // zeros around the m entries of nl staged lines
@@ -505,19 +491,14 @@ void band_divisor(int n1, FixBandJob& J) {
 
 // threads of a block whose x1 lines need `segs` threads each
 int band_threads(int block, int segs) {
-  const int t = block > 0 ? std::min(block, 256) : 256;
+  const int t = block > 0 ? std::min(block, kFixBandThreads) : kFixBandThreads;
   return std::max(t, (segs + 31) / 32 * 32);
 }
-// shared memory of a block of x1 lines: the operators' limbs and scales, and nline staged lines
-int band_along_smem(int nops, int nline, int segs, int H) {
-  return nops * segs * band_seg(H) * 16 + ((nops * segs + 1) & ~1) * 4 +
-         nline * kR * band_stage_s(segs, H) * 8;
-}
-
 template <int H, int NT, bool EPI>
 void launch_fix_band(const FixBandBatch& fb, int blocks, int threads, int smem, cudaStream_t s) {
   static std::atomic<int> attr{0};
-  raise_smem_limit(k_fix_band<H, NT, EPI>, attr, smem);
+  // (a refused size is left as the thread's last error, which every caller of the passes checks)
+  if (raise_smem_limit(k_fix_band<H, NT, EPI>, attr, smem) != cudaSuccess) return;
   launch_k(k_fix_band<H, NT, EPI>, blocks, threads, smem, s, fb);
 }
 template <int H>
@@ -535,7 +516,7 @@ void launch_fix_div(const double* u1, const double* u2, const double* u3, int a,
                     const double* q, double nu, const FixBandJob& J, double* y1, int blocks,
                     int threads, int smem, cudaStream_t s) {
   static std::atomic<int> attr{0};
-  raise_smem_limit(k_fix_div_x1<H>, attr, smem);
+  if (raise_smem_limit(k_fix_div_x1<H>, attr, smem) != cudaSuccess) return;
   launch_k(k_fix_div_x1<H>, blocks, threads, smem, s, u1, u2, u3, a, b, q, nu, J, y1);
 }
 
@@ -556,7 +537,7 @@ bool fix_band_ok(const PassArgs<double>* jobs, int njobs) {
         (a.nterms > 1 && (!a.f1.tab || a.f1.half != H || a.D1.rows != m || a.c1 != 1.0)) ||
         (a.Y2 && (!a.D2.fix.tab || a.D2.fix.half != H || a.D2.rows != m)) ||
         a.c0 != 1.0 ||
-        (a.axis == 1 && (a.g || a.hmode || (a.nterms > 1 && !a.Y2) || (m + kR - 1) / kR > 256)) ||
+        (a.axis == 1 && (a.g || a.hmode || (a.nterms > 1 && !a.Y2) || !fix_band_fits(m, H))) ||
         (a.Y2 && (a.g || a.hmode)) ||
         (H == 0 && a.D0.cols != a.in.get(a.axis)) ||
         a.in.size() / a.in.get(a.axis) * nb >= ((int64_t)1 << 30))
@@ -572,7 +553,7 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
   int threads = 32;
   for (int j = 0; j < njobs; ++j)
     threads = std::max(threads, band_threads(jobs[j].block, jobs[j].axis == 1
-                                                               ? (jobs[j].D0.rows + kR - 1) / kR
+                                                               ? band_segs(jobs[j].D0.rows)
                                                                : 1));
   int blocks = 0, smem = 3 * kR * band_row(H) * 16 + 16;
   bool epi = false;
@@ -607,13 +588,13 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
     J.bs = a.bs;
     const int m = a.D0.rows;
     J.rows = m;
-    J.segs = (m + kR - 1) / kR;
+    J.segs = band_segs(m);
     const int lines = (int)(a.in.size() / a.in.get(a.axis)) * J.nb;
     fb.first[j] = blocks;
     if (a.axis == 1) {
       const int lpb = threads / J.segs;
       blocks += (lines + lpb - 1) / lpb;
-      smem = std::max(smem, band_along_smem(J.nops, lpb * (a.nterms + (a.Y2 ? 2 : 1)), J.segs, H));
+      smem = std::max(smem, (int)band_along_smem(J.nops, lpb * (a.nterms + (a.Y2 ? 2 : 1)), J.segs, H));
     } else {
       blocks += (lines + threads - 1) / threads * J.segs;
     }
@@ -646,11 +627,11 @@ void fix_div_band_x1(const double* u1, const double* u2, const double* u3, int a
   J.nterms = J.nops = 1;
   J.nb = 1;
   band_divisor(b, J);
-  J.segs = (b + kR - 1) / kR;
+  J.segs = band_segs(b);
   const int nv = q ? 2 : 1;
   const int H = D.fix.half, threads = band_threads(block, J.segs * nv);
   const int lpb = threads / (J.segs * nv), blocks = (b * b + lpb - 1) / lpb;
-  const int smem = band_along_smem(1, 2 * nv * lpb, J.segs, H);
+  const int smem = (int)band_along_smem(1, 2 * nv * lpb, J.segs, H);
   const double np = (double)b * b * b;
   launch_begin(kClassDiv, s);
   switch (H) {
