@@ -1,0 +1,94 @@
+// Tables of the fixed-point FP64 passes, formed on the host at set-up (layouts: fix_band.h).
+#pragma once
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "fix_band.h"
+#include "host_setup.h"
+
+namespace shp {
+
+// Limbs of a band: per segment of 8 rows one scale 2^ex, below which the entries are integers of
+// magnitude at most 2^58, and rows of 2 H + 2 entries (8 if rectangular) as {hi, lo} with
+// v = hi 2^29 + lo, |lo| <= 2^28. Empty: the band has no such table.
+struct BandLimbs {
+  std::vector<int> tab, ex, w0;
+};
+
+// entry v of a band at the scale 2^ex into slot k
+inline void band_limb_entry(BandLimbs& t, size_t k, double x, int ex) {
+  const long long v = std::llrint(std::ldexp(x, -ex));
+  const int h = (int)((v + (1ll << 28)) >> 29);
+  t.tab[2 * k] = h;
+  t.tab[2 * k + 1] = (int)(v - ((long long)h << 29));
+}
+
+// largest magnitude of rows i0 .. i1 - 1
+inline double band_max(const Band& b, int i0, int i1) {
+  double mx = 0;
+  for (size_t k = (size_t)i0 * b.width; k < (size_t)i1 * b.width; ++k)
+    mx = std::max(mx, std::fabs(b.val[k]));
+  return mx;
+}
+
+// A square band, centred with half width H >= its own.
+inline BandLimbs band_limbs_square(const Band& b, int H) {
+  const int segs = band_segs(b.rows), per = 2 * band_row(H);
+  BandLimbs t;
+  t.tab.assign((size_t)segs * kR * per * 2, 0);
+  t.ex.assign(segs, 0);
+  for (int sg = 0; sg < segs; ++sg) {
+    const int i1 = std::min(b.rows, kR * sg + kR);
+    const double mx = band_max(b, kR * sg, i1);
+    if (mx == 0) continue;
+    t.ex[sg] = std::ilogb(mx) + 1 - 58;
+    for (int i = kR * sg; i < i1; ++i)
+      for (int w = 0; w < b.width; ++w) {
+        const int k = b.start[i] + w - i + H;
+        if (k < 0 || k > 2 * H) continue;   // (zero entries only: |k - H| > the half width)
+        band_limb_entry(t, (size_t)i * per + k, b.val[(size_t)i * b.width + w], t.ex[sg]);
+      }
+  }
+  return t;
+}
+
+// A pair of rectangular bands over the same inputs (a table's values and derivatives), which a pass
+// with two results applies to one window: every segment's window (first input w0) holds the inputs
+// of both, although exact zeros may make the bands start at different inputs. Returns false, with
+// empty tables, if a segment of the pair reads more than 8 inputs.
+inline bool band_limbs_rect(const Band& b0, const Band& b1, BandLimbs& t0, BandLimbs& t1) {
+  const Band* b[2] = {&b0, &b1};
+  BandLimbs* t[2] = {&t0, &t1};
+  const int rows = b0.rows, segs = band_segs(rows), per = 2 * band_row(0);
+  bool ok = b1.rows == rows && b1.cols == b0.cols;
+  for (int o = 0; o < 2; ++o) {
+    t[o]->tab.assign((size_t)segs * kR * per * 2, 0);
+    t[o]->ex.assign(segs, 0);
+    t[o]->w0.assign(segs, 0);
+  }
+  for (int sg = 0; ok && sg < segs; ++sg) {
+    const int i1 = std::min(rows, kR * sg + kR);
+    int lo = b0.cols, hi = 0;
+    for (int i = kR * sg; i < i1; ++i)
+      for (int o = 0; o < 2; ++o) {
+        lo = std::min(lo, b[o]->start[i]);
+        hi = std::max(hi, std::min(b[o]->start[i] + b[o]->width, b[o]->cols));
+      }
+    ok = hi - lo <= per;
+    for (int o = 0; ok && o < 2; ++o) {
+      t[o]->w0[sg] = lo;
+      const double mx = band_max(*b[o], kR * sg, i1);
+      if (mx == 0) continue;
+      t[o]->ex[sg] = std::ilogb(mx) + 1 - 58;
+      for (int i = kR * sg; i < i1; ++i)
+        for (int w = 0; w < b[o]->width && b[o]->start[i] + w < b[o]->cols; ++w)
+          band_limb_entry(*t[o], (size_t)i * per + (b[o]->start[i] + w - lo),
+                          b[o]->val[(size_t)i * b[o]->width + w], t[o]->ex[sg]);
+    }
+  }
+  if (!ok) t0 = t1 = BandLimbs{};
+  return ok;
+}
+
+}  // namespace shp

@@ -31,7 +31,7 @@
 #include <utility>
 #include <vector>
 
-#include "fix_band.h"
+#include "fix_tables.h"
 #include "host_setup.h"
 #include "internal.h"
 #include "mma.h"
@@ -182,72 +182,31 @@ BandD<T> upload_band(Arena& ar, const Band& b, cudaStream_t s, int min_half = 0)
   return d;
 }
 
-// Limb table of a square band for the fixed-point passes (k_fix_band.cu), centred with half width
-// H >= its own: per segment of 8 rows one scale, below which the entries are integers of magnitude
-// at most 2^58, and rows of 2 H + 2 entries (the last one zero) as {hi, lo} with
-// v = hi 2^29 + lo, |lo| <= 2^28.
-void upload_fix_band(Arena& ar, const Band& b, BandD<double>& d, int H, cudaStream_t s) {
-  if (b.rows != b.cols || d.half > H) return;
-  const int segs = (b.rows + 7) / 8, per = 2 * H + 2;
-  std::vector<int> tab((size_t)segs * 8 * per * 2, 0), ex(segs, 0);
-  for (int sg = 0; sg < segs; ++sg) {
-    double mx = 0;
-    const int i1 = std::min(b.rows, 8 * sg + 8);
-    for (int i = 8 * sg; i < i1; ++i)
-      for (int w = 0; w < b.width; ++w) mx = std::max(mx, std::fabs(b.val[(size_t)i * b.width + w]));
-    if (mx == 0) continue;
-    ex[sg] = std::ilogb(mx) + 1 - 58;
-    for (int i = 8 * sg; i < i1; ++i)
-      for (int w = 0; w < b.width; ++w) {
-        const int k = b.start[i] + w - i + H;
-        if (k < 0 || k > 2 * H) continue;   // (zero entries only: |k - H| > d.half)
-        const long long v = std::llrint(std::ldexp(b.val[(size_t)i * b.width + w], -ex[sg]));
-        const int h = (int)((v + (1ll << 28)) >> 29);
-        tab[((size_t)i * per + k) * 2] = h;
-        tab[((size_t)i * per + k) * 2 + 1] = (int)(v - ((long long)h << 29));
-      }
-  }
-  int* td = ar.alloc<int>(tab.size());
-  int* ed = ar.alloc<int>(ex.size());
-  ck(cudaMemcpyAsync(td, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
-  ck(cudaMemcpyAsync(ed, ex.data(), ex.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
+BandFix upload_limbs(Arena& ar, const BandLimbs& t, int H, cudaStream_t s) {
+  std::vector<int> all(t.tab);   // the 16-byte words of the limbs first
+  all.insert(all.end(), t.ex.begin(), t.ex.end());
+  all.insert(all.end(), t.w0.begin(), t.w0.end());
+  int* d = ar.alloc<int>(all.size());
+  ck(cudaMemcpyAsync(d, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
   ck(cudaStreamSynchronize(s), "fix");
-  d.fix = BandFix{reinterpret_cast<const int4*>(td), ed, nullptr, H};
+  const int* ex = d + t.tab.size();
+  return BandFix{reinterpret_cast<const int4*>(d), ex, t.w0.empty() ? nullptr : ex + t.ex.size(),
+                 H};
 }
 
-// The same for a rectangular band whose 8-row segments read at most 8 inputs each (none otherwise):
-// rows of 8 entries, from the segment's first input fw0.
-void upload_fix_rect(Arena& ar, const Band& b, BandD<double>& d, cudaStream_t s) {
-  const int segs = (b.rows + 7) / 8;
-  std::vector<int> tab((size_t)segs * 8 * 8 * 2, 0), ex(2 * (size_t)segs, 0);
-  for (int sg = 0; sg < segs; ++sg) {
-    const int i1 = std::min(b.rows, 8 * sg + 8);
-    int lo = b.cols, hi = 0;
-    double mx = 0;
-    for (int i = 8 * sg; i < i1; ++i) {
-      lo = std::min(lo, b.start[i]);
-      hi = std::max(hi, b.start[i] + b.width);
-      for (int w = 0; w < b.width; ++w) mx = std::max(mx, std::fabs(b.val[(size_t)i * b.width + w]));
-    }
-    if (hi - lo > 8) return;
-    ex[segs + sg] = lo;
-    if (mx == 0) continue;
-    ex[sg] = std::ilogb(mx) + 1 - 58;
-    for (int i = 8 * sg; i < i1; ++i)
-      for (int w = 0; w < b.width; ++w) {
-        const long long v = std::llrint(std::ldexp(b.val[(size_t)i * b.width + w], -ex[sg]));
-        const int h = (int)((v + (1ll << 28)) >> 29);
-        const size_t k = ((size_t)i * 8 + (b.start[i] + w - lo)) * 2;
-        tab[k] = h;
-        tab[k + 1] = (int)(v - ((long long)h << 29));
-      }
-  }
-  int* td = ar.alloc<int>(tab.size());
-  int* ed = ar.alloc<int>(ex.size());
-  ck(cudaMemcpyAsync(td, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
-  ck(cudaMemcpyAsync(ed, ex.data(), ex.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
-  ck(cudaStreamSynchronize(s), "fix");
-  d.fix = BandFix{reinterpret_cast<const int4*>(td), ed, ed + segs, 0};
+// The fixed-point form of a square band, centred with half width H (none if the band is wider)
+void upload_fix_band(Arena& ar, const Band& b, BandD<double>& d, int H, cudaStream_t s) {
+  if (b.rows != b.cols || d.half > H) return;
+  d.fix = upload_limbs(ar, band_limbs_square(b, H), H, s);
+}
+
+// The fixed-point form of a table's values and derivatives (none if their windows are too long)
+void upload_fix_rect(Arena& ar, const Band& v, const Band& dv, BandD<double>& d,
+                     BandD<double>& dd, cudaStream_t s) {
+  BandLimbs t[2];
+  if (!band_limbs_rect(v, dv, t[0], t[1])) return;
+  d.fix = upload_limbs(ar, t[0], 0, s);
+  dd.fix = upload_limbs(ar, t[1], 0, s);
 }
 
 template <typename T>
@@ -2339,15 +2298,15 @@ void init_quad(stokes_ctx* c) {
   q->s = s;
   q->band_block = c->od.band_block;
   // tables in band form (exact zeros outside the supports)
-  q->BN = upload_band<double>(ar, to_band(qt.BN, 0.0), s);
-  q->DN = upload_band<double>(ar, to_band(qt.DN, 0.0), s);
-  q->BM = upload_band<double>(ar, to_band(qt.BM, 0.0), s);
-  q->DM = upload_band<double>(ar, to_band(qt.DM, 0.0), s);
+  const Band BN = to_band(qt.BN, 0.0), DN = to_band(qt.DN, 0.0);
+  const Band BM = to_band(qt.BM, 0.0), DM = to_band(qt.DM, 0.0);
+  q->BN = upload_band<double>(ar, BN, s);
+  q->DN = upload_band<double>(ar, DN, s);
+  q->BM = upload_band<double>(ar, BM, s);
+  q->DM = upload_band<double>(ar, DM, s);
   if (qt.nq >= kFixRectMin) {
-    upload_fix_rect(ar, to_band(qt.BN, 0.0), q->BN, s);
-    upload_fix_rect(ar, to_band(qt.DN, 0.0), q->DN, s);
-    upload_fix_rect(ar, to_band(qt.BM, 0.0), q->BM, s);
-    upload_fix_rect(ar, to_band(qt.DM, 0.0), q->DM, s);
+    upload_fix_rect(ar, BN, DN, q->BN, q->DN, s);
+    upload_fix_rect(ar, BM, DM, q->BM, q->DM, s);
   }
   q->BNt = upload_band<double>(ar, to_band(transposed(qt.BN), 0.0), s);
   q->DNt = upload_band<double>(ar, to_band(transposed(qt.DN), 0.0), s);

@@ -5,6 +5,7 @@ import os
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -53,3 +54,41 @@ def test_banded_passes_that_do_not_fit_are_not_offered(lib, H):
     # the sizes that a set-up used to fail at
     for b, half in ((489, 6), (585, 5), (673, 4), (881, 3), (1265, 2)):
         assert not lib.fits(b, half)
+
+
+def _ptr(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+@pytest.mark.parametrize("zeros", ["leading", "trailing", "none"])
+def test_rectangular_tables_of_a_pair_share_their_windows(lib, zeros):
+    """A pass with two results loads one window: exact zeros at one end of one band must not move
+    its table against the other's."""
+    rng = np.random.default_rng(3)
+    rows, cols, width = 21, 12, 4
+    first = np.arange(rows) // 3                      # the inputs of the values
+    second = first + {"leading": 1, "trailing": -1, "none": 0}[zeros]
+    second = np.clip(second, 0, cols - width).astype(np.int32)
+    first = np.clip(first, 0, cols - width).astype(np.int32)
+    val = [rng.uniform(0.5, 1.0, (rows, width)) for _ in range(2)]
+    w0 = np.zeros((2, 3), np.int32)
+    dense = np.zeros((2, rows, cols))
+    assert lib.rect_pair(rows, cols, width, _ptr(first), _ptr(val[0]), _ptr(second), _ptr(val[1]),
+                         _ptr(w0), _ptr(dense)) == 1
+    assert np.array_equal(w0[0], w0[1])
+    for o, start in enumerate((first, second)):
+        ref = np.zeros((rows, cols))
+        for i in range(rows):
+            ref[i, start[i]:start[i] + width] = val[o][i]
+        assert np.abs(dense[o] - ref).max() <= 2.0 ** -53
+
+
+def test_rectangular_tables_need_windows_of_eight(lib):
+    """A pair whose segments read nine inputs together has no tables, though each band alone would."""
+    rows, cols, width = 8, 16, 4
+    a, b = np.full(rows, 0, np.int32), np.full(rows, 5, np.int32)
+    val = np.ones((rows, width))
+    w0, dense = np.zeros((2, 1), np.int32), np.zeros((2, rows, cols))
+    args = [_ptr(val), _ptr(w0), _ptr(dense)]
+    assert lib.rect_pair(rows, cols, width, _ptr(a), args[0], _ptr(b), *args) == 0
+    assert lib.rect_pair(rows, cols, width, _ptr(a), args[0], _ptr(a + 4), *args) == 1
