@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
 
 #ifdef __CUDACC__
 #define SHP_HD __host__ __device__ __forceinline__
@@ -60,37 +61,73 @@ struct FixTabs {
   FixTab fw, bw;
 };
 
-#ifdef __CUDACC__
 // biased exponents of the largest entry of a line that the fixed-point form takes
 constexpr unsigned kFixMinExp = 200, kFixMaxExp = 1800;
 
+// The words of a double, and a funnel shift (the arithmetic below also compiles for the host, where
+// its tests run it).
+SHP_HD unsigned hi_word(double x) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2hiint(x);
+#else
+  uint64_t u;
+  std::memcpy(&u, &x, sizeof u);
+  return (unsigned)(u >> 32);
+#endif
+}
+SHP_HD unsigned lo_word(double x) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2loint(x);
+#else
+  uint64_t u;
+  std::memcpy(&u, &x, sizeof u);
+  return (unsigned)u;
+#endif
+}
+SHP_HD double from_words(unsigned hi, unsigned lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double((int)hi, (int)lo);
+#else
+  const uint64_t u = (uint64_t)hi << 32 | lo;
+  double x;
+  std::memcpy(&x, &u, sizeof x);
+  return x;
+#endif
+}
+SHP_HD unsigned funnel_left(unsigned lo, unsigned hi, int n) {   // 0 < n < 32
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(lo, hi, n);
+#else
+  return hi << n | lo >> (32 - n);
+#endif
+}
+
 // Magnitude key of an entry: its exponent field and leading bits (the low word only marks a
 // nonzero). The largest key of a line gives its scale; 0 only for a line of zeros.
-__device__ __forceinline__ unsigned fix_key(double x) {
-  return ((unsigned)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
+SHP_HD unsigned fix_key(double x) {
+  return (hi_word(x) & 0x7fffffffu) | (lo_word(x) != 0 ? 1u : 0u);
 }
-__device__ __forceinline__ bool fix_slow(unsigned key) {
+SHP_HD bool fix_slow(unsigned key) {
   const unsigned e = key >> 20;
   return key != 0u && (e < kFixMinExp || e > kFixMaxExp);
 }
 // x / 2^(emax - 1022) * 2^xbits, rounded (emax: exponent field of the largest entry)
-__device__ __forceinline__ long long fix_of(double x, int emax, int xbits) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+SHP_HD long long fix_of(double x, int emax, int xbits) {
+  const unsigned hi = hi_word(x), lo = lo_word(x);
   const int e = (int)((hi >> 20) & 0x7ffu);
   const unsigned m = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
   // the 53-bit significand with its leading bit at bit 62
-  const unsigned long long n = ((unsigned long long)__funnelshift_l(lo, m, 10) << 32) | (lo << 10);
-  const int sh = min(62 - xbits + emax - e, 63);
+  const unsigned long long n = ((unsigned long long)funnel_left(lo, m, 10) << 32) | (lo << 10);
+  const int t = 62 - xbits + emax - e, sh = t < 63 ? t : 63;
   const long long v = (long long)(((n >> sh) + 1) >> 1);
   return (int)hi < 0 ? -v : v;
 }
 // s * 2^ex as a double (ex keeps it in the normal range). By the conversion instruction, on the FP64
 // pipe that these kernels leave idle (in about 20 integer instructions instead: 128^3 K apply 526
 // against 501 us, P_0^-1 914 against 901).
-__device__ __forceinline__ double fix_to_double(long long s, int ex) {
+SHP_HD double fix_to_double(long long s, int ex) {
   const double d = (double)s;
-  return s == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + ex * (1 << 20), __double2loint(d));
+  return s == 0 ? 0.0 : from_words(hi_word(d) + (unsigned)ex * (1u << 20), lo_word(d));
 }
-#endif
 
 }  // namespace shp

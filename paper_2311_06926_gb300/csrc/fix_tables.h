@@ -9,9 +9,11 @@
 
 namespace shp {
 
-// Limbs of a band: per segment of 8 rows one scale 2^ex, below which the entries are integers of
-// magnitude at most 2^58, and rows of 2 H + 2 entries (8 if rectangular) as {hi, lo} with
-// v = hi 2^29 + lo, |lo| <= 2^28. Empty: the band has no such table.
+// Limbs of a band: per row one scale 2^ex (row r of segment seg at r segs + seg), at which the
+// entries are integers of magnitude at most 2^58, and 2 H + 2 entries (8 if rectangular) as {hi, lo}
+// with v = hi 2^29 + lo, |lo| <= 2^28. (One scale for the 8 rows of a segment is not enough: the
+// rows beside the penalty row of T-check are 2^4 to 2^10 smaller, and held only that many bits
+// fewer.) Empty: the band has no such table.
 struct BandLimbs {
   std::vector<int> tab, ex, w0;
 };
@@ -24,12 +26,11 @@ inline void band_limb_entry(BandLimbs& t, size_t k, double x, int ex) {
   t.tab[2 * k + 1] = (int)(v - ((long long)h << 29));
 }
 
-// largest magnitude of rows i0 .. i1 - 1
-inline double band_max(const Band& b, int i0, int i1) {
+// the scale of row i (0: a row of zeros)
+inline int band_row_scale(const Band& b, int i) {
   double mx = 0;
-  for (size_t k = (size_t)i0 * b.width; k < (size_t)i1 * b.width; ++k)
-    mx = std::max(mx, std::fabs(b.val[k]));
-  return mx;
+  for (int w = 0; w < b.width; ++w) mx = std::max(mx, std::fabs(b.val[(size_t)i * b.width + w]));
+  return mx > 0 ? std::ilogb(mx) + 1 - 58 : 0;
 }
 
 // A square band, centred with half width H >= its own.
@@ -37,18 +38,15 @@ inline BandLimbs band_limbs_square(const Band& b, int H) {
   const int segs = band_segs(b.rows), per = 2 * band_row(H);
   BandLimbs t;
   t.tab.assign((size_t)segs * kR * per * 2, 0);
-  t.ex.assign(segs, 0);
-  for (int sg = 0; sg < segs; ++sg) {
-    const int i1 = std::min(b.rows, kR * sg + kR);
-    const double mx = band_max(b, kR * sg, i1);
-    if (mx == 0) continue;
-    t.ex[sg] = std::ilogb(mx) + 1 - 58;
-    for (int i = kR * sg; i < i1; ++i)
-      for (int w = 0; w < b.width; ++w) {
-        const int k = b.start[i] + w - i + H;
-        if (k < 0 || k > 2 * H) continue;   // (zero entries only: |k - H| > the half width)
-        band_limb_entry(t, (size_t)i * per + k, b.val[(size_t)i * b.width + w], t.ex[sg]);
-      }
+  t.ex.assign((size_t)segs * kR, 0);
+  for (int i = 0; i < b.rows; ++i) {
+    const int ex = band_row_scale(b, i);
+    t.ex[(size_t)(i % kR) * segs + i / kR] = ex;
+    for (int w = 0; w < b.width; ++w) {
+      const int k = b.start[i] + w - i + H;
+      if (k < 0 || k > 2 * H) continue;   // (zero entries only: |k - H| > the half width)
+      band_limb_entry(t, (size_t)i * per + k, b.val[(size_t)i * b.width + w], ex);
+    }
   }
   return t;
 }
@@ -64,7 +62,7 @@ inline bool band_limbs_rect(const Band& b0, const Band& b1, BandLimbs& t0, BandL
   bool ok = b1.rows == rows && b1.cols == b0.cols;
   for (int o = 0; o < 2; ++o) {
     t[o]->tab.assign((size_t)segs * kR * per * 2, 0);
-    t[o]->ex.assign(segs, 0);
+    t[o]->ex.assign((size_t)segs * kR, 0);
     t[o]->w0.assign(segs, 0);
   }
   for (int sg = 0; ok && sg < segs; ++sg) {
@@ -78,13 +76,13 @@ inline bool band_limbs_rect(const Band& b0, const Band& b1, BandLimbs& t0, BandL
     ok = hi - lo <= per;
     for (int o = 0; ok && o < 2; ++o) {
       t[o]->w0[sg] = lo;
-      const double mx = band_max(*b[o], kR * sg, i1);
-      if (mx == 0) continue;
-      t[o]->ex[sg] = std::ilogb(mx) + 1 - 58;
-      for (int i = kR * sg; i < i1; ++i)
+      for (int i = kR * sg; i < i1; ++i) {
+        const int ex = band_row_scale(*b[o], i);
+        t[o]->ex[(size_t)(i % kR) * segs + sg] = ex;
         for (int w = 0; w < b[o]->width && b[o]->start[i] + w < b[o]->cols; ++w)
           band_limb_entry(*t[o], (size_t)i * per + (b[o]->start[i] + w - lo),
-                          b[o]->val[(size_t)i * b[o]->width + w], t[o]->ex[sg]);
+                          b[o]->val[(size_t)i * b[o]->width + w], ex);
+      }
     }
   }
   if (!ok) t0 = t1 = BandLimbs{};

@@ -4,7 +4,7 @@
 // (measured: 18.4 against 0.62 T per second). A thread forms 8 consecutive outputs of one line from
 // the window of 8 + 2 H inputs they read. It scales the window by one power of two (that of its
 // largest entry) to integers below 2^57 and splits each into two limbs of 29 bits; the operator's
-// entries are kept as two limbs of integers below 2^58, one scale per 8 rows. A product of two
+// entries are kept as two limbs of integers below 2^58, one scale per row. A product of two
 // such pairs takes three multiply-adds, xh ch and xh cl + xl ch, into two 64-bit sums that cannot
 // overflow (13 terms); xl cl, below 2^-58 of the largest product, is dropped. The sum is rounded
 // to a double once, where an FMA chain rounds at every term (host emulation, 9 and 18 terms: rms
@@ -26,11 +26,9 @@
 namespace shp {
 namespace {
 
-constexpr int kBandLimb = 29, kBandXBits = 57;
-
 struct FixBandOp {
   const int4* tab;   // [segment][8 rows][band_row]: {hi, lo, hi, lo} of entries 2 q, 2 q + 1
-  const int* ex;     // scale of each segment
+  const int* ex;     // scale of row r of segment seg at r segs + seg
   const int* w0;     // rectangular bands (H = 0): first input of each segment's window
   const double* val;    // the band in doubles (windows that cannot be scaled): row i's entries from
   const int* start;     // input start[i]
@@ -61,116 +59,6 @@ struct FixBandBatch {
   int njobs;
 };
 
-__device__ __forceinline__ void band_mad(long long& c, int a, int b) {
-  c += (long long)a * b;
-}
-
-// The window's exponent (the biased one of its largest entry; -1 if all are zero; slow set when it
-// cannot be scaled) and its entries as limbs: x / 2^(exponent - 1022) 2^57 rounded to
-// hi 2^29 + lo, |lo| <= 2^28.
-template <int N>
-__device__ __forceinline__ int band_limbs(const double (&x)[N], int2 (&v)[N], bool& slow) {
-  unsigned key = 0, low = 0;   // key: the largest exponent and leading bits, one place to the left
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    key = max(key, (unsigned)__double2hiint(x[k]) << 1);
-    low |= (unsigned)__double2loint(x[k]);
-  }
-  const int e = (int)(key >> 21);
-  const bool zero = (key | low) == 0;
-  slow = slow || (!zero && (e < (int)kFixMinExp || e > (int)kFixMaxExp));
-  const int top = zero ? 4000 : 62 - kBandXBits + e;   // (4000: everything shifts out)
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const unsigned hi = (unsigned)__double2hiint(x[k]), lo = (unsigned)__double2loint(x[k]);
-    // the significand with its leading one at bit 62 (an entry without one shifts out)
-    const unsigned long long n =
-        ((unsigned long long)__funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 10) << 32) |
-        (lo << 10);
-    // one bit more than kept, then rounded (truncated entries would all err towards zero, and that
-    // smooth error is what the preconditioner amplifies), the low limb of either sign
-    const int sh = min(top - (int)((hi >> 20) & 0x7ffu), 63);
-    const unsigned long long t = (n >> sh) + (1ull << kBandLimb) + 1;
-    const int h = (int)(t >> (kBandLimb + 1));
-    const int l = (int)((unsigned)(t >> 1) - (1u << (kBandLimb - 1)) - ((unsigned)h << kBandLimb));
-    const int sg = (int)hi >> 31;
-    v[k].x = (h ^ sg) - sg;
-    v[k].y = (l ^ sg) - sg;
-  }
-  return zero ? -1 : e;
-}
-
-// Row r of the segment times the window, in units of 2^58 of the product of the two scales, plus hh.
-template <int H, int N>
-__device__ __forceinline__ long long band_row_dot(const int4* c, const int2 (&v)[N], int r,
-                                                  long long hh = 0) {
-  long long md = 1ll << (kBandLimb - 1);
-  const int k0 = H ? r : 0;
-#pragma unroll
-  for (int q = 0; q < band_row(H); ++q) {
-    const int4 w = c[r * band_row(H) + q];
-    const int2 a = v[k0 + 2 * q];
-    band_mad(hh, a.x, w.x);
-    band_mad(md, a.x, w.y);
-    band_mad(md, a.y, w.x);
-    if (H == 0 || q < H) {   // (entry 2 H + 1 is padding)
-      const int2 b = v[k0 + 2 * q + 1];
-      band_mad(hh, b.x, w.z);
-      band_mad(md, b.x, w.w);
-      band_mad(md, b.y, w.z);
-    }
-  }
-  return hh + (md >> kBandLimb);
-}
-
-// Scale of a window of zeros (below every other) and from scales to the exponent of a result.
-constexpr int kNoScale = -(1 << 20);
-constexpr int kBandShift = 2 * kBandLimb - 1022 - kBandXBits;
-
-// The outputs 8 seg .. 8 seg + 7 of one line. load(t, x): the window of term t; c: the operators'
-// limbs of the segment, cstep int4 apart; ex: their scales, estep apart; put(y, r, value): output r
-// of Y (y = 0) or Y2 (1). Returns false, without outputs, if a window cannot be scaled.
-// ready(): called once the first window is scaled, before the limbs and scales are read.
-template <int H, int NT, bool DUAL, typename Load, typename Ready, typename Put>
-__device__ __forceinline__ bool band_outputs(const int4* c, int cstep, const int* ex, int estep,
-                                             Load&& load, Ready&& ready, Put&& put) {
-  constexpr int N = kR + 2 * H;
-  bool slow = false;
-  int2 v[N];
-  long long s[kR];   // NT = 2: the first term's sums
-  int es = 0, e = 0;
-#pragma unroll
-  for (int t = 0; t < NT; ++t) {
-    double x[N];
-    load(t, x);
-    e = band_limbs<N>(x, v, slow);
-    if (t == 0) ready();
-    const int en = e < 0 ? kNoScale : e + ex[t * estep];
-    if (t + 1 < NT) {
-      es = en;
-#pragma unroll
-      for (int r = 0; r < kR; ++r) s[r] = band_row_dot<H, N>(c, v, r);
-      c += cstep;
-      continue;
-    }
-    if (slow) return false;
-    // both sums at the larger of the two scales
-    const int top = NT > 1 ? max(es, en) : en;
-    const int da = min(top - es, 62), db = min(top - en, 62);
-    const long long ha = (1ll << da) >> 1, hb = (1ll << db) >> 1;   // half a unit, if shifted
-    const int e2 = DUAL ? (e < 0 ? kNoScale : e + ex[NT * estep]) : 0;
-#pragma unroll
-    for (int r = 0; r < kR; ++r) {
-      long long y = band_row_dot<H, N>(c, v, r, NT > 1 ? hb : 0);
-      if (NT > 1) y = ((s[r] + ha) >> da) + (y >> db);
-      put(0, r, fix_to_double(y, top + kBandShift));
-      if (DUAL)
-        put(1, r, fix_to_double(band_row_dot<H, N>(c + cstep, v, r), e2 + kBandShift));
-    }
-  }
-  return true;
-}
-
 // The same outputs by FMA chains over the bands; at(t, j): entry j of term t's line of m entries.
 template <typename At, typename Put>
 __device__ __forceinline__ void band_chains(const FixBandJob& J, int seg, int m, At&& at,
@@ -198,13 +86,13 @@ __device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4
   constexpr int N = kR + 2 * H, kSegIn = kR * band_row(H), kOps = NT + (DUAL ? 1 : 0);
   const int tid = threadIdx.x, nth = blockDim.x;
   const int lb = local / J.segs, seg = local - lb * J.segs;
-  int* es = reinterpret_cast<int*>(sh + kOps * kSegIn);
+  int* es = reinterpret_cast<int*>(sh + kOps * kSegIn);   // [kOps][8]
   // (the operators are written once at setup: their copy does not wait for the preceding kernel)
 #pragma unroll
   for (int o = 0; o < kOps; ++o) {
     for (int w = tid; w < kSegIn; w += nth)
       sh[o * kSegIn + w] = __ldg(J.D[o].tab + (int64_t)seg * kSegIn + w);
-    if (tid == o) es[o] = __ldg(J.D[o].ex + seg);
+    if (tid < kR) es[kR * o + tid] = __ldg(J.D[o].ex + tid * J.segs + seg);
   }
   pdl_begin();
   const int n1 = J.in.n1, n12 = n1 * J.in.n2;
@@ -257,7 +145,7 @@ __device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4
     (y ? J.Y2 : J.Y)[o] = v;
   };
   const bool done = band_outputs<H, NT, DUAL>(
-      sh, kSegIn, es, 1,
+      sh, kSegIn, [&](int o, int r) { return es[kR * o + r]; },
       [&](int t, double (&x)[N]) {
         if constexpr (H == 0) {
           const int w0 = __ldg(J.D[t].w0 + seg);
@@ -294,15 +182,14 @@ __device__ __forceinline__ void band_stage_zero(double* raw, int nl, int m, int 
   }
 }
 
-// the limbs of all segments of one operator (pitch band_seg), and the scales
+// the limbs of all segments of one operator (pitch band_seg)
 template <int H>
-__device__ __forceinline__ void band_stage_op(const FixBandOp& D, int segs, int4* sh, int* es) {
+__device__ __forceinline__ void band_stage_op(const FixBandOp& D, int segs, int4* sh) {
   constexpr int kSegIn = kR * band_row(H);
   for (int idx = threadIdx.x; idx < segs * kSegIn; idx += blockDim.x) {
     const int sg = idx / kSegIn;
     sh[sg * band_seg(H) + idx - sg * kSegIn] = __ldg(D.tab + idx);
   }
-  for (int sg = threadIdx.x; sg < segs; sg += blockDim.x) es[sg] = __ldg(D.ex + sg);
 }
 
 // A pass along x1: the block takes whole lines, staged in shared memory with their results, one
@@ -314,12 +201,11 @@ __device__ __forceinline__ void band_along(const FixBandJob& J, int local, int4*
   const int segs = J.segs, m = J.in.n1, lines1 = J.in.n2 * J.in.n3;
   const int lpb = nth / segs, line0 = local * lpb, nl = min(lpb, lines1 * J.nb - line0);
   const int S = band_stage_s(segs, H);
-  int* es = reinterpret_cast<int*>(sh + kOps * segs * band_seg(H));
-  double* raw = reinterpret_cast<double*>(es + ((kOps * segs + 1) & ~1));   // [NT][lpb][8 S]
+  double* raw = reinterpret_cast<double*>(sh + kOps * segs * band_seg(H));   // [NT][lpb][8 S]
   double* out = raw + NT * lpb * kR * S;                                    // [1 or 2][lpb][8 S]
 #pragma unroll
   for (int o = 0; o < kOps; ++o)
-    band_stage_op<H>(J.D[o], segs, sh + o * segs * band_seg(H), es + o * segs);
+    band_stage_op<H>(J.D[o], segs, sh + o * segs * band_seg(H));
 #pragma unroll
   for (int t = 0; t < NT; ++t) band_stage_zero<H>(raw + t * lpb * kR * S, nl, m, segs, S);
   auto line_of = [&](int idx) -> int {   // idx / m
@@ -350,7 +236,8 @@ __device__ __forceinline__ void band_along(const FixBandJob& J, int local, int4*
     double* q = out + l * kR * S + seg;
     auto put = [&](int y, int r, double v) { q[(y ? lpb * kR * S : 0) + r * S] = v; };
     const bool done = band_outputs<H, NT, DUAL>(
-        sh + seg * band_seg(H), segs * band_seg(H), es + seg, segs,
+        sh + seg * band_seg(H), segs * band_seg(H),
+        [&](int o, int r) { return __ldg(J.D[o].ex + r * segs + seg); },
         [&](int t, double (&x)[N]) {
 #pragma unroll
           for (int k = 0; k < N; ++k) x[k] = p[t * lpb * kR * S + (k & 7) * S + (k >> 3)];
@@ -425,10 +312,9 @@ __global__ void __launch_bounds__(256, 2) k_fix_div_x1(const double* __restrict_
   const int nv = q ? 2 : 1;
   const int segs = J.segs, lpb = nth / (segs * nv), m = b, S = band_stage_s(segs, H);
   const int lines = b * b, line0 = (int)blockIdx.x * lpb, nl = min(lpb, lines - line0);
-  int* es = reinterpret_cast<int*>(shb + segs * band_seg(H));
-  double* raw = reinterpret_cast<double*>(es + ((segs + 1) & ~1));   // delta, then e
+  double* raw = reinterpret_cast<double*>(shb + segs * band_seg(H));   // delta, then e
   double* out = raw + nv * lpb * kR * S;
-  band_stage_op<H>(J.D[0], segs, shb, es);
+  band_stage_op<H>(J.D[0], segs, shb);
   band_stage_zero<H>(raw, nv * lpb, m, segs, S);
   pdl_begin();
   const int64_t b2 = (int64_t)b * b;
@@ -459,7 +345,7 @@ __global__ void __launch_bounds__(256, 2) k_fix_div_x1(const double* __restrict_
     double* y = out + row * kR * S + seg;
     auto put = [&](int, int r, double v) { y[r * S] = v; };
     const bool done = band_outputs<H, 1, false>(
-        shb + seg * band_seg(H), 0, es + seg, 0,
+        shb + seg * band_seg(H), 0, [&](int, int r) { return __ldg(J.D[0].ex + r * segs + seg); },
         [&](int, double (&x)[N]) {
 #pragma unroll
           for (int k = 0; k < N; ++k) x[k] = p[(k & 7) * S + (k >> 3)];
@@ -555,7 +441,7 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
     threads = std::max(threads, band_threads(jobs[j].block, jobs[j].axis == 1
                                                                ? band_segs(jobs[j].D0.rows)
                                                                : 1));
-  int blocks = 0, smem = 3 * kR * band_row(H) * 16 + 16;
+  int blocks = 0, smem = 3 * kR * (band_row(H) * 16 + 4);   // (passes along x2 and x3)
   bool epi = false;
   int nt = 1;
   double flops = 0, bytes = 0;

@@ -1,10 +1,86 @@
 // Host entry points to the rules, tables and arithmetic of the fixed-point FP64 passes, for
 // test_fix_host.py (compiled with the host compiler).
+#include <cmath>
+
 #include "fix_tables.h"
 
 using namespace shp;
 
+namespace {
+// One line of m entries through the passes of the library's 1D matrices: y = D0 x0 (+ D1 x1), and
+// with a third matrix y2 = D2 x(last).
+template <int H, int NT, bool DUAL>
+void line(const BandLimbs* t, int m, const double* const* x, double* y, double* y2) {
+  const int segs = band_segs(m);
+  constexpr int per = kR * band_row(H);
+  for (int seg = 0; seg < segs; ++seg) {
+    int4 c[3 * per];
+    for (int o = 0; o < NT + (DUAL ? 1 : 0); ++o)
+      for (int w = 0; w < per; ++w) {
+        const int* v = &t[o].tab[((size_t)seg * per + w) * 4];
+        c[o * per + w] = int4{v[0], v[1], v[2], v[3]};
+      }
+    const bool done = band_outputs<H, NT, DUAL>(
+        c, per, [&](int o, int r) { return t[o].ex[r * segs + seg]; },
+        [&](int k, double (&w)[kR + 2 * H]) {
+          for (int j = 0; j < kR + 2 * H; ++j) {
+            const int i = kR * seg + j - H;
+            w[j] = i >= 0 && i < m ? x[k][i] : 0.0;
+          }
+        },
+        [] {},
+        [&](int q, int r, double v) {
+          if (kR * seg + r < m) (q ? y2 : y)[kR * seg + r] = v;
+        });
+    if (!done)
+      for (int r = 0; r < kR && kR * seg + r < m; ++r) {
+        y[kR * seg + r] = NAN;
+        if (DUAL) y2[kR * seg + r] = NAN;
+      }
+  }
+}
+
+Dense matrix(const Univariate& u, int which) {
+  return which == 0 ? u.M : (which == 1 ? u.K : (which == 2 ? u.Mc : u.Tc));
+}
+}  // namespace
+
 extern "C" {
+// Dense row-major copies of the bands (M, K: a x a; M-check, T-check: b x b) that the passes of n
+// elements of degree p take, into val (nmat of them, one after the other), and the passes' results
+// for `lines` lines of x0 (and x1); nterms and results as in line(). Returns the half width.
+int band_lines(int n, int p, int nterms, int results, const int* which, double* val, int lines,
+               const double* x0, const double* x1, double* y, double* y2) {
+  const Univariate u = build_univariate(n, p, 14.0);
+  const int nops = nterms + results - 1, H = p + 1;
+  BandLimbs t[3];
+  int m = 0;
+  for (int o = 0; o < nops; ++o) {
+    const Band b = to_band(matrix(u, which[o]), 1e-15);
+    m = b.rows;
+    t[o] = band_limbs_square(b, H);
+    for (int i = 0; i < m; ++i)
+      for (int w = 0; w < b.width; ++w)
+        val[((size_t)o * m + i) * m + b.start[i] + w] = b.val[(size_t)i * b.width + w];
+  }
+  for (int l = 0; l < lines; ++l) {
+    const double* x[2] = {x0 + (size_t)l * m, x1 ? x1 + (size_t)l * m : nullptr};
+    double *r = y + (size_t)l * m, *r2 = y2 ? y2 + (size_t)l * m : nullptr;
+#define LINE(h)                                                                      \
+  case h:                                                                            \
+    if (nterms == 1 && results == 1) line<h, 1, false>(t, m, x, r, r2);              \
+    if (nterms == 1 && results == 2) line<h, 1, true>(t, m, x, r, r2);               \
+    if (nterms == 2 && results == 1) line<h, 2, false>(t, m, x, r, r2);              \
+    if (nterms == 2 && results == 2) line<h, 2, true>(t, m, x, r, r2);               \
+    break;
+    switch (H) {
+      LINE(2) LINE(3) LINE(4) LINE(5) LINE(6)
+      default: return -1;
+    }
+  }
+  return H;
+}
+
 int fits(int b, int H) { return fix_band_fits(b, H); }
 long long along_smem(int nops, int nline, int segs, int H) {
   return band_along_smem(nops, nline, segs, H);

@@ -1,6 +1,7 @@
 """Rules, tables and arithmetic of the fixed-point FP64 passes (csrc/fix.h, csrc/fix_band.h), which
 compile for the host: no GPU needed."""
 import ctypes
+import math
 import os
 import shutil
 import subprocess
@@ -51,8 +52,8 @@ def test_banded_passes_that_do_not_fit_are_not_offered(lib, H):
                                                       lines * (nterms + results), segs, H))
         assert offered == (largest <= limit), (b, H, largest)
     assert seen == {True, False}
-    # the sizes that a set-up used to fail at
-    for b, half in ((489, 6), (585, 5), (673, 4), (881, 3), (1265, 2)):
+    # far above the line
+    for b, half in ((700, 6), (700, 5), (800, 4), (1000, 3), (1400, 2)):
         assert not lib.fits(b, half)
 
 
@@ -92,3 +93,82 @@ def test_rectangular_tables_need_windows_of_eight(lib):
     args = [_ptr(val), _ptr(w0), _ptr(dense)]
     assert lib.rect_pair(rows, cols, width, _ptr(a), args[0], _ptr(b), *args) == 0
     assert lib.rect_pair(rows, cols, width, _ptr(a), args[0], _ptr(a + 4), *args) == 1
+
+
+M, K, MC, TC = range(4)
+
+
+def _band_lines(lib, n, p, ops, x, results=1):
+    """Results of the passes of the matrices `ops` for lines of x (one array per term), and the
+    matrices."""
+    nterms, (lines, m) = len(x), x[0].shape
+    val = np.zeros((len(ops), m, m))
+    y = [np.zeros((lines, m)) for _ in range(results)]
+    x = [np.ascontiguousarray(t) for t in x]
+    assert lib.band_lines(n, p, nterms, results, _ptr(np.array(ops, np.int32)), _ptr(val), lines,
+                          _ptr(x[0]), _ptr(x[1]) if nterms > 1 else None, _ptr(y[0]),
+                          _ptr(y[1]) if results > 1 else None) == p + 1
+    return val, y
+
+
+def _units(D, x, y, rows):
+    """Error of y against sum_t D_t x_t in units of 2^-53 sum_t |D_t| |x_t|, for the given rows. The
+    exact sums by math.fsum of exact products (each product as its rounding and fma remainder)."""
+    worst = 0.0
+    for l in range(y.shape[0]):
+        for i in rows:
+            terms, size = [], 0.0
+            for Dt, xt in zip(D, x):
+                for j in np.flatnonzero(Dt[i]):
+                    terms += _product(float(Dt[i, j]), float(xt[l, j]))
+                    size += abs(Dt[i, j] * xt[l, j])
+            if size:
+                worst = max(worst, abs(math.fsum(terms + [-float(y[l, i])])) / size * 2.0 ** 53)
+    return worst
+
+
+def _product(a, b):
+    """a b as two doubles, by Dekker's splitting."""
+    p = a * b
+    ah = a * 134217729.0
+    ah -= ah - a
+    bh = b * 134217729.0
+    bh -= bh - b
+    al, bl = a - ah, b - bh
+    return [p, ((ah * bh - p) + ah * bl + al * bh) + al * bl]
+
+
+# the 1D matrices alone, then the forms of the operator's passes: two results of one input (K and M;
+# T-check and M-check), two terms (M-check and T-check), two terms with two results
+FORMS = [([M], 1), ([K], 1), ([MC], 1), ([TC], 1), ([K, M], 2), ([TC, MC], 2), ([MC, TC], 1),
+         ([MC, TC, MC], 2)]
+
+
+def _form(n, p, ops, results, rng, lines):
+    nterms = len(ops) - results + 1
+    m = n + p - (1 if ops[0] in (M, K) else 0)
+    return [rng.uniform(0.5, 1.0, (lines, m)) * rng.choice([-1.0, 1.0], (lines, m))
+            for _ in range(nterms)]
+
+
+def _outputs(D, x, y):
+    """(matrices, inputs, result) of each result of a pass."""
+    nterms = len(x)
+    out = [(D[:nterms], x, y[0])]
+    if len(y) > 1:
+        out.append((D[nterms:], x[-1:], y[1]))
+    return out
+
+
+@pytest.mark.parametrize("n,p", [(60, 1), (61, 2), (64, 3), (64, 4), (60, 5)])
+@pytest.mark.parametrize("ops,results", FORMS)
+def test_rows_beside_the_walls_keep_their_accuracy(lib, n, p, ops, results):
+    """Every output of a pass, the small rows beside T-check's penalty row above all, is as close as
+    an FMA chain is bound to be: 2^-53 per term, of sum |D| |x| over its own row. Entries of one
+    magnitude, so that only the scales of the rows count."""
+    x = _form(n, p, ops, results, np.random.default_rng(n + p), 40)
+    D, y = _band_lines(lib, n, p, ops, x, results)
+    m = D.shape[1]
+    for Dt, xt, yt in _outputs(D, x, y):
+        rows = [*range(16), m // 2, m // 2 + 1, *range(m - 16, m)]
+        assert _units(Dt, xt, yt, rows) <= sum((np.count_nonzero(d, axis=1).max()) for d in Dt)
