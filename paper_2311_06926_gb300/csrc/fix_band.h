@@ -40,17 +40,25 @@ constexpr bool fix_band_fits(int b, int H) {
 }
 
 // ---- arithmetic -------------------------------------------------------------------------------
-constexpr int kBandLimb = 29, kBandXBits = 57;   // bits of a limb, of a scaled window entry
+// bits of a limb and of a scaled window entry: two terms of 13 products of hi limbs, 2^29 by 2^29,
+// stay below 2^63
+constexpr int kBandLimb = 29, kBandXBits = 58;
 
 SHP_HD void band_mad(long long& c, int a, int b) {
   c += (long long)a * b;
 }
 
+// Row r of a segment weighs the 5 entries around its centre (H = 1: 3; rectangular: the whole
+// window). first: the first of them in the window; words of four entries, two per row, from
+// first / 4 on.
+SHP_HD constexpr int band_first(int H, int r) { return H ? r + (H > 2 ? H - 2 : 0) : 0; }
+SHP_HD constexpr int band_words(int H) { return band_first(H, H ? kR - 1 : 0) / 4 + 2; }
+
 // The window's exponent (the biased one of its largest entry; -1 if all are zero; slow set when it
-// cannot be scaled) and its entries as limbs: x / 2^(exponent - 1022) 2^57 rounded to
-// hi 2^29 + lo, |lo| <= 2^28.
-template <int N>
-SHP_HD int band_limbs(const double (&x)[N], int2 (&v)[N], bool& slow) {
+// cannot be scaled), its entries as limbs: x / 2^(exponent - 1022) 2^58 rounded to
+// hi 2^29 + lo, |lo| <= 2^28, and their magnitudes in 128ths of the scale, four to a word.
+template <int N, int NW>
+SHP_HD int band_limbs(const double (&x)[N], int2 (&v)[N], unsigned (&mag)[NW], bool& slow) {
   unsigned key = 0, low = 0;   // key: the largest exponent and leading bits, one place to the left
 #pragma unroll
   for (int k = 0; k < N; ++k) {
@@ -58,6 +66,8 @@ SHP_HD int band_limbs(const double (&x)[N], int2 (&v)[N], bool& slow) {
     key = m > key ? m : key;
     low |= lo_word(x[k]);
   }
+#pragma unroll
+  for (int w = 0; w < NW; ++w) mag[w] = 0;
   const int e = (int)(key >> 21);
   const bool zero = (key | low) == 0;
   slow = slow || (!zero && (e < (int)kFixMinExp || e > (int)kFixMaxExp));
@@ -75,11 +85,43 @@ SHP_HD int band_limbs(const double (&x)[N], int2 (&v)[N], bool& slow) {
     const unsigned long long t = (n >> sh) + (1ull << kBandLimb) + 1;
     const int h = (int)(t >> (kBandLimb + 1));
     const int l = (int)((unsigned)(t >> 1) - (1u << (kBandLimb - 1)) - ((unsigned)h << kBandLimb));
+    if (k < 4 * NW) mag[k / 4] |= (unsigned)(h >> (kBandXBits - kBandLimb - 7)) << (8 * (k % 4));
     const int sg = (int)hi >> 31;
     v[k].x = (h ^ sg) - sg;
     v[k].y = (l ^ sg) - sg;
   }
   return zero ? -1 : e;
+}
+
+// sum of the products of the bytes of a and b, plus c
+SHP_HD unsigned dot_bytes(unsigned a, unsigned b, unsigned c) {
+#ifdef __CUDA_ARCH__
+  return __dp4a(a, b, c);
+#else
+  for (int k = 0; k < 32; k += 8) c += (a >> k & 255u) * (b >> k & 255u);
+  return c;
+#endif
+}
+
+// Rows whose own entries are too small for the scales of the window and the row (weak rows), bit
+// 7 - r: the sum of the products of the weighed magnitudes (rounded down: a lower bound of
+// sum |D| |x|) is below 2^-6 of the product of the scales. Above that line the roundings at the
+// common scale, about 2^-59 of it, stay below those of an FMA chain over the row: host emulation,
+// p = 1 .. 4, lines that are normal, spiked or geometric (factors 4 and 10): rms 0.26 to 0.46 units of
+// 2^-53 sum |D| |x|, at most 2.2, against 0.42 to 0.85 and 5.6. (At 2^-7 0.58 and 4.1.) Weighing all
+// rows before the products costs about 10% of a launch; within their loop its registers spilled.
+constexpr unsigned kBandWeak = 1u << (7 + 8 - 6);
+template <int H, int NW, typename Row>
+SHP_HD unsigned band_weak(const unsigned (&mag)[NW], Row&& row, int o) {
+  unsigned weak = 0;
+#pragma unroll
+  for (int r = 0; r < kR; ++r) {
+    const int4 w = row(o, r);
+    const int m = band_first(H, r) / 4;
+    const unsigned s = dot_bytes(mag[m], (unsigned)w.x, 0u - kBandWeak);
+    weak = funnel_left(dot_bytes(mag[m + 1], (unsigned)w.y, s), weak, 1);   // (its sign bit)
+  }
+  return weak;
 }
 
 // Row r of the segment times the window, in units of 2^58 of the product of the two scales, plus hh.
@@ -109,23 +151,32 @@ constexpr int kNoScale = -(1 << 20);
 constexpr int kBandShift = 2 * kBandLimb - 1022 - kBandXBits;
 
 // The outputs 8 seg .. 8 seg + 7 of one line. load(t, x): the window of term t; c: the operators'
-// limbs of the segment, cstep int4 apart; ex(o, r): scale of row r of operator o; put(y, r, value):
-// output r of Y (y = 0) or Y2 (1). Returns false, without outputs, if a window cannot be scaled.
+// limbs of the segment, cstep int4 apart; row(o, r): weights and scale of row r of operator o
+// (BandLimbs); put(y, r, value): output r of Y (y = 0) or Y2 (1). Returns the outputs that are left
+// to FMA chains, bit 7 - r (Y) and 15 - r (Y2): all if a window cannot be scaled, else those of weak
+// rows (of either term). ONCE: these are not put before; else they may be, and are put again.
 // ready(): called once the first window is scaled, before the limbs and scales are read.
-template <int H, int NT, bool DUAL, typename Ex, typename Load, typename Ready, typename Put>
-SHP_HD bool band_outputs(const int4* c, int cstep, Ex&& ex, Load&& load, Ready&& ready,
-                         Put&& put) {
-  constexpr int N = kR + 2 * H;
+template <int H, int NT, bool DUAL, bool ONCE, typename Row, typename Load, typename Ready,
+          typename Put>
+SHP_HD unsigned band_outputs(const int4* c, int cstep, Row&& row, Load&& load, Ready&& ready,
+                             Put&& put) {
+  constexpr int N = kR + 2 * H, NW = band_words(H);
   bool slow = false;
   int2 v[N];
   long long s[kR];   // NT = 2: the first term's sums
   int e0 = 0, e = 0;
+  unsigned weak = 0, weak2 = 0;
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
     double x[N];
+    unsigned mag[NW];
     load(t, x);
-    e = band_limbs<N>(x, v, slow);
+    e = band_limbs<N, NW>(x, v, mag, slow);
     if (t == 0) ready();
+    if (e >= 0) {   // (a window of zeros is exact at any scale)
+      weak |= band_weak<H, NW>(mag, row, t);
+      if (DUAL && t + 1 == NT) weak2 = band_weak<H, NW>(mag, row, NT);
+    }
     if (t + 1 < NT) {
       e0 = e;
 #pragma unroll
@@ -133,14 +184,14 @@ SHP_HD bool band_outputs(const int4* c, int cstep, Ex&& ex, Load&& load, Ready&&
       c += cstep;
       continue;
     }
-    if (slow) return false;
+    if (slow) return DUAL ? 0xffffu : 0xffu;
 #pragma unroll
     for (int r = 0; r < kR; ++r) {
-      int top = e < 0 ? kNoScale : e + ex(t, r);
+      int top = e < 0 ? kNoScale : e + row(t, r).z;
       long long y;
       if (NT > 1) {
         // both sums at the larger of the two scales, half a unit added to one that is shifted
-        const int en = top, es = e0 < 0 ? kNoScale : e0 + ex(0, r);
+        const int en = top, es = e0 < 0 ? kNoScale : e0 + row(0, r).z;
         top = es > en ? es : en;
         const int da = top - es < 62 ? top - es : 62, db = top - en < 62 ? top - en : 62;
         y = band_row_dot<H, N>(c, v, r, (1ll << db) >> 1);
@@ -148,14 +199,13 @@ SHP_HD bool band_outputs(const int4* c, int cstep, Ex&& ex, Load&& load, Ready&&
       } else {
         y = band_row_dot<H, N>(c, v, r);
       }
-      put(0, r, fix_to_double(y, top + kBandShift));
-      if (DUAL) {
-        const int e2 = e < 0 ? kNoScale : e + ex(NT, r);
-        put(1, r, fix_to_double(band_row_dot<H, N>(c + cstep, v, r), e2 + kBandShift));
-      }
+      if (!ONCE || !(weak >> (kR - 1 - r) & 1u)) put(0, r, fix_to_double(y, top + kBandShift));
+      if (DUAL)
+        put(1, r, fix_to_double(band_row_dot<H, N>(c + cstep, v, r),
+                                (e < 0 ? kNoScale : e + row(NT, r).z) + kBandShift));
     }
   }
-  return true;
+  return weak | weak2 << kR;
 }
 
 }  // namespace shp

@@ -107,7 +107,7 @@ struct BandCore {
 // rectangular (half = 0) with the first input of each 8-row segment in w0.
 struct BandFix {
   const int4* tab;
-  const int* ex;
+  const int4* rows;   // weights and scale of each row
   const int* w0;
   int half;
 };

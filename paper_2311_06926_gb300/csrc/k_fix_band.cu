@@ -3,17 +3,22 @@
 // GB300 runs 64 32 x 32 + 64-bit integer multiply-adds per clock and SM against 2 FP64 FMAs
 // (measured: 18.4 against 0.62 T per second). A thread forms 8 consecutive outputs of one line from
 // the window of 8 + 2 H inputs they read. It scales the window by one power of two (that of its
-// largest entry) to integers below 2^57 and splits each into two limbs of 29 bits; the operator's
+// largest entry) to integers below 2^58 and splits each into two limbs of 29 bits; the operator's
 // entries are kept as two limbs of integers below 2^58, one scale per row. A product of two
 // such pairs takes three multiply-adds, xh ch and xh cl + xl ch, into two 64-bit sums that cannot
 // overflow (13 terms); xl cl, below 2^-58 of the largest product, is dropped. The sum is rounded
-// to a double once, where an FMA chain rounds at every term (host emulation, 9 and 18 terms: rms
-// error 0.3 to 0.5 of the chain's). The window is what the scale is taken over, so an entry loses
-// precision only against entries that meet it in the same outputs.
+// to a double once, where an FMA chain rounds at every term.
 //
-// Bound by instruction issue: about 125 instructions per result, of which the 27 multiply-adds of a
-// row of 9 take twice their slots. Measured against the FMA passes: K apply 1052 -> 530 us at 128^3
-// p = 3, 150 -> 83 at 64^3.
+// The scale is that of a window's largest entry, which not every row of the segment reads, and the
+// row's scale that of its largest coefficient, which may meet a small entry. So every output is
+// weighed: where its own sum |D| |x| is too far below the product of the scales (band_weak), its
+// thread forms it by an FMA chain as well and stores that. Every output is as close as a chain
+// then: its error is relative to its own terms, not to the window (1e-4 to 1.6e-3 of the outputs are
+// left to chains for lines of normal entries).
+//
+// Bound by instruction issue: about 140 instructions per result, of which the 27 multiply-adds of a
+// row of 9 take twice their slots. Measured against the FMA passes: K apply 1052 -> 616 us at 128^3
+// p = 3 (533 without weighing and chains), 61^3 p = 2 81, 48^3 p = 3 65 (70 and 50 without).
 //
 // A window with an infinity or a NaN, or outside [2^-823, 2^777], takes FMA chains instead.
 #include <algorithm>
@@ -28,11 +33,13 @@ namespace {
 
 struct FixBandOp {
   const int4* tab;   // [segment][8 rows][band_row]: {hi, lo, hi, lo} of entries 2 q, 2 q + 1
-  const int* ex;     // scale of row r of segment seg at r segs + seg
+  const int4* rows;  // weights and scale of row r of segment seg at r segs + seg
   const int* w0;     // rectangular bands (H = 0): first input of each segment's window
-  const double* val;    // the band in doubles (windows that cannot be scaled): row i's entries from
-  const int* start;     // input start[i]
-  int width;
+  // the band in doubles (outputs left to FMA chains): row i's `width` entries at val + i pitch, from
+  // input start[i] or, start null, i - half
+  const double* val;
+  const int* start;
+  int width, pitch, half;
 };
 
 struct FixBandJob {
@@ -59,24 +66,98 @@ struct FixBandBatch {
   int njobs;
 };
 
-// The same outputs by FMA chains over the bands; at(t, j): entry j of term t's line of m entries.
+// position of entry j - H of a staged line (fix_band.h)
+__device__ __forceinline__ int band_stage(int j, int S) { return (j & 7) * S + (j >> 3); }
+
+// Outputs left to FMA chains (band_outputs): at(t, j): entry j of term t's line of nin entries. Few
+// threads come here; what they cost is latency, so nothing is looked up before the operands.
 template <typename At, typename Put>
-__device__ __forceinline__ void band_chains(const FixBandJob& J, int seg, int m, At&& at,
-                                            Put&& put) {
-#pragma unroll 1
-  for (int r = 0; r < kR && kR * seg + r < m; ++r) {
-    const int i = kR * seg + r;
+__device__ __forceinline__ void band_chains(const FixBandJob& J, int seg, int m, int nin,
+                                            unsigned redo, At&& at, Put&& put) {
+  const int rows = min(m - kR * seg, kR);
+  redo &= (0xff00u >> rows & 0xffu) * 0x101u;
+  while (redo) {
+    const int bit = __ffs(redo) - 1, r = kR - 1 - bit % kR, i = kR * seg + r;
+    redo &= redo - 1;
+    const int o0 = bit < kR ? 0 : J.nterms, o1 = bit < kR ? J.nterms : J.nops;
     double y = 0.0;
 #pragma unroll 1
-    for (int o = 0; o < J.nops; ++o) {
+    for (int o = o0; o < o1; ++o) {
       const FixBandOp& D = J.D[o];
-      if (o == J.nterms) y = 0.0;
-#pragma unroll 1
-      for (int k = 0; k < D.width; ++k)
-        y = fma(D.val[(int64_t)i * D.width + k], at(min(o, J.nterms - 1), D.start[i] + k), y);
-      if (o + 1 >= J.nterms) put(o + 1 - J.nterms, r, y);
+      const int t = min(o, J.nterms - 1);
+      const int j0 = D.start ? D.start[i] : i - D.half;   // input of the row's first entry
+      const int k0 = max(0, -j0), k1 = min(D.width, nin - j0);
+      const double* d = D.val + (int64_t)i * D.pitch;
+#pragma unroll 4
+      for (int k = k0; k < k1; ++k) y = fma(d[k], at(t, j0 + k), y);
+    }
+    put(bit / kR, r, y);
+  }
+}
+
+// The segment of a thread of a pass along x2 or x3 (block `local` of the job).
+struct BandPlace {
+  int64_t first, at0;   // entry 0 of the line and output 0 of the segment
+  int64_t kb;           // offset of the line's item
+  int i1, q;            // x1 index, and x3 (axis 2) or x2 index
+  int stride, i0, m, rows;   // rows: of the segment to write
+};
+__device__ __forceinline__ BandPlace band_place(const FixBandJob& J, int local) {
+  BandPlace p;
+  const int lb = local / J.segs, seg = local - lb * J.segs;
+  const int n1 = J.in.n1, n12 = n1 * J.in.n2;
+  const bool ax2 = J.axis == 2;
+  const int lines1 = ax2 ? n1 * J.in.n3 : n12;
+  int line = lb * (int)blockDim.x + (int)threadIdx.x;
+  const bool on = line < lines1 * J.nb;
+  if (!on) line = 0;
+  p.kb = 0;
+  if (J.nb > 1) {
+    const int k = line / lines1;
+    p.kb = (int64_t)k * J.bs;
+    line -= k * lines1;
+  }
+  p.q = n1 == 1 ? line : (int)(__umulhi((unsigned)line, J.n1_mul) >> J.n1_sh);
+  p.i1 = line - p.q * n1;
+  p.first = p.kb + (ax2 ? p.i1 + (int64_t)n12 * p.q : (int64_t)line);
+  p.stride = ax2 ? n1 : n12;
+  p.i0 = kR * seg;
+  p.m = J.rows;
+  p.rows = on ? p.m - p.i0 : 0;
+  // (a rectangular pass along x2 has result planes of another size)
+  p.at0 = (ax2 ? p.kb + p.i1 + (int64_t)n1 * p.m * p.q : p.first) + (int64_t)p.stride * p.i0;
+  return p;
+}
+
+// Stores output r of the segment: a result, or with EPI what the job makes of it.
+template <bool EPI>
+__device__ __forceinline__ void band_put(const FixBandJob& J, const BandPlace& p, int y, int r,
+                                         double v) {
+  if (r >= p.rows) return;
+  const int64_t o = p.at0 + (int64_t)p.stride * r;
+  if (EPI) {
+    if (J.g) {
+      const bool ax2 = J.axis == 2;
+      const int gstride = ax2 ? J.gd1 : J.gd12;
+      const int gstep = J.gaxis == 1 ? 1 : (J.gaxis == 2 ? J.gd1 : J.gd12);
+      const double* g = J.g + p.kb + p.i1 + (int64_t)(ax2 ? J.gd12 : J.gd1) * p.q +
+                        (int64_t)gstride * (p.i0 + r);
+      v += g[0] - g[gstep];
+    }
+    if (J.hmode == 1) {
+      const double xi = J.hx[o], ri = xi - v;
+      J.hr[o] = ri;
+      J.hacc[o] = xi + ri;
+      return;
+    }
+    if (J.hmode == 2) {
+      const double ri = J.hr[o] - v;
+      J.hr[o] = ri;
+      J.hacc[o] += ri;
+      return;
     }
   }
+  (y ? J.Y2 : J.Y)[o] = v;
 }
 
 // A pass along x2 or x3: the block takes one segment of blockDim neighbouring lines, so every load
@@ -86,91 +167,43 @@ __device__ __forceinline__ void band_across(const FixBandJob& J, int local, int4
   constexpr int N = kR + 2 * H, kSegIn = kR * band_row(H), kOps = NT + (DUAL ? 1 : 0);
   const int tid = threadIdx.x, nth = blockDim.x;
   const int lb = local / J.segs, seg = local - lb * J.segs;
-  int* es = reinterpret_cast<int*>(sh + kOps * kSegIn);   // [kOps][8]
+  int4* rw = sh + kOps * kSegIn;   // [kOps][8]
   // (the operators are written once at setup: their copy does not wait for the preceding kernel)
 #pragma unroll
   for (int o = 0; o < kOps; ++o) {
     for (int w = tid; w < kSegIn; w += nth)
       sh[o * kSegIn + w] = __ldg(J.D[o].tab + (int64_t)seg * kSegIn + w);
-    if (tid < kR) es[kR * o + tid] = __ldg(J.D[o].ex + tid * J.segs + seg);
+    if (tid < kR) rw[kR * o + tid] = __ldg(J.D[o].rows + tid * J.segs + seg);
   }
   pdl_begin();
-  const int n1 = J.in.n1, n12 = n1 * J.in.n2;
-  const bool ax2 = J.axis == 2;
-  const int nin = ax2 ? J.in.n2 : J.in.n3, m = H ? nin : J.rows;
-  const int lines1 = ax2 ? n1 * J.in.n3 : n12;
-  int line = lb * nth + tid;
-  const bool on = line < lines1 * J.nb;
-  if (!on) line = 0;
-  int64_t kb = 0;   // offset of the line's item
-  if (J.nb > 1) {
-    const int k = line / lines1;
-    kb = (int64_t)k * J.bs;
-    line -= k * lines1;
-  }
-  const int q =
-      n1 == 1 ? line : (int)(__umulhi((unsigned)line, J.n1_mul) >> J.n1_sh);   // x3 (axis 2) or x2 index
-  const int i1 = line - q * n1;
-  const int64_t first = kb + (ax2 ? i1 + (int64_t)n12 * q : (int64_t)line);
-  const int stride = ax2 ? n1 : n12;
-  const int i0 = kR * seg;
-  // the segment's outputs (a rectangular pass along x2 has planes of another size)
-  const int64_t at0 = (H == 0 && ax2 ? kb + i1 + (int64_t)n1 * m * q : first) + (int64_t)stride * i0;
-  const double* g = nullptr;
-  int gstride = 0, gstep = 0;
-  if (EPI && J.g) {
-    gstride = ax2 ? J.gd1 : J.gd12;
-    gstep = J.gaxis == 1 ? 1 : (J.gaxis == 2 ? J.gd1 : J.gd12);
-    g = J.g + kb + i1 + (int64_t)(ax2 ? J.gd12 : J.gd1) * q + (int64_t)gstride * i0;
-  }
-  const int rows = on ? m - i0 : 0;   // rows of the segment to write
-  auto put = [&](int y, int r, double v) {
-    if (r >= rows) return;
-    const int64_t o = at0 + (int64_t)stride * r;
-    if (EPI) {
-      if (J.g) v += g[gstride * r] - g[gstride * r + gstep];
-      if (J.hmode == 1) {
-        const double xi = J.hx[o], ri = xi - v;
-        J.hr[o] = ri;
-        J.hacc[o] = xi + ri;
-        return;
-      }
-      if (J.hmode == 2) {
-        const double ri = J.hr[o] - v;
-        J.hr[o] = ri;
-        J.hacc[o] += ri;
-        return;
-      }
-    }
-    (y ? J.Y2 : J.Y)[o] = v;
-  };
-  const bool done = band_outputs<H, NT, DUAL>(
-      sh, kSegIn, [&](int o, int r) { return es[kR * o + r]; },
+  const BandPlace p = band_place(J, local);
+  const int64_t stride = p.stride;
+  auto put = [&](int y, int r, double v) { band_put<EPI>(J, p, y, r, v); };
+  const unsigned redo = band_outputs<H, NT, DUAL, EPI>(
+      sh, kSegIn, [&](int o, int r) { return rw[kR * o + r]; },
       [&](int t, double (&x)[N]) {
         if constexpr (H == 0) {
-          const int w0 = __ldg(J.D[t].w0 + seg);
-          const double* p = J.X[t] + first + (int64_t)stride * w0;
+          const int w0 = __ldg(J.D[t].w0 + seg), nin = J.axis == 2 ? J.in.n2 : J.in.n3;
+          const double* x0 = J.X[t] + p.first + stride * w0;
 #pragma unroll
-          for (int k = 0; k < N; ++k) x[k] = w0 + k < nin ? p[(int64_t)stride * k] : 0.0;
+          for (int k = 0; k < N; ++k) x[k] = w0 + k < nin ? x0[stride * k] : 0.0;
           return;
         }
-        const double* p = J.X[t] + at0;
-        if (i0 >= H && i0 + kR + H <= m) {
+        const double* x0 = J.X[t] + p.at0;
+        if (p.i0 >= H && p.i0 + kR + H <= p.m) {
 #pragma unroll
-          for (int k = 0; k < N; ++k) x[k] = p[(int64_t)stride * (k - H)];
+          for (int k = 0; k < N; ++k) x[k] = x0[stride * (k - H)];
         } else {
 #pragma unroll
           for (int k = 0; k < N; ++k)
-            x[k] = i0 + k >= H && i0 + k < m + H ? p[(int64_t)stride * (k - H)] : 0.0;
+            x[k] = p.i0 + k >= H && p.i0 + k < p.m + H ? x0[stride * (k - H)] : 0.0;
         }
       },
       [] { __syncthreads(); }, put);
-  if (!done && on)
-    band_chains(J, seg, m, [&](int t, int j) { return J.X[t][first + (int64_t)stride * j]; }, put);
+  if (redo && p.rows > 0)
+    band_chains(J, seg, p.m, J.axis == 2 ? J.in.n2 : J.in.n3, redo,
+                [&](int t, int j) { return J.X[t][p.first + stride * j]; }, put);
 }
-
-// position of entry j - H of a staged line (fix_band.h)
-__device__ __forceinline__ int band_stage(int j, int S) { return (j & 7) * S + (j >> 3); }
 
 // zeros around the m entries of nl staged lines
 template <int H>
@@ -235,16 +268,16 @@ __device__ __forceinline__ void band_along(const FixBandJob& J, int local, int4*
     const double* p = raw + l * kR * S + seg;
     double* q = out + l * kR * S + seg;
     auto put = [&](int y, int r, double v) { q[(y ? lpb * kR * S : 0) + r * S] = v; };
-    const bool done = band_outputs<H, NT, DUAL>(
+    const unsigned redo = band_outputs<H, NT, DUAL, false>(
         sh + seg * band_seg(H), segs * band_seg(H),
-        [&](int o, int r) { return __ldg(J.D[o].ex + r * segs + seg); },
+        [&](int o, int r) { return __ldg(J.D[o].rows + r * segs + seg); },
         [&](int t, double (&x)[N]) {
 #pragma unroll
           for (int k = 0; k < N; ++k) x[k] = p[t * lpb * kR * S + (k & 7) * S + (k >> 3)];
         },
         [] {}, put);
-    if (!done)
-      band_chains(J, seg, m,
+    if (redo)
+      band_chains(J, seg, m, m, redo,
                   [&](int t, int j) { return raw[(t * lpb + l) * kR * S + band_stage(j + H, S)]; },
                   put);
   }
@@ -344,15 +377,15 @@ __global__ void __launch_bounds__(256, 2) k_fix_div_x1(const double* __restrict_
     const double* p = raw + row * kR * S + seg;
     double* y = out + row * kR * S + seg;
     auto put = [&](int, int r, double v) { y[r * S] = v; };
-    const bool done = band_outputs<H, 1, false>(
-        shb + seg * band_seg(H), 0, [&](int, int r) { return __ldg(J.D[0].ex + r * segs + seg); },
+    const unsigned redo = band_outputs<H, 1, false, false>(
+        shb + seg * band_seg(H), 0, [&](int, int r) { return __ldg(J.D[0].rows + r * segs + seg); },
         [&](int, double (&x)[N]) {
 #pragma unroll
           for (int k = 0; k < N; ++k) x[k] = p[(k & 7) * S + (k >> 3)];
         },
         [] {}, put);
-    if (!done)
-      band_chains(J, seg, m,
+    if (redo)
+      band_chains(J, seg, m, m, redo,
                   [&](int, int j) { return raw[row * kR * S + band_stage(j + H, S)]; }, put);
   }
   __syncthreads();
@@ -365,7 +398,8 @@ __global__ void __launch_bounds__(256, 2) k_fix_div_x1(const double* __restrict_
 }
 
 FixBandOp band_op(const BandCore<double>& D, const BandFix& f) {
-  return FixBandOp{f.tab, f.ex, f.w0, D.val, D.start, D.width};
+  if (f.half == 0) return FixBandOp{f.tab, f.rows, f.w0, D.val, D.start, D.width, D.width, 0};
+  return FixBandOp{f.tab, f.rows, nullptr, D.cval, nullptr, 2 * D.half + 1, D.cpitch, D.half};
 }
 
 void band_divisor(int n1, FixBandJob& J) {
@@ -441,7 +475,7 @@ void fix_band_multi(const PassArgs<double>* jobs, int njobs, cudaStream_t s) {
     threads = std::max(threads, band_threads(jobs[j].block, jobs[j].axis == 1
                                                                ? band_segs(jobs[j].D0.rows)
                                                                : 1));
-  int blocks = 0, smem = 3 * kR * (band_row(H) * 16 + 4);   // (passes along x2 and x3)
+  int blocks = 0, smem = 3 * kR * (band_row(H) + 1) * 16;   // (passes along x2 and x3)
   bool epi = false;
   int nt = 1;
   double flops = 0, bytes = 0;

@@ -184,14 +184,14 @@ BandD<T> upload_band(Arena& ar, const Band& b, cudaStream_t s, int min_half = 0)
 
 BandFix upload_limbs(Arena& ar, const BandLimbs& t, int H, cudaStream_t s) {
   std::vector<int> all(t.tab);   // the 16-byte words of the limbs first
-  all.insert(all.end(), t.ex.begin(), t.ex.end());
+  all.insert(all.end(), t.rows.begin(), t.rows.end());
   all.insert(all.end(), t.w0.begin(), t.w0.end());
   int* d = ar.alloc<int>(all.size());
   ck(cudaMemcpyAsync(d, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, s), "fix");
   ck(cudaStreamSynchronize(s), "fix");
-  const int* ex = d + t.tab.size();
-  return BandFix{reinterpret_cast<const int4*>(d), ex, t.w0.empty() ? nullptr : ex + t.ex.size(),
-                 H};
+  const int* rows = d + t.tab.size();
+  return BandFix{reinterpret_cast<const int4*>(d), reinterpret_cast<const int4*>(rows),
+                 t.w0.empty() ? nullptr : rows + t.rows.size(), H};
 }
 
 // The fixed-point form of a square band, centred with half width H (none if the band is wider)

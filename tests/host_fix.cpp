@@ -20,8 +20,12 @@ void line(const BandLimbs* t, int m, const double* const* x, double* y, double* 
         const int* v = &t[o].tab[((size_t)seg * per + w) * 4];
         c[o * per + w] = int4{v[0], v[1], v[2], v[3]};
       }
-    const bool done = band_outputs<H, NT, DUAL>(
-        c, per, [&](int o, int r) { return t[o].ex[r * segs + seg]; },
+    const unsigned redo = band_outputs<H, NT, DUAL, false>(
+        c, per,
+        [&](int o, int r) {
+          const int* v = &t[o].rows[((size_t)r * segs + seg) * 4];
+          return int4{v[0], v[1], v[2], v[3]};
+        },
         [&](int k, double (&w)[kR + 2 * H]) {
           for (int j = 0; j < kR + 2 * H; ++j) {
             const int i = kR * seg + j - H;
@@ -32,11 +36,10 @@ void line(const BandLimbs* t, int m, const double* const* x, double* y, double* 
         [&](int q, int r, double v) {
           if (kR * seg + r < m) (q ? y2 : y)[kR * seg + r] = v;
         });
-    if (!done)
-      for (int r = 0; r < kR && kR * seg + r < m; ++r) {
-        y[kR * seg + r] = NAN;
-        if (DUAL) y2[kR * seg + r] = NAN;
-      }
+    for (int r = 0; r < kR && kR * seg + r < m; ++r) {   // outputs left to FMA chains
+      if (redo >> (kR - 1 - r) & 1) y[kR * seg + r] = NAN;
+      if (redo >> (2 * kR - 1 - r) & 1) y2[kR * seg + r] = NAN;
+    }
   }
 }
 
@@ -47,8 +50,9 @@ Dense matrix(const Univariate& u, int which) {
 
 extern "C" {
 // Dense row-major copies of the bands (M, K: a x a; M-check, T-check: b x b) that the passes of n
-// elements of degree p take, into val (nmat of them, one after the other), and the passes' results
-// for `lines` lines of x0 (and x1); nterms and results as in line(). Returns the half width.
+// elements of degree p take, into val (one after the other), and the passes' results for `lines`
+// lines of x0 (and x1), NaN where an output is left to an FMA chain; nterms and results as in
+// line(). Returns the half width.
 int band_lines(int n, int p, int nterms, int results, const int* which, double* val, int lines,
                const double* x0, const double* x1, double* y, double* y2) {
   const Univariate u = build_univariate(n, p, 14.0);
@@ -109,7 +113,8 @@ int rect_pair(int rows, int cols, int width, const int* start0, const double* va
       for (int i = kR * sg; i < rows && i < kR * sg + kR; ++i)
         for (int k = 0; k < 8; ++k) {
           const int* v = &t[o].tab[((size_t)i * 8 + k) * 2];
-          const double x = std::ldexp((double)v[0] * 0x1p29 + v[1], t[o].ex[sg]);
+          const int ex = t[o].rows[((size_t)(i % kR) * band_segs(rows) + sg) * 4 + 2];
+          const double x = std::ldexp((double)v[0] * 0x1p29 + v[1], ex);
           if (t[o].w0[sg] + k < cols) dense[((size_t)o * rows + i) * cols + t[o].w0[sg] + k] = x;
           else if (x != 0) return -1;
         }

@@ -122,7 +122,7 @@ def _units(D, x, y, rows):
                 for j in np.flatnonzero(Dt[i]):
                     terms += _product(float(Dt[i, j]), float(xt[l, j]))
                     size += abs(Dt[i, j] * xt[l, j])
-            if size:
+            if size and not np.isnan(y[l, i]):
                 worst = max(worst, abs(math.fsum(terms + [-float(y[l, i])])) / size * 2.0 ** 53)
     return worst
 
@@ -172,3 +172,33 @@ def test_rows_beside_the_walls_keep_their_accuracy(lib, n, p, ops, results):
     for Dt, xt, yt in _outputs(D, x, y):
         rows = [*range(16), m // 2, m // 2 + 1, *range(m - 16, m)]
         assert _units(Dt, xt, yt, rows) <= sum((np.count_nonzero(d, axis=1).max()) for d in Dt)
+
+
+def _wide(name, rng, lines, m):
+    x = rng.standard_normal((lines, m))
+    if name == "spike":
+        x[np.arange(lines), rng.integers(0, m, lines)] *= 1e6
+    elif name == "falls by 4":
+        x *= 4.0 ** -(np.arange(m) % 40)
+    elif name == "rises by 10":
+        x *= 10.0 ** (np.arange(m) % 13)
+    elif name == "steps":
+        x *= np.where(np.arange(m) // 5 % 2, 1.0, 1e-9)
+    return x
+
+
+@pytest.mark.parametrize("n,p", [(60, 1), (61, 2), (64, 3), (64, 4), (60, 5)])
+@pytest.mark.parametrize("ops,results", FORMS)
+@pytest.mark.parametrize("kind", ["normal", "spike", "falls by 4", "rises by 10", "steps"])
+def test_entries_do_not_lose_bits_to_larger_neighbours(lib, n, p, ops, results, kind):
+    """Lines of wide range: every output that the fixed-point form keeps is as close as an FMA chain
+    is bound to be, 2^-53 per term of sum |D| |x| over its own row (the others it leaves to a
+    chain). Of lines of one magnitude it keeps nearly all."""
+    rng = np.random.default_rng(7 * n + p)
+    x = [_wide(kind, rng, 12, t.shape[1]) for t in _form(n, p, ops, results, rng, 12)]
+    D, y = _band_lines(lib, n, p, ops, x, results)
+    for Dt, xt, yt in _outputs(D, x, y):
+        bound = sum((np.count_nonzero(d, axis=1).max()) for d in Dt)
+        assert _units(Dt, xt, yt, range(D.shape[1])) <= bound
+        if kind == "normal":
+            assert np.isnan(yt).mean() < 0.03

@@ -12,6 +12,7 @@ import torch
 from paper_2311_06926_gb300 import Stokes, synthetic
 
 from gpu_common import dev, host, oracle, relerr
+from oracle.matfree import kron3_apply
 
 pytestmark = pytest.mark.gpu
 
@@ -133,4 +134,63 @@ def test_quadrature_segment_edges(n, p, nu):
         assert relerr(host(G.apply_K(dev(x))), ref) < 1e-12
     for e in (-900, 800):   # windows that cannot be scaled take chains
         assert relerr(np.ldexp(host(G.apply_K(dev(x) * 2.0 ** e)), -e), ref) < 1e-12
+    G.close()
+
+
+def _wide_vector(G, seed):
+    """Entries of wide range next to each other: steps of 2^-20 along x1, a fall by 4 per entry along
+    x2 (12 entries, then again), single entries 1e6 times their neighbours."""
+    rng = np.random.default_rng(seed)
+    a, b = G.a, G.b
+    out = []
+    for e1, e2, e3 in ((a, b, b), (b, a, b), (b, b, a), (b, b, b)):
+        t = rng.standard_normal((e3, e2, e1))
+        t *= np.where(np.arange(e1) // 5 % 2, 1.0, 2.0 ** -20)
+        t *= (4.0 ** -(np.arange(e2) % 12))[:, None]
+        spikes = rng.integers(0, t.size, 200)
+        t.reshape(-1)[spikes] *= 1e6
+        out.append(t.reshape(-1))
+    return np.concatenate(out)
+
+
+@pytest.mark.parametrize("n,p,nu", [(45, 1, 1.0), (44, 2, 0.3), (43, 3, 2.0), (42, 4, 1.0),
+                                    (41, 5, 1.0)])
+def test_operator_entries_keep_their_own_accuracy(n, p, nu):
+    """K x entry by entry against the FMA chains, which the same vector times 2^900 takes: each path
+    rounds an entry at most once per term of its passes (six sums of at most 2 p + 3 terms, and the
+    divergence), relative to the sum of the magnitudes of the entry's own products."""
+    S, _, _, _ = oracle(n, p, nu)
+    G = Stokes(n, p, nu=nu, max_order=2, max_steps=0, autotune=False)
+    x = _wide_vector(G, n)
+    m, k, nv = S.uv, kron3_apply, G.n_vel
+    M, K, Mc, Tc = (np.abs(t) for t in (m.M, m.K, m.Mc, m.Tc))
+    sizes = [(G.b, G.b, G.a), (G.b, G.a, G.b), (G.a, G.b, G.b)]
+    u = [np.abs(t).reshape(s) for t, s in zip(np.split(x[:nv], 3), sizes)]
+    q = np.abs(x[nv:]).reshape(G.b, G.b, G.b)
+    delta = sum(np.pad(t, [(0, 1) if d == ax else (0, 0) for d in range(3)])
+                + np.pad(t, [(1, 0) if d == ax else (0, 0) for d in range(3)])
+                for t, ax in zip(u, (2, 1, 0)))
+    g = k(Mc, Mc, Mc, nu * delta + q)
+    size = []
+    for c, t in enumerate(u):
+        own, other = (K, M), (Mc, Tc)
+        A = 0
+        for at in range(3):   # the direction that carries K (own) or T-check (another one)
+            D = []
+            for d in range(3):
+                pair = own if d == c else other
+                hit = d == at
+                D.append(pair[0] if (hit == (d == c)) else pair[1])
+            A = A + (2 if at != c else 1) * nu * k(D[2], D[1], D[0], t)
+        ax = 2 - c
+        size.append((A + g[tuple(slice(0, -1) if d == ax else slice(None) for d in range(3))]
+                     + g[tuple(slice(1, None) if d == ax else slice(None) for d in range(3))])
+                    .reshape(-1))
+    size = np.concatenate(size + [k(Mc, Mc, Mc, delta).reshape(-1)])
+    bound = 2.0 * (6 * (2 * p + 3) + 16) * 2.0 ** -53
+    for block in (128, 256):
+        G.set_tuning(512, block, 0)
+        y = host(G.apply_K(dev(x)))
+        z = np.ldexp(host(G.apply_K(dev(np.ldexp(x, 900)))), -900)
+        assert (np.abs(y - z) / size).max() < bound
     G.close()
