@@ -6,14 +6,20 @@
 // entry) to integers, those of an operator column to integers below 2^58, and each integer is
 // written in six balanced digits of ten bits, sum_i d_i 2^(50 - 10 i), |d_i| <= 512, which FP16
 // holds exactly. Products of digits are exact in the tensor cores, and the 21 digit pairs with
-// i + j <= 5 are summed by level l = i + j in FP32. Level 2 is moved to an integer after every 32
-// terms and all levels after every 80 (input integers below 2^57: folded entries and modes) or
-// 64 (below 2^58: plain matrices). Levels 0 to 2 then stay below 2^24 whatever the digits, since
-// |d_0| <= 2^7 or 2^8 and <= 2^8; the higher levels do too unless nearly all digits are extreme,
-// and a rounding there is below 2^-52 of the largest sum. The integer result is rounded to a
-// double once, where an FMA chain rounds at every term. The dropped pairs (i + j >= 6) and the
-// scaling leave an error below that of the FMA chain (host emulation, 9 to 66 terms, rms over
-// random, decaying and smooth lines: 0.2 to 0.56 of the chain's).
+// i + j <= 5 are summed by level l = i + j in FP32, which holds integers up to 2^24. The levels are
+// moved to integers before they can pass that, whatever the digits (fix_every, fix_peak): 3 after
+// every step of 16 terms, 2 after two, 0 and 1 after five (input integers below 2^57: folded entries
+// and modes) or four (below 2^58: plain matrices). Lines and columns of equal entries do reach the
+// bounds: level 3 over 66 equal terms passed 2^24 for one pair of values in twenty when it was moved
+// every five steps, and truncated sums cost 2^-48 of the result. Level 4, in units of the result,
+// may reach 2^25 over its two steps and lose its last bit; level 5 stays until the end and loses
+// less than 2^-4 of a unit. (The moves cost 1% of P_0^-1 at 128^3: 906 -> 915 us; with 64-bit sums
+// in place of the moved integers 974 to 994.) The integer result is rounded to a double once, where
+// an FMA chain rounds at every term. The dropped pairs (i + j >= 6) and the scaling leave an error
+// below that of the FMA chain (host emulation, 9 to 66 terms, rms over random, decaying and smooth
+// lines: 0.2 to 0.56 of the chain's). Splitting products into slices that the matrix unit sums
+// exactly follows Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication", 2012.
 //
 // The integer sums do not depend on the tile or the kernel that forms them, so every launch form
 // gives the same bits.
@@ -38,6 +44,27 @@ constexpr int kFixSlices = 6, kFixDigit = 10;
 // bits of a scaled operator entry, and of the sum of an output's operator magnitudes: the 64-bit
 // sums, in units of 2^60, stay below 2^62
 constexpr int kFixUBits = 58, kFixSumBits = 63, kFixUnit = 60;
+
+// Steps of 16 terms after which level l's sums are moved, for input integers below 2^xbits, and the
+// largest sum they can reach by then (leading digits are smaller than the others).
+SHP_HD constexpr int fix_drain(int xbits) { return xbits == 58 ? 4 : 5; }
+SHP_HD constexpr int fix_every(int l, int xbits) {
+  return l == 2 || l == 4 ? 2 : (l == 3 ? 1 : fix_drain(xbits));
+}
+constexpr int64_t fix_digit_max(int i, int bits) {
+  return 1ll << (i ? kFixDigit - 1 : bits - kFixDigit * (kFixSlices - 1));
+}
+constexpr int64_t fix_peak(int l, int xbits) {
+  int64_t sum = 0;
+  for (int i = 0; i <= l; ++i) sum += fix_digit_max(i, xbits) * fix_digit_max(l - i, kFixUBits);
+  return 16 * fix_every(l, xbits) * sum;
+}
+constexpr bool fix_exact(int xbits) {
+  for (int l = 0; l < 4; ++l)
+    if (fix_peak(l, xbits) > 1 << 24) return false;
+  return fix_peak(4, xbits) <= 1 << 25;
+}
+static_assert(fix_exact(56) && fix_exact(57) && fix_exact(58), "level sums must stay exact");
 
 // One direction of a parity-split operator (host_setup.h, generalized_eigh_parity) as digit slices
 // in the operand order of mma.sync m16n8k16: half `par` (0: even terms, 1: odd terms), 8 outputs

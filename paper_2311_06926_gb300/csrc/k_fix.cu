@@ -32,7 +32,8 @@ struct FixOp {
 FixOp fix_op(const FixTabs& f, const double* U, int K, int he, int use) {
   return FixOp{use == kFixBackward ? f.bw : f.fw, U, K, use == kFixPlain ? K : he,
                use == kFixForward, use == kFixPlain ? 1 : 2,
-               use == kFixPlain ? 58 : (use == kFixBackward ? 57 : 56), use == kFixPlain ? 4 : 5};
+               use == kFixPlain ? 58 : (use == kFixBackward ? 57 : 56),
+               fix_drain(use == kFixPlain ? 58 : 57)};
 }
 
 // uint4 entries of the line operand: the halves of mt tiles of 16 lines
@@ -49,6 +50,15 @@ __device__ __forceinline__ void fix_mma(float (&c)[4], const uint4& a, unsigned 
       "{%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+// the product alone
+__device__ __forceinline__ void fix_mma0(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1), "f"(0.f));
 }
 
 // a b + c
@@ -71,13 +81,13 @@ __device__ __forceinline__ void fix_gemm(const FixOp& op, const uint4* xf, int m
 #pragma unroll
   for (int c = 0; c < 3; ++c) b[c] = __ldg(bp + 32 * c);
   float acc[kFixSlices][4];
-  int i2[4];
+  int i2[4], i3[4], i4[4];   // moved sums of levels 2, 3, 4
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
 #pragma unroll
     for (int l = 0; l < kFixSlices; ++l) acc[l][r] = 0.f;
     s1[r] = 0;
-    i2[r] = 0;
+    i2[r] = i3[r] = i4[r] = 0;
   }
   const int total = op.halves * ks;
   int left = min(ks, op.drain);   // steps until the levels are added up
@@ -95,29 +105,36 @@ __device__ __forceinline__ void fix_gemm(const FixOp& op, const uint4* xf, int m
     for (int i = 0; i < kFixSlices; ++i) {
       const uint4 a = ap[i * 32];
 #pragma unroll
-      for (int j = 0; i + j < kFixSlices; ++j) fix_mma(acc[i + j], a, bw[j][0], bw[j][1]);
+      for (int j = 0; i + j < kFixSlices; ++j) {
+        // (level 3 is moved after every step)
+        if (i == 0 && j == 3) fix_mma0(acc[j], a, bw[j][0], bw[j][1]);
+        else fix_mma(acc[i + j], a, bw[j][0], bw[j][1]);
+      }
     }
     ap += kFixSlices * 32;
     --left;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) i3[r] += __float2int_rn(acc[3][r]);
     if (left == 0) {
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        const int a5 = __float2int_rn(acc[5][r]), a4 = __float2int_rn(acc[4][r]);
+        const int a5 = __float2int_rn(acc[5][r]), a4 = i4[r] + __float2int_rn(acc[4][r]);
         long long v = s1[r] + (a4 + ((a5 + (1 << (kFixDigit - 1))) >> kFixDigit));
-        v = mad_wide(__float2int_rn(acc[3][r]), 1 << kFixDigit, v);
+        v = mad_wide(i3[r], 1 << kFixDigit, v);
         v = mad_wide(i2[r] + __float2int_rn(acc[2][r]), 1 << (2 * kFixDigit), v);
         v = mad_wide(__float2int_rn(acc[1][r]), 1 << (3 * kFixDigit), v);
         s1[r] = v + ((long long)__float2int_rn(acc[0][r]) << (4 * kFixDigit));
 #pragma unroll
         for (int l = 0; l < kFixSlices; ++l) acc[l][r] = 0.f;
-        i2[r] = 0;
+        i2[r] = i3[r] = i4[r] = 0;
       }
       left = min(it + 1 < ks ? ks - it - 1 : (it + 1 == ks ? ks : 2 * ks - it - 1), op.drain);
     } else if (((op.drain - left) & 1) == 0) {   // 32 terms
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         i2[r] += __float2int_rn(acc[2][r]);
-        acc[2][r] = 0.f;
+        i4[r] += __float2int_rn(acc[4][r]);
+        acc[2][r] = acc[4][r] = 0.f;
       }
     }
     if (it + 1 == ks) {   // the even half is complete

@@ -85,6 +85,9 @@ int band_lines(int n, int p, int nterms, int results, const int* which, double* 
   return H;
 }
 
+// steps between the moves of a level's sums
+int level_every(int level, int xbits) { return fix_every(level, xbits); }
+
 int fits(int b, int H) { return fix_band_fits(b, H); }
 long long along_smem(int nops, int nline, int segs, int H) {
   return band_along_smem(nops, nline, segs, H);

@@ -202,3 +202,36 @@ def test_entries_do_not_lose_bits_to_larger_neighbours(lib, n, p, ops, results, 
         assert _units(Dt, xt, yt, range(D.shape[1])) <= bound
         if kind == "normal":
             assert np.isnan(yt).mean() < 0.03
+
+
+def _digits(v):
+    """Balanced digits of ten bits, the leading one first (weight 2^50)."""
+    out = []
+    for _ in range(6):
+        d = (v + 512) % 1024 - 512
+        out.append(d)
+        v = (v - d) >> 10
+    return out[::-1]
+
+
+@pytest.mark.parametrize("xbits", [56, 57, 58])
+def test_level_sums_of_equal_entries_stay_exact(lib, xbits):
+    """FP32 holds the integer sums of a level exactly up to 2^24. Lines and columns of equal entries
+    (their digits too) reach the largest sums; the levels above the result's unit must be moved
+    before, level 4 (the unit) may lose its last bit, and the last level's truncations stay below
+    a unit."""
+    rng = np.random.default_rng(xbits)
+    pairs = [(int(rng.integers(2 ** (xbits - 1), 2 ** xbits)), int(rng.integers(2 ** 57, 2 ** 58)))
+             for _ in range(2000)]
+    # and the largest digits of one sign
+    low = sum(511 << (10 * k) for k in range(5))
+    pairs += [(2 ** xbits - 2 ** 50 + low, 2 ** 58 - 2 ** 50 + low)]
+    for v, u in pairs:
+        dv, du = _digits(v), _digits(u)
+        for level in range(6):
+            term = sum(dv[i] * du[level - i] for i in range(level + 1))
+            peak = abs(term) * 16 * lib.level_every(level, xbits)
+            if level < 5:
+                assert peak <= 2 ** (24 if level < 4 else 25), (level, v, u)
+            else:   # units of 2^50 against the result's 2^60
+                assert 5 * 2 ** max(0, peak.bit_length() - 24) < 2 ** 10
