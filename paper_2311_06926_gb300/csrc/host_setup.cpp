@@ -385,10 +385,9 @@ bool generalized_eigh_parity(const Dense& K, const Dense& M, std::vector<double>
   return true;
 }
 
-bool banded_inverse(const Dense& A, int p, Dense& inv, Dense& low) {
+bool banded_cholesky(const Dense& A, int p, std::vector<double>& lb) {
   const int n = A.rows, w = p + 1;
-  // L(i, k) at lb[i * w + (k - i + p)] for i - p <= k <= i
-  std::vector<double> lb((size_t)n * w, 0.0);
+  lb.assign((size_t)n * w, 0.0);
   auto L = [&](int i, int k) -> double& { return lb[(size_t)i * w + (k - i + p)]; };
   for (int j = 0; j < n; ++j) {
     double d = A(j, j);
@@ -401,6 +400,12 @@ bool banded_inverse(const Dense& A, int p, Dense& inv, Dense& low) {
       L(i, j) = t / L(j, j);
     }
   }
+  return true;
+}
+
+void banded_inverse(const Dense& A, int p, const std::vector<double>& lb, Dense& inv, Dense& low) {
+  const int n = A.rows, w = p + 1;
+  auto L = [&](int i, int k) { return lb[(size_t)i * w + (k - i + p)]; };
   auto solve = [&](std::vector<double>& v) {
     for (int i = 0; i < n; ++i) {
       double t = v[i];
@@ -436,7 +441,6 @@ bool banded_inverse(const Dense& A, int p, Dense& inv, Dense& low) {
       low(i, c) = r[i] - (inv(i, c) - x[i]);
     }
   }
-  return true;
 }
 
 Band to_band(const Dense& D, double drop_tol) {

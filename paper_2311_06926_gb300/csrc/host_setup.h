@@ -61,10 +61,13 @@ bool generalized_eigh(const Dense& K, const Dense& M, std::vector<double>& lam, 
 bool generalized_eigh_parity(const Dense& K, const Dense& M, std::vector<double>& lam, Dense& U,
                              int* he);
 
-// Inverse of a symmetric positive definite matrix of half bandwidth p by banded Cholesky, each
-// column refined once with a residual in twice the working precision: inv + low, low the part
-// of the refined entries that doubles lose. Returns false if A is not positive definite.
-bool banded_inverse(const Dense& A, int p, Dense& inv, Dense& low);
+// Cholesky factor of a symmetric positive definite matrix of half bandwidth p: L(i, k) at
+// lb[i (p + 1) + (k - i + p)] for i - p <= k <= i. Returns false if A is not positive definite.
+bool banded_cholesky(const Dense& A, int p, std::vector<double>& lb);
+
+// Its inverse by that factor, each column refined once with a residual in twice the working
+// precision: inv + low, low the part of the refined entries that doubles lose.
+void banded_inverse(const Dense& A, int p, const std::vector<double>& lb, Dense& inv, Dense& low);
 
 Band to_band(const Dense& D, double drop_tol);
 

@@ -315,6 +315,34 @@ template <typename T>
 void div_band_x1(const T* u1, const T* u2, const T* u3, int a, int b, const T* q, T nu,
                  const BandD<T>& D, T* y0, T* y1, cudaStream_t s);
 
+// Banded Cholesky solves along one direction of a (b, b, b) tensor: y <- post (L L^T)^-1 x (y may
+// be x) with L lower triangular of bandwidth p stored as rows lb[i * (p + 1) + (k - i + p)] for
+// k in [i - p, i], and inv_diag[i] = 1 / L[i][i] (pressure mass inverse). nb items, item k of x and
+// y at k * bs entries. Returns the launch status.
+template <typename T>
+cudaError_t chol_solve_axis(const T* x, T* y, int b, int p, int axis, const T* lb,
+                            const T* inv_diag, T post, cudaStream_t s, int nb = 1,
+                            int64_t bs = 0);
+constexpr int kCholLines = 32;   // lines per block
+// shared memory of a block: its lines, the factor and the reciprocal diagonal
+constexpr int64_t chol_smem(int b, int p) {
+  return (int64_t)b * (kCholLines + 1 + p + 1 + 1) * (int64_t)sizeof(double);
+}
+// Whether the pressure block takes these solves; below the line, long lines take the dense inverse in
+// slices. The solves' errors are relative to an entry's own neighbourhood. The slices' are relative
+// to the largest entry of a line, which the inverse hardly couples to distant ones: an entry 1e6
+// times the others costs those up to 1e6 units of rounding (checking every output and forming the
+// weak ones by chains: 32^3 p = 3 MINRES solve 13.8 -> 16.5 ms, 64^3 gradient 46 -> 65). Shorter
+// lines take the slices all the same, because the products by eigenvectors, their other fast form,
+// are no better there (host emulation, b = 34, normal and spiked lines: rms 2000 and 73000 units
+// against 0.4 and 12500) and one serial chain per line takes longest against them. us, solves :
+// slices: P_0^-1 64^3 p = 3 200 : 133, 96^3 p = 2 342 : 372, 128^3 p = 3 847 : 911; order-3, 1-step
+// preconditioner 96^3 p = 2 2122 : 2136; order-2, 2-step 64^3 p = 4 1516 : 1155.
+constexpr int kCholMin = 64;
+constexpr bool chol_route(int b, int p) {
+  return b >= kCholMin && chol_smem(b, p) <= 227 * 1024;
+}
+
 // ---- vector kernels (k_vec.cu) -----------------------------------------------------------
 // Deterministic dot product: fixed grid, fixed-order tree reduction. Result written to *out
 // (device). `partials` holds kDotBlocks values and, in the word after them, a completion counter

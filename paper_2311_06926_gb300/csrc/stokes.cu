@@ -337,6 +337,9 @@ struct Ops {
                              // with this many blocks per plane (0: six single-direction passes)
   FixTabs fx_Minv;           // FP64: M-check^-1 in slices (plain; null for short lines),
   const T* Minv = nullptr;   // and in doubles
+  const T* chol_lb = nullptr;          // FP64: banded Cholesky factor of M-check (long lines)
+  const T* chol_inv = nullptr;
+  int chol_p = 0;
   T *tK = nullptr, *tM = nullptr, *tS = nullptr, *tR = nullptr;   // component-size temporaries
   T *f1 = nullptr, *f2 = nullptr;                                 // mode-product ping-pong
   T *delta = nullptr, *m1 = nullptr, *m2 = nullptr;               // pressure-size temporaries
@@ -819,10 +822,20 @@ struct Ops {
 
   // pressure block: y = 2 nu (M-check^-1)^(x)3 x = 2 nu (U_T U_T^T)^(x)3 x
   void minv_Q(const T* x, T* y, bool staged = false) const {
-    // FP64, long lines: three passes with the dense M-check^-1 (not folded: the rounding of M-check's
-    // entries is not symmetric, and averaging the mirrored entries of its inverse would move it by
-    // 1e-14); below, the eigenvector route (its fused form takes as few launches).
+    // FP64: banded Cholesky line solves of long lines (chol_route); then three passes with the dense
+    // M-check^-1 (not folded: the rounding of M-check's entries is not symmetric, and averaging the
+    // mirrored entries of its inverse would move it by 1e-14); the eigenvector route for the
+    // shortest (its fused form takes as few launches).
     if constexpr (std::is_same<T, double>::value) {
+      if (chol_lb) {
+        const T* src = x;
+        for (int k = 1; k <= 3; ++k) {
+          ck(chol_solve_axis<T>(src, y, b, chol_p, k, chol_lb, chol_inv, k == 3 ? 2 * nu : T(1), s,
+                                nb, bs), "line solve");
+          src = y;
+        }
+        return;
+      }
       if (fx_Minv.fw.frag) {
         const T* src = x;
         T* dst[3] = {f1, f2, y};
@@ -2529,12 +2542,24 @@ int stokes_setup(stokes_t* out, int n_elems, int degree_p, double nu, const stok
       c->od.invd = upload<double>(c->arena, inv, c->stream);
     }
     {
-      Dense Minv, low;
-      if (!banded_inverse(u.Mc, degree_p, Minv, low))
+      // pressure block: the banded factor itself for long lines, the dense inverse below
+      std::vector<double> lb;
+      if (!banded_cholesky(u.Mc, degree_p, lb))
         throw SetupError{"pressure mass matrix is not positive definite"};
+      const int b = c->b, w = degree_p + 1;
       if (!reduced(c) && heT > kFixMinHalf) {
-        c->od.Minv = upload<double>(c->arena, Minv.v, c->stream);
-        c->od.fx_Minv = upload_fix_plain(c->arena, Minv, low, c->stream);
+        if (chol_route(b, degree_p)) {
+          std::vector<double> inv(b);
+          for (int i = 0; i < b; ++i) inv[i] = 1.0 / lb[(size_t)i * w + degree_p];
+          c->od.chol_lb = upload<double>(c->arena, lb, c->stream);
+          c->od.chol_inv = upload<double>(c->arena, inv, c->stream);
+          c->od.chol_p = degree_p;
+        } else {
+          Dense Minv, low;
+          banded_inverse(u.Mc, degree_p, lb, Minv, low);
+          c->od.Minv = upload<double>(c->arena, Minv.v, c->stream);
+          c->od.fx_Minv = upload_fix_plain(c->arena, Minv, low, c->stream);
+        }
       }
     }
     const Ops<double>* odq = nullptr;

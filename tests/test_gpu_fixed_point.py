@@ -77,6 +77,36 @@ def test_nonfinite_entry_reaches_its_whole_tensor_only(n, p, fused, bad):
     G.close()
 
 
+@pytest.mark.parametrize("n,p", [(63, 1), (62, 2), (64, 3), (61, 4)])
+def test_pressure_entries_keep_their_own_accuracy(n, p):
+    """The pressure block of long lines entry by entry, on vectors of wide range. To first order an
+    error of c 2^-53 |M| in M-check, in every direction, moves an entry by c 2^-53 of the sums below.
+    c = 40: 16 for the quadrature roundings in which two M-checks differ, 3 (p + 2) for a banded
+    Cholesky solve (M-check is totally positive, so |L| |L^T| = M)."""
+    S, _, _, _ = oracle(n, p)
+    G = _ctx(n, p, autotune=False)
+    x = _wide_vector(G, n)
+    x[:G.n_vel] = 0.0
+    M = S.uv.Mc.astype(np.longdouble)
+    inv = np.linalg.inv(S.uv.Mc).astype(np.longdouble)
+    for _ in range(3):   # Newton steps in extended precision
+        inv = inv + inv @ (np.eye(G.b, dtype=np.longdouble) - M @ inv)
+    q = x[G.n_vel:].reshape(G.b, G.b, G.b)
+
+    def passes(D, t):   # D[d] along direction d, in extended precision
+        for axis, d in zip((2, 1, 0), D):
+            t = np.moveaxis(np.tensordot(t, d, axes=([axis], [1])), -1, axis)
+        return t
+
+    ref = 2.0 * passes([inv] * 3, q.astype(np.longdouble))
+    a = np.abs(inv).astype(float)
+    wide = a @ np.abs(S.uv.Mc) @ a
+    size = sum(2.0 * passes([wide if k == d else a for k in range(3)], np.abs(q)) for d in range(3))
+    got = host(G.apply_P(dev(x)))[G.n_vel:].reshape(ref.shape)
+    G.close()
+    assert (np.abs(got - ref) / size).max() < 40 * 2.0 ** -53
+
+
 # extents from the smallest that takes the fixed-point passes, ragged and whole segments of 8 rows,
 # half widths 2 to 6, and 7, which does not (p = 6)
 @pytest.mark.parametrize("n,p,nu", [(38, 1, 1.0), (39, 1, 0.3), (38, 2, 2.0), (46, 2, 1.0),
