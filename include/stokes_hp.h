@@ -91,7 +91,7 @@ typedef struct stokes_opts {
                          preconditioner runs in reduced precision (z is then its FP32 output):
                          STOKES_OUTER_FP64 (default) or STOKES_OUTER_PAIR (every value carried as
                          an unevaluated sum of two FP32 numbers, about 48 significant bits, w
-                         rounded to FP64; about as fast as the FP64 form).
+                         rounded to FP64; on larger meshes about a tenth faster).
                          Residuals of the iterate (restarts, the final true residual),
                          stokes_apply_K and every FP64-preconditioned solve use the FP64
                          operator either way. Used with the Kronecker forward operator when

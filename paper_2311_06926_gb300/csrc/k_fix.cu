@@ -214,8 +214,9 @@ __device__ __forceinline__ void fix_chains(const FixOp& op, const unsigned* key,
   }
 }
 
-// Digit slices of terms 2 kp and 2 kp + 1 of one line into both halves of the operand. v: the entries of the two terms, then their partners (zero where there is none). A line that
-// cannot be scaled leaves zeros.
+// Digit slices of terms 2 kp and 2 kp + 1 of one line into both halves of the operand. v: the entries
+// of the two terms, then their partners (zero where there is none). A line that cannot be scaled
+// leaves zeros.
 __device__ __forceinline__ void fix_slices(const FixOp& op, uint4* xf, int mts, int line, int kp,
                                            unsigned key, const double (&v)[4]) {
   const int h = op.K - op.he, ks = op.t.ks;
@@ -356,10 +357,8 @@ struct FixJob {
   FixOp op;
   int64_t L, R;            // extents before and after the contracted direction
   const double* invd;      // optional multiplier per output entry
-  const double *lam1, *lam2, *lam3;
-  double scale, post;
+  double post;
   int has_post;            // post != 1 (an integer: an FP64 compare costs as much as an FMA)
-  Dims out;
 };
 struct FixBatch {
   FixJob job[kMaxModeJobs];
@@ -402,15 +401,8 @@ __global__ void __launch_bounds__(320, 2) k_fix_mode(const __grid_constant__ Fix
   __syncthreads();
   const auto emit = [&](IT first, int i, double v) {
     const IT o = first + JL * i;
-    if (J.invd) {
-      v *= J.invd[o];
-    } else if (J.lam1) {
-      const IT t2 = o / J.out.n1, t3 = t2 / J.out.n2;
-      v /= J.scale * (J.lam1[(int)(o - t2 * J.out.n1)] + J.lam2[(int)(t2 - t3 * J.out.n2)] +
-                      J.lam3[(int)t3]);
-    } else if (J.has_post) {
-      v *= J.post;
-    }
+    if (J.invd) v *= J.invd[o];
+    else if (J.has_post) v *= J.post;
     J.Y[o] = v;
   };
   for (int t = warp; t < op.t.nt; t += nw) fix_tile(op, xf, 1, 0, t, key, nl, row, emit);
@@ -516,9 +508,8 @@ struct FixLineJob {
   FixOp fwd, bwd;
   int64_t L;
   int n1;
-  const double* invd;
-  const double *lam1, *lam2, *lam3;
-  double scale, post;
+  const double* invd;   // multiplier per entry between the products
+  double post;
   int has_post;
 };
 struct FixLineBatch {
@@ -553,12 +544,7 @@ __global__ void __launch_bounds__(512) k_fix_line3(const __grid_constant__ FixLi
   fix_load<1>(A, xf, 1, nl, false, key[0], &any[0], J.L, ptr_a);
   __syncthreads();
   const auto emit_a = [&](int l, int i, double v) {
-    if (J.invd) {
-      v *= J.invd[line0 + l + J.L * i];
-    } else if (J.lam1) {
-      const int64_t g = line0 + l;
-      v /= J.scale * (J.lam1[(int)(g % J.n1)] + J.lam2[(int)(g / J.n1)] + J.lam3[i]);
-    }
+    v *= J.invd[line0 + l + J.L * i];
     raw[i * P + l] = v;
   };
   for (int t = warp; t < A.t.nt; t += nw) fix_tile(A, xf, 1, 0, t, key[0], nl, row, emit_a);
@@ -596,7 +582,7 @@ cudaError_t fix_mode_multi(const ModeArgs<double>* jobs, int njobs, cudaStream_t
   for (int j = 0; j < njobs; ++j) {
     const ModeArgs<double>& m = jobs[j];
     if (!m.fx.fw.frag || m.eo_he < 1 || m.m != m.in.get(m.axis) || m.ld != m.m ||
-        m.plain != jobs[0].plain)
+        m.plain != jobs[0].plain || (m.lam1 && !m.invd))
       return cudaErrorInvalidValue;
     nt = std::max(nt, m.fx.fw.nt);
     ks = std::max(ks, m.fx.fw.ks);
@@ -617,13 +603,8 @@ cudaError_t fix_mode_multi(const ModeArgs<double>* jobs, int njobs, cudaStream_t
     J.L = m.axis == 1 ? 1 : (m.axis == 2 ? in.n1 : (int64_t)in.n1 * in.n2);
     J.R = m.axis == 1 ? (int64_t)in.n2 * in.n3 : (m.axis == 2 ? in.n3 : 1);
     J.invd = m.invd;
-    J.lam1 = m.invd ? nullptr : m.lam1;
-    J.lam2 = m.lam2;
-    J.lam3 = m.lam3;
-    J.scale = m.scale;
-    J.post = m.lam1 ? 1.0 : m.post;
+    J.post = m.post;
     J.has_post = J.post != 1.0;
-    J.out = in;
     fb.first[j] = blocks;
     blocks += (int)((J.L * J.R + lb - 1) / lb);
     flops += (double)(J.L * J.R) * (m.plain ? 2.0 * m.m * m.m : eo_flops(m.m, m.eo_he));
@@ -699,7 +680,7 @@ bool fix_line3_multi(const FdLineArgs* jobs, int njobs, int block, cudaStream_t 
   fb.njobs = njobs;
   int ks = 1, K = 1;
   for (int j = 0; j < njobs; ++j) {
-    if (jobs[j].eo3 < 1 || !jobs[j].fx3.fw.frag) return false;
+    if (jobs[j].eo3 < 1 || !jobs[j].fx3.fw.frag || !jobs[j].invd) return false;
     ks = std::max(ks, jobs[j].fx3.fw.ks);
     K = std::max(K, jobs[j].in.n3);
   }
@@ -717,10 +698,6 @@ bool fix_line3_multi(const FdLineArgs* jobs, int njobs, int block, cudaStream_t 
     J.L = (int64_t)a.in.n1 * a.in.n2;
     J.n1 = a.in.n1;
     J.invd = a.invd;
-    J.lam1 = a.invd ? nullptr : a.lam1;
-    J.lam2 = a.lam2;
-    J.lam3 = a.lam3;
-    J.scale = a.scale;
     J.post = a.post;
     J.has_post = a.post != 1.0;
     fb.first[j] = blocks;

@@ -3,11 +3,12 @@
 //
 // On this part the FP64 pipe runs at about 1/64 of the FP32 rate, and FP64 banded passes of K as
 // FMA chains are bound by it (1052 us at 128^3 p = 3; the passes in fixed point that larger meshes
-// take in FP64, k_fix_band.cu, need 530 and this form 551). Here a value is the unevaluated sum hi + lo of two floats (Dekker, "A
-// floating-point technique for extending the available precision", 1971): a product is formed
-// exactly as p + e with p = a b rounded and e = fma(a, b, -p), a sum exactly as s + t by Knuth's
-// TwoSum, and the rounding errors are carried in the low word. Each multiply-add of a band row
-// costs about a dozen FP32 operations instead of one FP64 fused multiply-add, with about 48 significant bits instead of 53.
+// take in FP64, k_fix_band.cu, need 611 and this form 551). Here a value is the unevaluated sum
+// hi + lo of two floats (Dekker, "A floating-point technique for extending the available precision",
+// 1971): a product is formed exactly as p + e with p = a b rounded and e = fma(a, b, -p), a sum
+// exactly as s + t by Knuth's TwoSum, and the rounding errors are carried in the low word. Each
+// multiply-add of a band row costs about a dozen FP32 operations instead of one FP64 fused
+// multiply-add, with about 48 significant bits instead of 53.
 //
 // The input z of the Arnoldi product is the FP32 output of the preconditioner, so it enters as
 // pairs with lo = 0; the result is rounded to FP64. The sequence of passes is that of the FP64

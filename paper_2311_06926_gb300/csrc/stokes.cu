@@ -73,8 +73,6 @@ struct Arena {
   }
 };
 
-// The same banded matrix stored with a larger band width (zeros in the added slots); rows = 0 when
-// the matrix has fewer columns than the width.
 // s B (entrywise, FP64)
 Band scaled(const Band& B, double sc) {
   Band S = B;
@@ -82,6 +80,8 @@ Band scaled(const Band& B, double sc) {
   return S;
 }
 
+// The same banded matrix stored with a larger band width (zeros in the added slots); rows = 0 when
+// the matrix has fewer columns than the width.
 Band widen(const Band& B, int width) {
   Band W;
   if (width <= B.width || B.cols < width) return W;
@@ -573,7 +573,6 @@ struct Ops {
     adiag_all(x, y, m2);
   }
 
-  // y = A x; with h, the Horner step of h is applied to A x instead (y is scratch then)
   // the next fast diagonalisation after a Horner step whose result is one reads a staging copy
   bool stages() const { return std::is_same<T, float>::value && tc; }
 
@@ -592,6 +591,7 @@ struct Ops {
     }
   }
 
+  // y = A x; with h, the Horner step of h is applied to A x instead (y is scratch then)
   void apply_A(const T* x, T* y, const Horner<T>* h = nullptr) const {
     if (h && h->stage) {
       apply_A(x, y);
@@ -816,7 +816,6 @@ struct Ops {
             int eo = 0) const {
     ModeArgs<T> m = mjob(X, Y, U, n, trans, in, axis, nullptr, nullptr, nullptr, 1, post);
     m.eo_he = eo;
-    m.fx = fx_T;   // (the pressure block's products, all with U_T)
     ck(mode_product<T>(m, s), "mode product");
   }
 
@@ -858,10 +857,10 @@ struct Ops {
     const Dims d{b, b, b};
     if constexpr (std::is_same<T, double>::value) {
       if (fused_fd_ok()) {
-        FdPlaneArgs pa{x, f1, U_T, U_T, d, eo_T, eo_T, 1.0, fx_T, fx_T};
-        FdLineArgs la{f1, f2, U_T, d, eo_T, nullptr, nullptr, nullptr, nullptr, 1.0, 1.0, fx_T};
+        FdPlaneArgs pa{x, f1, U_T, U_T, d, eo_T, eo_T, 1.0, {}, {}};
+        FdLineArgs la{f1, f2, U_T, d, eo_T, nullptr, nullptr, nullptr, nullptr, 1.0, 1.0, {}};
         if (fd_plane_multi(&pa, 1, 1, mode_block, fd_fused, s) && fd_line3_multi(&la, 1, mode_block, s)) {
-          pa = FdPlaneArgs{f2, y, U_T, U_T, d, eo_T, eo_T, 2 * nu, fx_T, fx_T};
+          pa = FdPlaneArgs{f2, y, U_T, U_T, d, eo_T, eo_T, 2 * nu, {}, {}};
           if (fd_plane_multi(&pa, 1, 0, mode_block, fd_fused, s)) return;
         }
         throw CudaError{cudaErrorInvalidValue, "fused fast diagonalisation rejected its jobs"};

@@ -22,8 +22,8 @@ def _ctx(n, p, **kw):
 
 
 # halves of 12 (FMA chains), 13, 16, 17, 32, 33, 41 terms (tiles of 8 outputs, steps of 16 terms, the
-# level sums moved every 2 and 5 steps); b = 63, 64, 65, 82: the eigenvector route and the dense
-# inverse
+# level sums moved every 2 and 5 steps); b = 63 and below, 64, 65, 82: the dense inverse and the line
+# solves
 @pytest.mark.parametrize("n,p", [(23, 1), (24, 1), (31, 1), (31, 2), (61, 2), (63, 1), (62, 3),
                                  (78, 4)])
 def test_base_preconditioner_tile_edges(n, p):
