@@ -1361,7 +1361,7 @@ void init_ops(stokes_ctx* c, Ops<T>& o, const Band& M, const Band& K, const Band
     o.Mc_nu = upload_band<T>(ar, Mc_nu, s);
     o.Tc_2nu = upload_band<T>(ar, Tc_2nu, s);
     const int H = std::max({1, o.M.half, o.K.half, o.Mc.half, o.Tc.half});
-    if (c->b >= kFixBandMin && fix_band_fits(c->b, H)) {
+    if (c->b >= (c->p == 1 ? kFixBandMinLinear : kFixBandMin) && fix_band_fits(c->b, H)) {
       upload_fix_band(ar, M, o.M, H, s);
       upload_fix_band(ar, K, o.K, H, s);
       upload_fix_band(ar, Mc, o.Mc, H, s);

@@ -183,8 +183,8 @@ def _wide_vector(G, seed):
     return np.concatenate(out)
 
 
-@pytest.mark.parametrize("n,p,nu", [(45, 1, 1.0), (44, 2, 0.3), (43, 3, 2.0), (42, 4, 1.0),
-                                    (41, 5, 1.0)])
+@pytest.mark.parametrize("n,p,nu", [(60, 1, 1.0), (52, 2, 0.3), (51, 3, 2.0), (49, 4, 1.0),
+                                    (47, 5, 1.0)])
 def test_operator_entries_keep_their_own_accuracy(n, p, nu):
     """K x entry by entry against the FMA chains, which the same vector times 2^900 takes: each path
     rounds an entry at most once per term of its passes (six sums of at most 2 p + 3 terms, and the
@@ -223,4 +223,25 @@ def test_operator_entries_keep_their_own_accuracy(n, p, nu):
         y = host(G.apply_K(dev(x)))
         z = np.ldexp(host(G.apply_K(dev(np.ldexp(x, 900)))), -900)
         assert (np.abs(y - z) / size).max() < bound
+    G.close()
+
+
+# the smallest extents of the fixed-point passes (b = 60, else 52) and the largest below, ragged and
+# whole segments, half widths 2 to 6, and 7, which does not take them
+@pytest.mark.parametrize("n,p,nu", [(58, 1, 1.0), (59, 1, 0.3), (49, 2, 1.0), (50, 2, 2.0),
+                                    (49, 3, 0.7), (51, 4, 1.0), (47, 5, 3.0), (46, 6, 1.0)])
+def test_operator_at_the_line_of_the_fixed_point_passes(n, p, nu):
+    """Bound: that of test_operator_segment_edges; windows that cannot be scaled agree to it."""
+    S, _, Kop, F = oracle(n, p, nu)
+    x = synthetic.random_vector(S.size, 90 + n + p)
+    G = Stokes(n, p, nu=nu, max_order=2, max_steps=0, autotune=False)
+    ref = Kop(x)
+    for block in (128, 256, 512):
+        G.set_tuning(512, block, 0)
+        y = host(G.apply_K(dev(x)))
+        assert relerr(y, ref) < 1e-13
+        for e in (-900, 800):
+            assert relerr(np.ldexp(host(G.apply_K(dev(x) * 2.0 ** e)), -e), y) < 1e-13
+    assert not host(G.apply_K(torch.zeros(G.size, dtype=torch.float64, device="cuda"))).any()
+    assert relerr(host(G.apply_A(dev(x[:S.n_vel]))), F.apply_A(x[:S.n_vel])) < 1e-13
     G.close()
