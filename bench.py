@@ -27,6 +27,7 @@ launch). ``cpu_baseline``: the FP64 oracle on the host cores on a bounded sample
 import argparse
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -38,7 +39,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "Stokes solves/s to 1e-8 rel. residual; HBM GB/s & TC util vs peak; mixed vs FP64"
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
-# GB300 FP64 rate: nominal 1.25 TFLOP/s (an FMA-throughput probe on this machine measured 1.20).
+# GB300 FP64 rate: nominal 1.25 TFLOP/s (an FMA-throughput probe measured 1.20).
 FP64_PEAK_TFLOPS = 1.25
 TF32_NOMINAL_TFLOPS = 1100.0
 
@@ -68,17 +69,23 @@ KERNEL_NAMES = {
 }
 
 
+def library_constant(name):
+    """An integer constant of the library's internal header (a rule of its dispatch)."""
+    src = os.path.join(ROOT, "paper_2311_06926_gb300", "csrc", "internal.h")
+    with open(src) as fh:
+        return int(re.search(rf"\b{name} = (\d+)", fh.read()).group(1))
+
+
 def fixed_point_classes(n, p):
     """FP64 kernel classes that a mesh runs in fixed point (integer multipliers, FP16 tensor
     cores): their rate is not bounded by the FP64 pipe and is reported against HBM. The library's
-    rules: banded passes from 40 pressure entries per direction and p <= 5 (from 48 points for
-    the quadrature tables), mode products from half lengths above 12."""
+    rules (banded passes of half width p + 1 up to 6; mode products by their half length)."""
     b = n + p
     out = set()
-    if b >= 40 and p <= 5:
+    if b >= library_constant("kFixBandMinLinear" if p == 1 else "kFixBandMin") and p <= 5:
         out.add("band_pass_fp64")
-    if (b + 1) // 2 > 12:
-        out.update(("mode_product", "line_solve"))
+    if (b + 1) // 2 > library_constant("kFixMinHalf"):
+        out.add("mode_product")
     return out
 
 
@@ -529,7 +536,8 @@ def schur_variants(Stokes, n=32, p=3):
 def class_rooflines(prof, step_ms, prec, peaks, fixed=()):
     """Per kernel class of one profiled step: launches, time, share, and the achieved rate of its
     algorithmic work against the bound of that class (FP64 pipe for FP64 band passes and mode
-    products formed in FP64, HBM for the rest and for the classes in `fixed`). Times include the per-launch events of the profiled pass."""
+    products formed in FP64, HBM for the rest and for the classes in `fixed`). Times include the
+    per-launch events of the profiled pass."""
     hbm = peaks.get("hbm_gbs", 6800.0)
     out = {}
     for k, v in prof.items():
@@ -1199,8 +1207,9 @@ def run_sweep(args, wl):
     if dom_name == "mode_product" and prec == "fp64":
         # Live throughput of the class: the base preconditioner P_0 consists of dense products
         # only (velocity fast diagonalisation and pressure mass inverse, run as two concurrent
-        # branches; classes mode_product and line_solve), so back-to-back P_0 applications between two events on the library stream time exactly
-        # these kernels as they run inside the solves (no per-launch events in between).
+        # branches; classes mode_product and line_solve), so back-to-back P_0 applications between
+        # two events on the library stream time exactly these kernels as they run inside the solves
+        # (no per-launch events in between).
         xP = torch.randn(G.size, dtype=torch.float64, device="cuda")
         yP = torch.empty_like(xP)
         G.profile_begin()
