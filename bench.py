@@ -77,9 +77,10 @@ def library_constant(name):
 
 
 def fixed_point_classes(n, p):
-    """FP64 kernel classes that a mesh runs in fixed point (integer multipliers, FP16 tensor
-    cores): their rate is not bounded by the FP64 pipe and is reported against HBM. The library's
-    rules (banded passes of half width p + 1 up to 6; mode products by their half length)."""
+    """FP64 kernel classes that a mesh (one item) runs in fixed point (integer multipliers, FP16
+    tensor cores): their rate is not bounded by the FP64 pipe and is reported against HBM. The
+    library's rules (banded passes of half width p + 1 up to 6; mode products by their half
+    length)."""
     b = n + p
     out = set()
     if b >= library_constant("kFixBandMinLinear" if p == 1 else "kFixBandMin") and p <= 5:

@@ -226,10 +226,10 @@ def test_operator_entries_keep_their_own_accuracy(n, p, nu):
     G.close()
 
 
-# the smallest extents of the fixed-point passes (b = 60, else 52) and the largest below, ragged and
-# whole segments, half widths 2 to 6, and 7, which does not take them
-@pytest.mark.parametrize("n,p,nu", [(58, 1, 1.0), (59, 1, 0.3), (49, 2, 1.0), (50, 2, 2.0),
-                                    (49, 3, 0.7), (51, 4, 1.0), (47, 5, 3.0), (46, 6, 1.0)])
+# the smallest extents of the fixed-point passes (p = 1: b = 56, else 48) and the largest below, ragged
+# and whole segments, half widths 2 to 6, and 7, which does not take them
+@pytest.mark.parametrize("n,p,nu", [(54, 1, 1.0), (55, 1, 0.3), (45, 2, 1.0), (46, 2, 2.0),
+                                    (49, 3, 0.7), (44, 4, 1.0), (43, 5, 3.0), (46, 6, 1.0)])
 def test_operator_at_the_line_of_the_fixed_point_passes(n, p, nu):
     """Bound: that of test_operator_segment_edges; windows that cannot be scaled agree to it."""
     S, _, Kop, F = oracle(n, p, nu)
@@ -244,4 +244,19 @@ def test_operator_at_the_line_of_the_fixed_point_passes(n, p, nu):
             assert relerr(np.ldexp(host(G.apply_K(dev(x) * 2.0 ** e)), -e), y) < 1e-13
     assert not host(G.apply_K(torch.zeros(G.size, dtype=torch.float64, device="cuda"))).any()
     assert relerr(host(G.apply_A(dev(x[:S.n_vel]))), F.apply_A(x[:S.n_vel])) < 1e-13
+    G.close()
+
+
+# several items: the smallest extents of the fixed-point passes, and below
+@pytest.mark.parametrize("n,p,nrhs", [(39, 1, 2), (46, 2, 6), (45, 3, 3), (44, 4, 2)])
+def test_operator_of_several_items(n, p, nrhs):
+    """Bound: that of test_operator_segment_edges, item by item."""
+    S, _, Kop, _ = oracle(n, p)
+    G = Stokes(n, p, max_order=2, max_steps=1, precision="tf32", nrhs=nrhs, autotune=False)
+    X = [synthetic.random_vector(S.size, 200 + n + k) for k in range(nrhs)]
+    for block in (128, 256):
+        G.set_tuning(512, block, 0)
+        got = np.split(host(G.apply_K(dev(np.concatenate(X)))), nrhs)
+        for x, y in zip(X, got):
+            assert relerr(y, Kop(x)) < 1e-13
     G.close()
