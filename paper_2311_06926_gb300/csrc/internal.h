@@ -212,11 +212,10 @@ void fix_div_band_x1(const double* u1, const double* u2, const double* u3, int a
 // of a batch has the bits of a context of its own.
 constexpr int kFixBandMin = 48, kFixBandMinLinear = 56;   // (p >= 2, p = 1)
 // smallest number of points per direction of the fixed-point quadrature passes. K apply in us, chains
-// against fixed point: p = 1 39 points 141 / 141, 48 155 / 149, 63 202 / 178, 96 388 / 308; p = 2
-// 40 points 179 / 179, 48 198 / 193, 64 239 / 210; p = 3 40 points 222 / 217, 60 266 / 243, 95
-// 510 / 401; p = 4 36 points 260 / 261, 48 288 / 276, 96 557 / 429; below 40 the chains' launches
-// are the shorter ones (p = 1 24 points 123 / 128, p = 3 20 points 195 / 199).
-constexpr int kFixRectMin = 48;
+// against fixed point: p = 1 48 points 130 / 165, 72 212 / 214, 96 363 / 317; p = 2 48 168 / 199, 64
+// 219 / 223, 72 247 / 247, 96 402 / 343; p = 3 50 226 / 251, 70 301 / 296, 95 483 / 416; p = 4 48 260 /
+// 299, 72 351 / 346, 96 532 / 445; p = 5 56 341 / 360, 70 424 / 419, 98 678 / 566.
+constexpr int kFixRectMin = 72;
 
 // delta = sum_c D .c u_c: exact discrete divergence of the velocity coefficients (App. B.2),
 // output b^3. (D beta)_i = beta_i - beta_{i-1} with beta_{-1} = beta_a = 0.

@@ -260,3 +260,22 @@ def test_operator_of_several_items(n, p, nrhs):
         for x, y in zip(X, got):
             assert relerr(y, Kop(x)) < 1e-13
     G.close()
+
+
+# points per direction from 72 on (p + 2 per element), where the fixed-point evaluation passes begin,
+# and the largest below; the last segment of 8 rows ragged and whole
+@pytest.mark.parametrize("n,p,nu", [(23, 1, 1.0), (24, 1, 0.6), (25, 1, 1.0), (18, 2, 2.0),
+                                    (19, 2, 1.0), (15, 3, 1.0), (12, 4, 0.5), (13, 4, 1.0),
+                                    (11, 5, 1.0), (9, 6, 1.0), (10, 6, 1.0)])
+def test_quadrature_at_the_line_of_the_fixed_point_passes(n, p, nu):
+    """Bound: that of test_quadrature_operator_equals_kronecker_and_oracle."""
+    S, _, Kop, F = oracle(n, p, nu)
+    x = synthetic.random_vector(S.size, 80 + n + p)
+    ref = Kop(x)
+    G = Stokes(n, p, nu=nu, max_order=2, max_steps=0, autotune=False, forward="quadrature")
+    for block in (128, 256, 512):
+        G.set_tuning(512, block, 0)
+        assert relerr(host(G.apply_K(dev(x))), ref) < 1e-12
+    for e in (-900, 800):   # windows that cannot be scaled take chains
+        assert relerr(np.ldexp(host(G.apply_K(dev(x) * 2.0 ** e)), -e), ref) < 1e-12
+    G.close()
