@@ -4,8 +4,8 @@
 // form tiles of 16 lines by 8 outputs of both halves, the operator slices read from the
 // cache in operand order. Bound by instruction issue (scaling and slicing the lines, adding the
 // levels up and converting the sums take more slots than the multiplications). Measured against the
-// FMA-chain kernels they replace on lines of 25 entries or more: P_0^-1 4947 -> 915 us at 128^3
-// p = 3, 406 -> 134 at 64^3, 60 -> 46 at 32^3.
+// FMA-chain kernels they replace on lines of 25 entries or more: P_0^-1 4947 -> 860 us at 128^3
+// p = 3, 406 -> 200 at 64^3 (the pressure block of both by line solves), 60 -> 47 at 32^3.
 #include <algorithm>
 #include <atomic>
 

@@ -17,8 +17,8 @@
 // left to chains for lines of normal entries).
 //
 // Bound by instruction issue: about 140 instructions per result, of which the 27 multiply-adds of a
-// row of 9 take twice their slots. Measured against the FMA passes: K apply 1052 -> 616 us at 128^3
-// p = 3 (533 without weighing and chains), 61^3 p = 2 81, 48^3 p = 3 65 (70 and 50 without).
+// row of 9 take twice their slots. Measured against the FMA passes: K apply 1052 -> 613 us at 128^3
+// p = 3 (533 without weighing and chains), 61^3 p = 2 81, 48^3 p = 3 65 (66 and 50 without).
 //
 // A window with an infinity or a NaN, or outside [2^-823, 2^777], takes FMA chains instead.
 #include <algorithm>
