@@ -14,7 +14,8 @@ namespace shp {
 // (One scale for the 8 rows of a segment is not enough: the rows beside the penalty row of T-check
 // are 2^4 to 2^10 smaller, and held only that many bits fewer.) rows: {w, w, ex, 0} of row r of
 // segment seg at 4 (r segs + seg); the bytes of the words w are the magnitudes, in 256ths of the
-// scale (rounded down), of the entries that band_weigh weighs, at their places in the window. Empty: the band has no such table.
+// scale (rounded down), of the entries that band_weak weighs, at their places in the window.
+// Empty: the band has no such table.
 struct BandLimbs {
   std::vector<int> tab, rows, w0;
 };

@@ -201,15 +201,18 @@ void fix_div_band_x1(const double* u1, const double* u2, const double* u3, int a
                      const double* q, double nu, const BandD<double>& D, double* y0, double* y1,
                      int block, cudaStream_t s);
 // smallest pressure extent b of the fixed-point passes: below, a pass is a few waves of short chains
-// and the FMA kernels take less time. us, chains : fixed, of a K apply and of the FP64 order-2, 1-step
-// preconditioner: p = 1 b = 40 30 : 47, 160 : 183, b = 52 52 : 56, 215 : 230, b = 56 62 : 58, 249 : 259,
-// b = 60 73 : 65, 283 : 278; p = 2 b = 40 37 : 50, 167 : 179, b = 48 56 : 54, 213 : 213, b = 52 66 : 58,
-// 234 : 235; p = 3 b = 44 51 : 55, 197 : 212, b = 48 64 : 60, 220 : 227, b = 52 77 : 62, 246 : 246, b =
-// 72 182 : 113, 751 : 675; p = 4 b = 44 64 : 60, 208 : 232, b = 48 77 : 68, 234 : 246, b = 52 93 : 68,
-// 260 : 252; p = 5 b = 48 85 : 70, 242 : 258, b = 52 105 : 72, 274 : 272. The line suits the K apply:
-// reduced-precision contexts have no other FP64 passes, and their batches gain earlier (six items,
-// p = 3 b = 40 201 : 148, p = 1 132 : 117). It does not look at the number of items, because an item
-// of a batch has the bits of a context of its own.
+// and the FMA kernels take less time. us, chains : fixed, of a K apply and of the FP64 order-2,
+// 1-step preconditioner:
+//   p = 1  b = 40 30 : 47, 160 : 183; b = 52 52 : 56, 215 : 230; b = 56 62 : 58, 249 : 259; b = 60
+//          73 : 65, 283 : 278
+//   p = 2  b = 40 37 : 50, 167 : 179; b = 48 56 : 54, 213 : 213; b = 52 66 : 58, 234 : 235
+//   p = 3  b = 44 51 : 55, 197 : 212; b = 48 64 : 60, 220 : 227; b = 52 77 : 62, 246 : 246; b = 72
+//          182 : 113, 751 : 675
+//   p = 4  b = 44 64 : 60, 208 : 232; b = 48 77 : 68, 234 : 246; b = 52 93 : 68, 260 : 252
+//   p = 5  b = 48 85 : 70, 242 : 258; b = 52 105 : 72, 274 : 272
+// The line suits the K apply: reduced-precision contexts have no other FP64 passes, and their batches
+// gain earlier (six items, p = 3 b = 40 201 : 148, p = 1 132 : 117). It does not look at the number
+// of items, because an item of a batch has the bits of a context of its own.
 constexpr int kFixBandMin = 48, kFixBandMinLinear = 56;   // (p >= 2, p = 1)
 // smallest number of points per direction of the fixed-point quadrature passes. K apply in us, chains
 // against fixed point: p = 1 48 points 130 / 165, 72 212 / 214, 96 363 / 317; p = 2 48 168 / 199, 64
